@@ -231,3 +231,80 @@ def tolerance(case):
     if case["dtype"] == "fp16":
         return {"rel": 1.5e-3, "max": 1.5e-2}
     return {"rel": 4e-3 if peaked else 1.1e-2, "max": 0.08}
+
+
+def _codes64(x, scale=None):
+    """The paper's Eq. 2 per head: (e4m3 values of x / scale, times that scale, in 64 bits; the scale)."""
+    if scale is None:
+        amax = x.abs().amax(dim=(2, 3)).float()
+        scale = torch.where(amax == 0, torch.ones_like(amax), amax / torch.full_like(amax, 448.0))  # the IEEE division
+    s = scale[:, :, None, None]
+    codes = (x.float() / s).clamp(-448.0, 448.0).to(torch.float8_e4m3fn)
+    return codes.double() * s.double(), scale
+
+
+def _attention64(q, k, v):
+    out = torch.empty_like(q)
+    rows = max(1, (1 << 27) // k.shape[2])      # a block of scores of about 1 GB
+    for b in range(q.shape[0]):
+        for h in range(q.shape[1]):
+            for r in range(0, q.shape[2], rows):
+                p = torch.softmax(q[b, h, r:r + rows] @ k[b, h].T * q.shape[3] ** -0.5, dim=1)
+                out[b, h, r:r + rows] = p @ v[b, h]
+    return out
+
+
+def _shift_down(x, n):
+    """An int64 tensor shifted down by n as an unsigned word."""
+    return (x >> n) & ((1 << (64 - n)) - 1)
+
+
+def _mix64(x):
+    """The counter hash that ``perturb`` documents, on int64 tensors."""
+    def signed(c):
+        return c - (1 << 64) if c >= 1 << 63 else c
+    x = x + signed(0x9E3779B97F4A7C15)
+    x = (x ^ _shift_down(x, 30)) * signed(0xBF58476D1CE4E5B9)
+    x = (x ^ _shift_down(x, 27)) * signed(0x94D049BB133111EB)
+    return x ^ _shift_down(x, 31)
+
+
+def _perturbed64(x, epsilon, seed, stream):
+    B, H, rows, d = x.shape
+    x = x.reshape(B * H, rows * d // 2, 2).double()
+    rho = x.square().mean(dim=(1, 2)).sqrt()
+    dev = dict(dtype=torch.int64, device=x.device)
+    odd = 0x9E3779B97F4A7C15 - (1 << 64)
+    words = torch.arange(rows * d // 2, **dev) * odd
+    out = torch.empty_like(x)
+    for head in range(B * H):
+        key = _mix64(_mix64(torch.tensor(seed, **dev)) ^ (stream * (0xD6E8FEB86659FD93 - (1 << 64))))
+        bits = _mix64(words ^ _mix64(key ^ head))
+        u1, u2 = ((u.double() + 0.5) * 2.0 ** -32 for u in (_shift_down(bits, 32), bits & 0xffffffff))
+        r, angle = (-2.0 * u1.log()).sqrt(), 2.0 * math.pi * u2
+        out[head] = x[head] + epsilon * rho[head] * torch.stack((r * angle.cos(), r * angle.sin()), dim=1)
+    return out.reshape(B, H, rows, d), rho.reshape(B, H)
+
+
+def exact(case, seed):
+    """Where codes enter the attention, they are the definition's: what remains is what the kernels
+    lose in the scores, the weights, the sums and the results."""
+    kind = case["kind"]
+    if kind == "perturb":
+        return _perturbed64(_inputs(case, seed, ("k",))["k"], 0.0265, seed, 1)
+    if kind == "quant_one":
+        return [None, _inputs(case, seed, ("k",))["k"].abs().amax(dim=(2, 3)).double() / 448.0]
+    if kind != "quant_qkv":
+        rows = case["n_test"] + (0 if kind == "predict" else case["n_train"])
+        if case["B"] * case["H"] * case["n_train"] * rows > 5e11:
+            return None     # about 20 seconds of 64-bit matrix products
+    x = _inputs(case, seed, ("q_train", "k", "v", "q_test"))
+    if kind == "quant_qkv":
+        return {"s" + n[0]: x[n].abs().amax(dim=(2, 3)).double() / 448.0 for n in ("q_train", "k", "v")}
+    if kind in ("gated", "attn16"):
+        q, k, v, t = (x[n].double() for n in ("q_train", "k", "v", "q_test"))
+    else:
+        q, scale_q = _codes64(x["q_train"])
+        k, v, t = _codes64(x["k"])[0], _codes64(x["v"])[0], _codes64(x["q_test"], scale_q)[0]
+    out_test = _attention64(t, k, v)
+    return out_test if kind == "predict" else (_attention64(q, k, v), out_test)
