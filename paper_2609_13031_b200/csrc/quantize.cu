@@ -7,18 +7,12 @@
 // written for the conversion (5 B per element; 3 B when the scale is given).
 // The conversion walks each head backwards so that it starts on the part of the
 // head the maximum pass touched last, which is still in L2.
-// The IEEE division x/s is not evaluated per element: a 16-bit input is (1.m) * 2^e with a
-// 7-bit (bf16) or 10-bit (fp16) m, and RN((1.m) * 2^e / s) = RN((1.m) / s) * 2^e exactly
-// (scaling by a power of two is exact; where the product leaves the normal range the code
-// saturates or is zero either way).  Each block therefore divides once per mantissa into a
-// small table with the IEEE division, and an element costs a lookup and one multiplication
-// by +-2^e.  Codes are identical to those of the per-element division by construction.
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
+// The IEEE division x/s is not evaluated per element but by three multiply-adds that give the same
+// quotient (quantize_math.cuh).
 #include <mutex>
 
 #include "common.h"
+#include "quantize_math.cuh"
 
 namespace fp8attn {
 namespace {
@@ -33,32 +27,6 @@ int sm_count() {
         return 0;
     return sms;
 }
-
-__device__ __forceinline__ uint4 ld_nc_v4(const uint4* p) {
-    uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-    return v;
-}
-
-// The two 16-bit input types: packed |x| / max for the reduction, and the exact
-// fp32 value of the low and high half of a 32-bit word for the conversion.
-template <bool kHalf> struct In16;
-template <> struct In16<false> {
-    using V2 = __nv_bfloat162;
-    static constexpr int kMantBits = 7;
-    static __device__ __forceinline__ V2 as2(uint32_t u) { return *reinterpret_cast<V2*>(&u); }
-    // an fp32 with the bf16 bits in its upper half is that value
-    static __device__ __forceinline__ float lo(uint32_t w) { return __uint_as_float(w << 16); }
-    static __device__ __forceinline__ float hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
-};
-template <> struct In16<true> {
-    using V2 = __half2;
-    static constexpr int kMantBits = 10;
-    static __device__ __forceinline__ V2 as2(uint32_t u) { return *reinterpret_cast<V2*>(&u); }
-    static __device__ __forceinline__ float lo(uint32_t w) { return __low2float(as2(w)); }
-    static __device__ __forceinline__ float hi(uint32_t w) { return __high2float(as2(w)); }
-};
 
 // One block's share of max |x| over head blockIdx.y (vecs_per_head 16-byte vectors),
 // merged into amax_bits[blockIdx.y].
@@ -132,36 +100,6 @@ absmax_kernel(const uint4* __restrict__ x, int64_t vecs_per_head, uint32_t* __re
     absmax_body<kHalf>(x, vecs_per_head, amax_bits);
 }
 
-// two floats -> two e4m3 codes (lo in bits 0..7, hi in bits 8..15), RNE, saturating
-__device__ __forceinline__ uint32_t cvt_e4m3x2(float lo, float hi) {
-    uint16_t r;
-    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
-    return (uint32_t)r;
-}
-
-// x / s for a 16-bit x given as its exact fp32 value: the quotient of its mantissa from the
-// table, times its sign and power of two.  (Every fp32 that comes from a normal bf16, or from
-// any fp16, has at most kMantBits leading mantissa bits set.)  With kDirect the division is
-// evaluated per element: the block's scale is so small that subnormal inputs, which have no
-// normalised mantissa, can still give non-zero codes.
-template <bool kHalf, bool kDirect>
-__device__ __forceinline__ float quotient(float x, float s, const float* tab) {
-    if (kDirect) return __fdiv_rn(x, s);
-    const uint32_t u = __float_as_uint(x);
-    return tab[(u >> (23 - In16<kHalf>::kMantBits)) & ((1u << In16<kHalf>::kMantBits) - 1u)] *
-           __uint_as_float(u & 0xff800000u);
-}
-template <bool kHalf, bool kDirect>
-__device__ __forceinline__ uint32_t quant4(uint32_t w0, uint32_t w1, float s, const float* tab) {
-    // w0, w1: four 16-bit values
-    using T = In16<kHalf>;
-    float a = quotient<kHalf, kDirect>(T::lo(w0), s, tab);
-    float b = quotient<kHalf, kDirect>(T::hi(w0), s, tab);
-    float c = quotient<kHalf, kDirect>(T::lo(w1), s, tab);
-    float e = quotient<kHalf, kDirect>(T::hi(w1), s, tab);
-    return cvt_e4m3x2(a, b) | (cvt_e4m3x2(c, e) << 16);
-}
-
 // One block's share of head blockIdx.y.  Each thread turns 32 B of 16-bit input into
 // 16 B of e4m3 per step.  pairs_per_head = elems_per_head / 16.
 // `row_dest` (NULL: none) sends the codes of row r of a head to row row_dest[r] of the output;
@@ -173,45 +111,19 @@ __device__ __forceinline__ void quantize_body(const uint4* __restrict__ x, int64
                                               uint4* __restrict__ out, float* __restrict__ scale_out,
                                               const int32_t* __restrict__ row_dest = nullptr,
                                               int pairs_per_row_shift = 0) {
-    float s;
-    if (scale_in != nullptr) {
-        s = scale_in[blockIdx.y];
-    } else {
-        float amax = __uint_as_float(amax_bits[blockIdx.y]);
-        s = amax == 0.0f ? 1.0f : __fdiv_rn(amax, 448.0f);
-    }
+    const float s = scale_in != nullptr ? scale_in[blockIdx.y] : head_scale(__uint_as_float(amax_bits[blockIdx.y]));
     if (blockIdx.x == 0 && threadIdx.x == 0 && scale_out != nullptr) scale_out[blockIdx.y] = s;
-    // (1.m) / s for every mantissa m of the input type, by the IEEE division
-    constexpr int kTab = 1 << In16<kHalf>::kMantBits;
-    __shared__ float tab[kTab];
-    for (int m = threadIdx.x; m < kTab; m += kThreads)
-        tab[m] = __fdiv_rn(__uint_as_float(0x3f800000u | ((uint32_t)m << (23 - In16<kHalf>::kMantBits))), s);
-    __syncthreads();
+    const Divisor dv = divisor(s);
     const uint4* xh = x + (int64_t)blockIdx.y * pairs_per_head * 2;
     uint4* oh = out + (int64_t)blockIdx.y * pairs_per_head;
     int64_t stride = (int64_t)gridDim.x * kThreads;
-    // A bf16 subnormal (below 2^-126) is no (1.m) * 2^e; it can only give a non-zero code
-    // (|x/s| >= 2^-10) if s < 2^-116.  And (1.m) / s must itself be a normal number for the
-    // table entry to be the exact quotient's mantissa: s < 2^126.  Heads outside a scale range
-    // kept well inside both limits (and given scales that are zero, negative or not finite)
-    // take the per-element division.
-    const bool direct = !(s >= 1e-30f && s <= 1e30f);
     // walk the head from its end towards its start
     for (int64_t r = (int64_t)blockIdx.x * kThreads + threadIdx.x; r < pairs_per_head; r += stride) {
         int64_t i = pairs_per_head - 1 - r;
         uint4 a = ld_nc_v4(xh + 2 * i), b = ld_nc_v4(xh + 2 * i + 1);
-        uint4 o;
-        if (direct) {
-            o.x = quant4<kHalf, true>(a.x, a.y, s, tab);
-            o.y = quant4<kHalf, true>(a.z, a.w, s, tab);
-            o.z = quant4<kHalf, true>(b.x, b.y, s, tab);
-            o.w = quant4<kHalf, true>(b.z, b.w, s, tab);
-        } else {
-            o.x = quant4<kHalf, false>(a.x, a.y, s, tab);
-            o.y = quant4<kHalf, false>(a.z, a.w, s, tab);
-            o.z = quant4<kHalf, false>(b.x, b.y, s, tab);
-            o.w = quant4<kHalf, false>(b.z, b.w, s, tab);
-        }
+        const uint2 o0 = dv.direct ? quant8_direct<kHalf>(a, dv) : quant8<kHalf, true>(a, dv);
+        const uint2 o1 = dv.direct ? quant8_direct<kHalf>(b, dv) : quant8<kHalf, true>(b, dv);
+        const uint4 o = make_uint4(o0.x, o0.y, o1.x, o1.y);
         int64_t dst = i;
         if (row_dest != nullptr) {
             const int64_t row = i >> pairs_per_row_shift;
@@ -277,8 +189,8 @@ __global__ void __launch_bounds__(kThreads) quantize_batch_kernel(const QuantBat
 // maximum is needed.  All blocks then arrive on a counter and wait for the others (the launch
 // has at most two blocks per SM, so on an otherwise idle GPU they are all resident; the wait
 // is bounded all the same and records FP8ATTN_ERR_TIMEOUT on expiry).  Pass 2 takes the
-// maximum of a head over the slots of the blocks that share it, builds the mantissa table
-// and converts.  The last block to finish resets the two counters.
+// maximum of a head over the slots of the blocks that share it and converts.  The last block to
+// finish resets the two counters.
 // ---------------------------------------------------------------------------
 constexpr int kOneThreads = 512;
 constexpr int64_t kOneLaunchMaxBytes = 48ll << 20;   // 16-bit input bytes of a call that takes this path
@@ -297,8 +209,6 @@ template <bool kHalf>
 __global__ void __launch_bounds__(kOneThreads) quantize_one_launch_kernel(const OneLaunchArgs a) {
     using T = In16<kHalf>;
     using V2 = typename T::V2;
-    constexpr int kTab = 1 << T::kMantBits;
-    __shared__ float tab[kTab];
     __shared__ uint32_t warp_max[kOneThreads / 32];
     __shared__ float seg_amax;
     __shared__ int give_up;
@@ -380,7 +290,7 @@ __global__ void __launch_bounds__(kOneThreads) quantize_one_launch_kernel(const 
     __syncthreads();
     if (give_up) return;
 
-    // ---- pass 2: scale of each segment's head, mantissa table, conversion ----
+    // ---- pass 2: scale of each segment's head, conversion ----
     for (int z = 0; z < a.tensors; ++z) {
         const int64_t pph = a.b.pairs_per_head[z];
         const int64_t t_lo = lo > t_base[z] ? lo : t_base[z], t_hi = hi < t_base[z + 1] ? hi : t_base[z + 1];
@@ -408,30 +318,17 @@ __global__ void __launch_bounds__(kOneThreads) quantize_one_launch_kernel(const 
                 }
                 seg_amax = amax;
             }
-            __syncthreads();   // also: the lookups of the last segment are done
-            const float amax = seg_amax;
-            const float s = amax == 0.0f ? 1.0f : __fdiv_rn(amax, 448.0f);
-            if (p0 == 0 && threadIdx.x == 0 && a.b.scale_out[z] != nullptr) a.b.scale_out[z][head] = s;
-            for (int mnt = threadIdx.x; mnt < kTab; mnt += kOneThreads)
-                tab[mnt] = __fdiv_rn(__uint_as_float(0x3f800000u | ((uint32_t)mnt << (23 - T::kMantBits))), s);
             __syncthreads();
-            const bool direct = !(s >= 1e-30f && s <= 1e30f);
+            const float s = head_scale(seg_amax);
+            if (p0 == 0 && threadIdx.x == 0 && a.b.scale_out[z] != nullptr) a.b.scale_out[z][head] = s;
+            __syncthreads();   // seg_amax has been read
+            const Divisor dv = divisor(s);
             const uint4* xh = a.b.x[z] + head * pph * 2;
             uint4* oh = a.b.out[z] + head * pph;
             auto convert = [&](const uint4& u, const uint4& v) {
-                uint4 o;
-                if (direct) {
-                    o.x = quant4<kHalf, true>(u.x, u.y, s, tab);
-                    o.y = quant4<kHalf, true>(u.z, u.w, s, tab);
-                    o.z = quant4<kHalf, true>(v.x, v.y, s, tab);
-                    o.w = quant4<kHalf, true>(v.z, v.w, s, tab);
-                } else {
-                    o.x = quant4<kHalf, false>(u.x, u.y, s, tab);
-                    o.y = quant4<kHalf, false>(u.z, u.w, s, tab);
-                    o.z = quant4<kHalf, false>(v.x, v.y, s, tab);
-                    o.w = quant4<kHalf, false>(v.z, v.w, s, tab);
-                }
-                return o;
+                const uint2 o0 = dv.direct ? quant8_direct<kHalf>(u, dv) : quant8<kHalf, true>(u, dv);
+                const uint2 o1 = dv.direct ? quant8_direct<kHalf>(v, dv) : quant8<kHalf, true>(v, dv);
+                return make_uint4(o0.x, o0.y, o1.x, o1.y);
             };
             int64_t i = p0 + threadIdx.x;
             for (; i + kOneThreads < p1; i += 2 * kOneThreads) {   // four loads in flight
