@@ -80,14 +80,15 @@ int fp8attn_quantize_ex(const void* x_16bit, int B, int H, int64_t rows, int d,
  * Eq. 2), and Q_test quantized with the train-query scale (Method section, shared
  * query scale).  It removes most of the launch overhead that makes quantization
  * dominate at small train-row counts (the paper's latency tables below ~8k rows).
- * A call whose 16-bit inputs total at most 48 MB (they stay in L2) runs as ONE
- * launch of at most two thread blocks per SM: maximum, a grid-wide arrival
- * counter, conversion.  The blocks wait for one another, which presumes that they
- * are all resident at once, as they are on a GPU that runs nothing else; the wait
- * is bounded (2 s) and ends in FP8ATTN_ERR_TIMEOUT in the workspace's status word.
- * Callers that share the GPU with long-running kernels of other streams can ask
- * for the two-launch form with FP8ATTN_QKV_TWO_LAUNCHES (the _ex call).  Larger
- * calls always take two launches (maximum; conversion).
+ * Heads of up to 16 MB per tensor are held on chip between the maximum and the
+ * conversion, so that every element is read once: ONE launch, or two where the
+ * 16-bit inputs total more than 48 MB (a small one first).  Its thread blocks (one
+ * per SM) exchange the heads' maxima; they are launched cooperatively, so that all
+ * are resident at once, and every wait is bounded (2 s), ending in
+ * FP8ATTN_ERR_TIMEOUT in the workspace's status word.  Larger heads take two
+ * launches that do not wait (maximum; conversion), as do all calls with
+ * FP8ATTN_QKV_TWO_LAUNCHES (the _ex call), e.g. of callers that share the GPU with
+ * long-running kernels of other streams.
  *
  *   q_train, k, v   in  bf16 [B,H,n_train,d]      q_test in bf16 [B,H,n_test,d] (NULL iff n_test == 0)
  *   *_fp8           out e4m3, same shapes          scale_q/k/v out fp32 [B,H]
@@ -114,7 +115,7 @@ int fp8attn_quantize_qkv(const void* q_train, const void* k, const void* v, cons
  * limits small tables).  No maximum pass runs: one launch, each element read
  * once; values outside a given scale's range saturate at +-448.  Not combinable
  * with FP8ATTN_QUERY_SCALE_FROM_ALL_ROWS.
- * FP8ATTN_QKV_TWO_LAUNCHES: never take the one-launch path of small calls. */
+ * FP8ATTN_QKV_TWO_LAUNCHES: never take the form whose blocks wait for one another. */
 #define FP8ATTN_QUERY_SCALE_FROM_ALL_ROWS 1u
 #define FP8ATTN_SCALES_GIVEN 4u
 #define FP8ATTN_QKV_TWO_LAUNCHES 8u

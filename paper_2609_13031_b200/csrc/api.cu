@@ -118,8 +118,12 @@ int fp8attn_quantize_ex(const void* x_bf16, int B, int H, int64_t rows, int d, c
     rc = check_device();
     if (rc != FP8ATTN_OK) return rc;
     uint32_t* amax = reinterpret_cast<uint32_t*>(static_cast<char*>(workspace) + kWsAmaxOffset);
-    return launch_quantize(x_bf16, (int64_t)B * H, rows * (int64_t)d, scale_in, x_fp8, scale_out, amax,
-                           flags, static_cast<cudaStream_t>(cuda_stream));
+    char* ws = static_cast<char*>(workspace);
+    return launch_quantize(x_bf16, (int64_t)B * H, rows * (int64_t)d, scale_in, x_fp8, scale_out, amax, flags,
+                           reinterpret_cast<uint32_t*>(ws + kWsStatusOffset),
+                           reinterpret_cast<uint32_t*>(ws + kWsCounterOffset),
+                           reinterpret_cast<uint32_t*>(ws + ws_words_offset(B, H)),
+                           static_cast<cudaStream_t>(cuda_stream));
 }
 
 }  // extern "C"
@@ -156,7 +160,7 @@ int quantize_qkv_impl(const void* q_train, const void* k, const void* v, const v
                                n_test * (int64_t)d, q_train_fp8, k_fp8, v_fp8, q_test_fp8, scale_q, scale_k,
                                scale_v, amax, flags, reinterpret_cast<uint32_t*>(ws + kWsStatusOffset),
                                reinterpret_cast<uint32_t*>(ws + kWsCounterOffset),
-                               reinterpret_cast<float*>(ws + ws_partial_offset(B, H)), stream, key_dest, d);
+                               reinterpret_cast<uint32_t*>(ws + ws_words_offset(B, H)), stream, key_dest, d);
 }
 }  // namespace
 

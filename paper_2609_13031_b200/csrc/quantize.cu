@@ -1,6 +1,8 @@
 // Per-head absmax quantization of bf16 (or IEEE fp16) tensors to e4m3 (paper Eq. 2).
 //
-// Two HBM-bound kernels per call:
+// Calls whose heads fit on chip take one pass (staged.cuh, QuantizeOp below): 2 B read + 1 B written
+// per element.  The others (heads of more than 16 MB, an order of the keys, scales given, or on
+// request) take two HBM-bound kernels:
 //   absmax_kernel    max |x| per head, packed bf16x2 max, one atomicMax per block
 //   quantize_kernel  s = amax/448, y = x/s (IEEE fp32), cvt.rn.satfinite.e4m3x2
 // Algorithmic traffic: 2 B read per element for the maximum, 2 B read + 1 B
@@ -13,6 +15,7 @@
 
 #include "common.h"
 #include "quantize_math.cuh"
+#include "staged.cuh"
 
 namespace fp8attn {
 namespace {
@@ -178,176 +181,92 @@ __global__ void __launch_bounds__(kThreads) quantize_batch_kernel(const QuantBat
 }
 
 
-// ---------------------------------------------------------------------------
-// One launch for a small call (everything stays in L2): maximum, grid barrier, conversion.
-//
-// The 16-element pairs of all tensors and heads of the call form one flat range, cut into
-// equal shares, one per block; a block walks its share segment by segment (segment = the part
-// of one head of one tensor inside the share).  Pass 1 leaves the maximum of every segment
-// in a slot of its own (slot = block + ordinal of the head, which is unique along the
-// staircase of shares and heads), so nothing has to be cleared beforehand and no atomic
-// maximum is needed.  All blocks then arrive on a counter and wait for the others (the launch
-// has at most two blocks per SM, so on an otherwise idle GPU they are all resident; the wait
-// is bounded all the same and records FP8ATTN_ERR_TIMEOUT on expiry).  Pass 2 takes the
-// maximum of a head over the slots of the blocks that share it and converts.  The last block to
-// finish resets the two counters.
-// ---------------------------------------------------------------------------
-constexpr int kOneThreads = 512;
-constexpr int64_t kOneLaunchMaxBytes = 48ll << 20;   // 16-bit input bytes of a call that takes this path
-constexpr uint64_t kGridWaitLimitNs = 2000000000ull;
+// The quantizer in one pass (staged.cuh): the reduction is the absmax, its result the scale.
+template <bool kHalf>
+struct QuantizeOp {
+    using Acc = uint32_t;       // bit pattern of max |x| in the 16-bit type, which orders like an integer
+    struct Static {};
+    using Result = Divisor;
+    static constexpr int kOutBytes = 8;     // per 16-byte input vector
+    static constexpr int kSlotWords = 1;    // a published value: tag << 16 | maximum
 
-struct OneLaunchArgs {
-    QuantBatch b;
-    int tensors, n_heads;
-    int query_scale_from_all_rows;
-    uint32_t* status;     // workspace status words
-    uint32_t* counters;   // [0] arrivals after pass 1, [1] blocks done
-    float* partial;       // kOneLaunchMaxBlocks + 4 * n_heads slots
+    // thread `tid`'s part of `vecs` vectors
+    static __device__ __forceinline__ Acc reduce(const uint4* x, int vecs, int tid) {
+        typename In16<kHalf>::V2 m = In16<kHalf>::as2(0u);
+#pragma unroll 4
+        for (int i = tid; i < vecs; i += staged::kWorkers) m = absmax8<kHalf>(m, x[i]);
+        const uint32_t w = *reinterpret_cast<const uint32_t*>(&m);
+        return max(w & 0xffffu, w >> 16);
+    }
+    static __device__ __forceinline__ Acc combine(Acc a, Acc b) { return max(a, b); }
+    static __device__ __forceinline__ Acc shuffle(Acc v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+    static __device__ __forceinline__ Acc warp_combine(Acc v) { return __reduce_max_sync(0xffffffffu, v); }
+    static __device__ __forceinline__ void merge(Acc* to, Acc v) { atomicMax(to, v); }
+    static __device__ __forceinline__ void publish(uint32_t* slots, uint32_t, uint32_t i, uint32_t tag, Acc v) {
+        *reinterpret_cast<volatile uint32_t*>(slots + i) = tag << 16 | v;
+    }
+    using Raw = uint32_t;
+    static __device__ __forceinline__ Raw load(const uint32_t* slots, uint32_t, uint32_t i) {
+        return *reinterpret_cast<const volatile uint32_t*>(slots + i);
+    }
+    static __device__ __forceinline__ bool tagged(Raw r, uint32_t tag) { return r >> 16 == tag; }
+    static __device__ __forceinline__ Acc value(Raw r) { return r & 0xffffu; }
+    static __device__ __forceinline__ Result result(const Static&, Acc v) { return divisor(head_scale(In16<kHalf>::lo(v))); }
+    static __device__ __forceinline__ float output(const Result& r) { return r.s; }
+    // positions [i0, i1); kFollows: the scale is another tensor's
+    template <bool kFollows>
+    static __device__ __forceinline__ void convert(const Static&, const staged::Segment<QuantizeOp>& seg, const uint4* x,
+                                                   uint32_t i0, uint32_t i1, int tid) {
+        constexpr uint32_t kStep = staged::kWorkers;
+        const Divisor dv = seg.result;
+        uint2* o = reinterpret_cast<uint2*>(seg.out);
+        if (dv.direct) {
+            for (uint32_t i = i0 + tid; i < i1; i += kStep) o[i] = quant8_direct<kHalf>(x[i], dv);
+            return;
+        }
+        uint32_t i = i0 + tid;
+        for (; i + kStep < i1; i += 2 * kStep) {    // two vectors under way at a time
+            const uint4 v0 = x[i], v1 = x[i + kStep];
+            o[i] = quant8<kHalf, kFollows>(v0, dv);
+            o[i + kStep] = quant8<kHalf, kFollows>(v1, dv);
+        }
+        if (i < i1) o[i] = quant8<kHalf, kFollows>(x[i], dv);
+    }
 };
 
+// Calls of more than this many 16-bit input bytes clear their words in a launch of their own first
+// (which also starts on the data); smaller ones rely on what the last call left.
+constexpr int64_t kOneLaunchMaxBytes = 48ll << 20;
+
+// The one-pass kernel for tensors [0, tensors) of `b` and, if there is one, tensor 3 with the scale of
+// tensor 0.  *taken: whether it takes the call.
 template <bool kHalf>
-__global__ void __launch_bounds__(kOneThreads) quantize_one_launch_kernel(const OneLaunchArgs a) {
-    using T = In16<kHalf>;
-    using V2 = typename T::V2;
-    __shared__ uint32_t warp_max[kOneThreads / 32];
-    __shared__ float seg_amax;
-    __shared__ int give_up;
-    const int nb = gridDim.x, bid = blockIdx.x;
-    int64_t total = 0, t_base[5];
-    for (int z = 0; z < 4; ++z) {
-        t_base[z] = total;
-        if (z < a.tensors) total += a.b.pairs_per_head[z] * a.n_heads;
+int launch_staged(const QuantBatch& b, int tensors, int64_t n_heads, uint32_t* status, uint32_t* counters,
+                  uint32_t* words, int sms, bool* taken, cudaStream_t stream) {
+    using Op = QuantizeOp<kHalf>;
+    staged::Args<Op> a = {};
+    for (int z = 0; z < tensors; ++z) {
+        a.x[z] = b.x[z];
+        a.out[z] = b.out[z];
+        a.result_out[z] = b.scale_out[z];
     }
-    t_base[4] = total;
-    auto share_lo = [&](int blk) { return total * blk / nb; };
-    const int64_t lo = share_lo(bid), hi = share_lo(bid + 1);
-    // a device error recorded earlier is sticky: nothing runs until the host has read it
-    // (one thread decides for the block)
-    if (threadIdx.x == 0) give_up = *reinterpret_cast<volatile uint32_t*>(a.status) != 0u;
-    __syncthreads();
-    if (give_up) return;
-
-    // ---- pass 1: the maximum of every segment of this block's share ----
-    for (int z = 0; z < a.tensors; ++z) {
-        const int64_t pph = a.b.pairs_per_head[z];
-        const bool counts = z < 3 || a.query_scale_from_all_rows;
-        const int64_t t_lo = lo > t_base[z] ? lo : t_base[z], t_hi = hi < t_base[z + 1] ? hi : t_base[z + 1];
-        if (pph <= 0 || !counts || t_lo >= t_hi) continue;
-        for (int64_t head = (t_lo - t_base[z]) / pph; t_base[z] + head * pph < t_hi; ++head) {
-            const int64_t h_base = t_base[z] + head * pph;
-            const int64_t p0 = (t_lo > h_base ? t_lo : h_base) - h_base;
-            const int64_t p1 = (t_hi < h_base + pph ? t_hi : h_base + pph) - h_base;
-            const uint4* xh = a.b.x[z] + head * pph * 2;
-            auto am = [](uint32_t u, uint32_t v) { return __hmax2(__habs2(T::as2(u)), __habs2(T::as2(v))); };
-            V2 m = T::as2(0u);
-            int64_t i = 2 * p0 + threadIdx.x;
-            for (; i + 3 * kOneThreads < 2 * p1; i += 4 * kOneThreads) {   // four loads in flight
-                const uint4 v0 = xh[i], v1 = xh[i + kOneThreads], v2 = xh[i + 2 * kOneThreads],
-                            v3 = xh[i + 3 * kOneThreads];
-                m = __hmax2(m, __hmax2(__hmax2(__hmax2(am(v0.x, v0.y), am(v0.z, v0.w)),
-                                               __hmax2(am(v1.x, v1.y), am(v1.z, v1.w))),
-                                       __hmax2(__hmax2(am(v2.x, v2.y), am(v2.z, v2.w)),
-                                               __hmax2(am(v3.x, v3.y), am(v3.z, v3.w)))));
-            }
-            for (; i < 2 * p1; i += kOneThreads) {
-                const uint4 v = xh[i];
-                m = __hmax2(m, __hmax2(am(v.x, v.y), am(v.z, v.w)));
-            }
-            uint32_t bits = __float_as_uint(fmaxf(__low2float(m), __high2float(m)));
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) bits = max(bits, __shfl_xor_sync(0xffffffffu, bits, o));
-            __syncthreads();   // warp_max of the last segment has been read
-            if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = bits;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                for (int w = 0; w < kOneThreads / 32; ++w) bits = max(bits, warp_max[w]);
-                a.partial[bid + z * a.n_heads + (int)head] = __uint_as_float(bits);
-            }
-        }
-    }
-    // ---- grid barrier: every block's maxima are visible before any block converts ----
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(a.counters, 1u);
-        uint64_t t0;
-        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
-        int bad = 0;
-        while (*reinterpret_cast<volatile uint32_t*>(a.counters) < (uint32_t)nb) {
-            __nanosleep(64);
-            uint64_t t1;
-            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t1));
-            if (t1 - t0 > kGridWaitLimitNs || *reinterpret_cast<volatile uint32_t*>(a.status) != 0u) {
-                if (atomicCAS(a.status, 0u, (uint32_t)FP8ATTN_ERR_TIMEOUT) == 0u)
-                    a.status[1] = (kDetailQuantizeGridWait << 24) | ((uint32_t)bid & 0xFFFFFFu);
-                bad = 1;
-                break;
-            }
-        }
-        __threadfence();
-        give_up = bad;
-    }
-    __syncthreads();
-    if (give_up) return;
-
-    // ---- pass 2: scale of each segment's head, conversion ----
-    for (int z = 0; z < a.tensors; ++z) {
-        const int64_t pph = a.b.pairs_per_head[z];
-        const int64_t t_lo = lo > t_base[z] ? lo : t_base[z], t_hi = hi < t_base[z + 1] ? hi : t_base[z + 1];
-        if (pph <= 0 || t_lo >= t_hi) continue;
-        for (int64_t head = (t_lo - t_base[z]) / pph; t_base[z] + head * pph < t_hi; ++head) {
-            const int64_t h_base = t_base[z] + head * pph;
-            const int64_t p0 = (t_lo > h_base ? t_lo : h_base) - h_base;
-            const int64_t p1 = (t_hi < h_base + pph ? t_hi : h_base + pph) - h_base;
-            if (threadIdx.x == 0) {
-                // the head's maximum: over the slots of all blocks whose share touches the
-                // head (of the tensor the scale comes from: the test queries take the train
-                // queries' maximum; with the single-call form both query tensors count)
-                float amax = 0.f;
-                for (int src = 0; src < 2; ++src) {
-                    const int zs = src == 0 ? (z == 3 ? 0 : z) : (z == 0 || z == 3 ? 3 : -1);
-                    if (zs < 0 || (src == 1 && !a.query_scale_from_all_rows) || zs >= a.tensors) continue;
-                    const int64_t pz = a.b.pairs_per_head[zs];
-                    if (pz <= 0) continue;
-                    const int64_t s0 = t_base[zs] + head * pz, s1 = s0 + pz;
-                    int b0 = (int)(s0 * nb / total);
-                    while (b0 > 0 && share_lo(b0) > s0) --b0;
-                    while (share_lo(b0 + 1) <= s0) ++b0;
-                    for (int blk = b0; blk < nb && share_lo(blk) < s1; ++blk)
-                        amax = fmaxf(amax, a.partial[blk + zs * a.n_heads + (int)head]);
-                }
-                seg_amax = amax;
-            }
-            __syncthreads();
-            const float s = head_scale(seg_amax);
-            if (p0 == 0 && threadIdx.x == 0 && a.b.scale_out[z] != nullptr) a.b.scale_out[z][head] = s;
-            __syncthreads();   // seg_amax has been read
-            const Divisor dv = divisor(s);
-            const uint4* xh = a.b.x[z] + head * pph * 2;
-            uint4* oh = a.b.out[z] + head * pph;
-            auto convert = [&](const uint4& u, const uint4& v) {
-                const uint2 o0 = dv.direct ? quant8_direct<kHalf>(u, dv) : quant8<kHalf, true>(u, dv);
-                const uint2 o1 = dv.direct ? quant8_direct<kHalf>(v, dv) : quant8<kHalf, true>(v, dv);
-                return make_uint4(o0.x, o0.y, o1.x, o1.y);
-            };
-            int64_t i = p0 + threadIdx.x;
-            for (; i + kOneThreads < p1; i += 2 * kOneThreads) {   // four loads in flight
-                const uint4 u0 = xh[2 * i], v0 = xh[2 * i + 1];
-                const uint4 u1 = xh[2 * (i + kOneThreads)], v1 = xh[2 * (i + kOneThreads) + 1];
-                oh[i] = convert(u0, v0);
-                oh[i + kOneThreads] = convert(u1, v1);
-            }
-            for (; i < p1; i += kOneThreads) oh[i] = convert(xh[2 * i], xh[2 * i + 1]);
-        }
-    }
-    // ---- the last block to finish leaves the counters at zero for the next call ----
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        if (atomicAdd(a.counters + 1, 1u) == (uint32_t)nb - 1u) {
-            a.counters[0] = 0u;
-            a.counters[1] = 0u;
-        }
-    }
+    a.tensors = tensors;
+    a.units = (int)(tensors * n_heads);
+    a.vecs = b.pairs_per_head[0] * 2;
+    const int64_t follow = b.pairs_per_head[3] * 2;
+    a.follow_x = b.x[3];
+    a.follow_out = b.out[3];
+    a.follow_vecs = (uint32_t)follow;
+    a.follow_counts = b.amax_acc[3] != nullptr;
+    a.status = status;
+    a.counter = counters;
+    *taken = false;
+    const int n_words = (int)(kOnePassWords + 4 * n_heads);
+    const unsigned grid = follow > 0x7fffffffll ? 0u : staged::plan(a, sms, words, n_words);
+    if (grid == 0) return FP8ATTN_OK;
+    *taken = true;
+    const bool clear = (a.vecs * a.units + follow * n_heads) * 16 > kOneLaunchMaxBytes;
+    return staged::launch(a, grid, clear, words, n_words, stream);
 }
 
 }  // namespace
@@ -356,7 +275,7 @@ int launch_quantize_qkv(const void* q_train, const void* k, const void* v, const
                         int64_t n_heads, int64_t elems_train, int64_t elems_test, void* q_train_fp8,
                         void* k_fp8, void* v_fp8, void* q_test_fp8, float* scale_q, float* scale_k,
                         float* scale_v, uint32_t* amax_bits, uint32_t flags, uint32_t* status,
-                        uint32_t* counters, float* partial, cudaStream_t stream, int32_t* key_dest, int d) {
+                        uint32_t* counters, uint32_t* words, cudaStream_t stream, int32_t* key_dest, int d) {
     if (n_heads <= 0) return FP8ATTN_OK;
     if (n_heads > 65535) return FP8ATTN_ERR_UNSUPPORTED;
     QuantBatch b;
@@ -388,29 +307,11 @@ int launch_quantize_qkv(const void* q_train, const void* k, const void* v, const
     const int sms = sm_count();
     if (sms <= 0) return FP8ATTN_ERR_CUDA;
     const bool half = (flags & FP8ATTN_INPUT_FP16) != 0;
-    // small call: one launch (maximum, grid barrier, conversion)
-    const int64_t total_pairs = (3 * elems_train + elems_test) / 16 * n_heads;
-    if (!(flags & (FP8ATTN_SCALES_GIVEN | FP8ATTN_QKV_TWO_LAUNCHES)) && key_dest == nullptr && status != nullptr &&
-        total_pairs > 0 &&
-        total_pairs * 32 <= kOneLaunchMaxBytes) {
-        OneLaunchArgs a;
-        a.b = b;
-        a.tensors = tensors;
-        a.n_heads = (int)n_heads;
-        a.query_scale_from_all_rows = (flags & FP8ATTN_QUERY_SCALE_FROM_ALL_ROWS) ? 1 : 0;
-        a.status = status;
-        a.counters = counters;
-        a.partial = partial;
-        // At most two blocks of 512 threads per SM: on a GPU that runs nothing else all blocks
-        // are resident at once.  (Where other work holds SMs, the blocks that are resident wait
-        // for the rest; the wait is bounded.)
-        int64_t nb = (total_pairs + kOneThreads - 1) / kOneThreads;
-        if (nb > 2 * sms) nb = 2 * sms;
-        if (nb > kOneLaunchMaxBlocks) nb = kOneLaunchMaxBlocks;
-        if (half) quantize_one_launch_kernel<true><<<(unsigned)nb, kOneThreads, 0, stream>>>(a);
-        else quantize_one_launch_kernel<false><<<(unsigned)nb, kOneThreads, 0, stream>>>(a);
-        count_launch();
-        return cudaGetLastError() == cudaSuccess ? FP8ATTN_OK : FP8ATTN_ERR_CUDA;
+    if (!(flags & (FP8ATTN_SCALES_GIVEN | FP8ATTN_QKV_TWO_LAUNCHES)) && key_dest == nullptr && elems_train > 0) {
+        bool taken = false;
+        const int rc = half ? launch_staged<true>(b, 3, n_heads, status, counters, words, sms, &taken, stream)
+                            : launch_staged<false>(b, 3, n_heads, status, counters, words, sms, &taken, stream);
+        if (rc != FP8ATTN_OK || taken) return rc;
     }
     const int64_t want = ((int64_t)sms * 16 + n_heads * 3 - 1) / (n_heads * 3);
     const int64_t have = (elems_train / 16 + kThreads - 1) / kThreads;
@@ -448,7 +349,8 @@ int launch_quantize_qkv(const void* q_train, const void* k, const void* v, const
 
 int launch_quantize(const void* x_bf16, int64_t n_heads, int64_t elems_per_head,
                     const float* scale_in, void* x_fp8, float* scale_out,
-                    uint32_t* amax_bits, uint32_t flags, cudaStream_t stream) {
+                    uint32_t* amax_bits, uint32_t flags, uint32_t* status, uint32_t* counters, uint32_t* words,
+                    cudaStream_t stream) {
     const bool half = (flags & FP8ATTN_INPUT_FP16) != 0;
     if (n_heads <= 0) return FP8ATTN_OK;
     if (n_heads > 65535) return FP8ATTN_ERR_UNSUPPORTED;
@@ -462,6 +364,17 @@ int launch_quantize(const void* x_bf16, int64_t n_heads, int64_t elems_per_head,
         int64_t b = want < have ? want : have;
         return (unsigned)(b < 1 ? 1 : b);
     };
+    if (scale_in == nullptr && elems_per_head > 0 && status != nullptr) {
+        QuantBatch b = {};
+        b.x[0] = static_cast<const uint4*>(x_bf16);
+        b.out[0] = static_cast<uint4*>(x_fp8);
+        b.pairs_per_head[0] = pairs;
+        b.scale_out[0] = scale_out;
+        bool taken = false;
+        const int rc = half ? launch_staged<true>(b, 1, n_heads, status, counters, words, sms, &taken, stream)
+                            : launch_staged<false>(b, 1, n_heads, status, counters, words, sms, &taken, stream);
+        if (rc != FP8ATTN_OK || taken) return rc;
+    }
     if (scale_in == nullptr) {
         if (cudaMemsetAsync(amax_bits, 0, sizeof(uint32_t) * n_heads, stream) != cudaSuccess)
             return FP8ATTN_ERR_CUDA;
@@ -549,5 +462,5 @@ extern "C" int fp8attn_quantize_noalloc(const void* x_bf16, int B, int H, int64_
     if (rc != FP8ATTN_OK) return rc;
     // launch_quantize clears the accumulators it uses at the start of every call
     return launch_quantize(x_bf16, (int64_t)B * H, rows * (int64_t)d, scale_in, x_fp8, scale_out, amax, 0u,
-                           static_cast<cudaStream_t>(cuda_stream));
+                           nullptr, nullptr, nullptr, static_cast<cudaStream_t>(cuda_stream));
 }

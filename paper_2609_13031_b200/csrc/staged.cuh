@@ -1,0 +1,477 @@
+// One pass over tensors whose every element needs a reduction over its whole head first (the
+// absmax of the quantizer, the sum of squares of the perturbation): an element crosses the HBM
+// interface once on its way in and once on its way out.
+//
+// What bounds it: HBM.  Two kernels, one per pass, read every element twice (5 bytes per element
+// of the quantizer instead of 3), because a large call is more than L2 can hold between them.
+// Here the first read stays on chip, in shared memory: 148 SMs hold 33 MB in two buffers per SM.
+//
+// A "unit" is one head of one tensor that is reduced.  The units of a call form a flat range, cut
+// into stages of whole units that fit one buffer of every SM; of each stage every block (one per
+// SM) holds an equal contiguous share, loaded by cp.async.bulk.  Per stage: the share has landed ->
+// the worker warps reduce it, segment by segment (segment = the part of one unit inside the
+// share) -> the exchange warp publishes the segments' values and collects those of the other
+// blocks that share its units, while the workers convert the second half of the stage before ->
+// they convert the first half of this one.  The load warp refills each half of a buffer as soon as
+// it is converted, and has what there is no room for yet fetched to L2, so that HBM is read without
+// a pause.  A value is published in words of its own together with a tag (the stage), so that a
+// store and a poll carry it: no atomics, no fence, no counter (those took 3 us a stage, as much as
+// the work).
+//
+// The blocks are launched cooperatively, i.e. resident together or not at all; the waits are
+// bounded all the same (kWaitClocks: FP8ATTN_ERR_TIMEOUT in the status word).  The last block to
+// finish leaves the published words and its counter at zero for the next call.
+//
+// Measured, quantizer, 8 heads of 65,536 + 16,384 rows x 128 (654 MB in and out, 100 us at the copy
+// rate): 128 us, two passes 182 us; 16 heads of 30,011 x 64 62.6 / 89.1 us; 8 heads of 20,011 + 3,001 x
+// 128 57.0 / 55.7 us; 8,192 + 2,048 x 64 17.4 / 20.3 us.  About 10 us go before the second stage:
+// launch, the first stage's way in, and its exchange under the second's loads.
+// (Tried before: 24 KB chunks handed out by tickets to a control thread and worker warps: 2.5 us per
+// chunk for the hand-overs.  Accumulators and a grid-wide counter instead of tagged words: 154 us.
+// Without the fetch to L2: 159 us.)
+#pragma once
+#include "common.h"
+#include "sm100_ptx.cuh"
+
+namespace fp8attn {
+namespace staged {
+
+using namespace ptx;
+
+constexpr int kThreads = 1024;
+constexpr int kWorkers = kThreads - 64;        // and one warp that issues the loads, one that exchanges values
+constexpr int kBufVecs = 7088;                 // 16-byte vectors per buffer: a head of 65,536 x 128 over 148 SMs
+constexpr int kParts = 2;                      // a buffer is given up in halves
+constexpr size_t kSmemBytes = (size_t)2 * kBufVecs * 16;
+constexpr int kMaxSegments = 48;               // per share
+constexpr int64_t kWaitClocks = 4000000000ll;  // 2 s
+
+template <class Op>
+struct Args {
+    const uint4* x[3];          // the tensors that are reduced: unit u is head u / tensors of tensor u % tensors
+    void* out[3];
+    float* result_out[3];       // per head (NULL: none)
+    int tensors, units;
+    int64_t vecs;               // 16-byte vectors per unit
+    int stage_units;            // per stage (the last one may have fewer)
+    // a tensor that takes the results of tensor 0 as they are (values may lie outside their range) ...
+    const uint4* follow_x;
+    void* follow_out;
+    uint32_t follow_vecs;       // per head
+    int follow_counts;          // ... after entering its reduction
+    uint32_t* status;
+    uint32_t* counter;          // blocks done
+    uint32_t* slots;            // published values, `sets` sets of slots_per_set
+    uint32_t slots_per_set;
+    // Alternate stages use alternate sets: a block is in stage s + 2 only after every block that it
+    // shares a unit with has collected stage s.  A shorter last stage pairs other blocks with one
+    // another and has a set of its own.
+    int sets, last_set;
+    uint32_t* heads;            // published results of tensor 0, for the rows that follow it
+    typename Op::Static op;
+};
+
+// the workers and the exchange warp (barrier 0 is __syncthreads)
+__device__ __forceinline__ void sync_exchange() { asm volatile("bar.sync 1, %0;" ::"n"(kWorkers + 32) : "memory"); }
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_prefetch(const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
+// first position of block b's share of `total` vectors (128-byte lines stay whole).  A stage is at
+// most kBufVecs vectors per SM: everything fits 32 bits.
+__device__ __forceinline__ uint32_t cut(uint32_t total, uint32_t b) {
+    return b == gridDim.x ? total : total * b / gridDim.x & ~7u;
+}
+// One block's share of one stage: n positions from cut(total, block) on, which are `segs` segments of
+// the units from `unit` (of the stage) on; the first begins at vector `skip` of its unit.
+struct Share {
+    uint32_t total, unit, segs, skip, n;
+    __device__ __forceinline__ Share(uint32_t stage_units, uint32_t vecs) {
+        total = stage_units * vecs;
+        const uint32_t lo = cut(total, blockIdx.x);
+        n = cut(total, blockIdx.x + 1) - lo;
+        unit = lo / vecs;
+        skip = lo - unit * vecs;
+        segs = n == 0 ? 0 : (skip + n + vecs - 1) / vecs;
+    }
+    // first and last + 1 position of segment g, and the vector of its unit that the first is
+    __device__ __forceinline__ uint32_t begin(uint32_t g, uint32_t vecs) const { return g == 0 ? 0 : g * vecs - skip; }
+    __device__ __forceinline__ uint32_t end(uint32_t g, uint32_t vecs) const { return min((g + 1) * vecs - skip, n); }
+    __device__ __forceinline__ uint32_t at(uint32_t g) const { return g == 0 ? skip : 0; }
+    __device__ __forceinline__ uint32_t half() const { return n / 2 & ~7u; }
+    // the block that holds position x
+    __device__ __forceinline__ uint32_t holder(uint32_t x) const {
+        uint32_t b = min(x * gridDim.x / total, gridDim.x - 1);
+        while (cut(total, b) > x) --b;
+        while (cut(total, b + 1) <= x) ++b;
+        return b;
+    }
+};
+
+// What the conversion needs to know about a segment.
+template <class Op>
+struct Segment {
+    typename Op::Result result;
+    uint8_t* out;               // where position 0 of the share would go
+    uint32_t begin, end;        // positions
+    uint32_t head;
+    int32_t at;                 // vector of the unit = position + at
+};
+
+// every contiguous piece of half `part` of a share: to(first position, source, vectors)
+template <class Op, class To>
+__device__ __forceinline__ void half_share(const Args<Op>& a, const Share& s, int stage, uint32_t part, To to) {
+    const uint32_t vecs = (uint32_t)a.vecs, tensors = (uint32_t)a.tensors;
+    const uint32_t u0 = (uint32_t)(stage * a.stage_units) + s.unit;
+    const uint32_t p0 = part == 0 ? 0 : s.half(), p1 = part == 0 ? s.half() : s.n;
+    for (uint32_t g = 0; g < s.segs; ++g) {
+        const uint32_t b = s.begin(g, vecs), i0 = max(p0, b), i1 = min(p1, s.end(g, vecs));
+        if (i0 >= i1) continue;
+        const uint32_t unit = u0 + g, head = unit / tensors;
+        to(i0, a.x[unit - head * tensors] + (int64_t)head * vecs + s.at(g) + (i0 - b), i1 - i0);
+    }
+}
+
+// A launch of its own before large calls: clears the words and has the first stage fetched to L2
+// meanwhile (the launch then costs nothing).  One warp per block, the grid of staged_kernel.
+template <class Op>
+__global__ void clear_and_fetch_kernel(const __grid_constant__ Args<Op> a, uint32_t* words, int n_words) {
+    const Share s((uint32_t)min(a.stage_units, a.units), (uint32_t)a.vecs);
+    if (threadIdx.x == 0)
+        for (uint32_t part = 0; part < kParts; ++part)
+            half_share(a, s, 0, part, [](uint32_t, const uint4* src, uint32_t n) { bulk_prefetch(src, n * 16); });
+    for (int i = blockIdx.x * 32 + threadIdx.x; i < n_words; i += gridDim.x * 32) words[i] = 0u;
+}
+
+template <class Op>
+__global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_constant__ Args<Op> a) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ uint64_t full[2], known[2], part_free[2][kParts];
+    __shared__ typename Op::Acc seg_acc[kMaxSegments];
+    __shared__ Segment<Op> segment[2][kMaxSegments];
+    __shared__ uint16_t holders[kMaxSegments][2];       // first and last block of every segment's unit
+    __shared__ volatile int lost, give_up;
+    __shared__ int last;
+    static_assert(kSmemBytes + sizeof(segment) + sizeof(seg_acc) + 768 <= 232448, "shared memory of a block");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int stages = (a.units + a.stage_units - 1) / a.stage_units;
+    const uint32_t vecs = (uint32_t)a.vecs, tensors = (uint32_t)a.tensors;
+    if (tid == 0) {
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(smem_u32(&full[i]), 1);
+            mbar_init(smem_u32(&known[i]), 1);
+            for (int part = 0; part < kParts; ++part) mbar_init(smem_u32(&part_free[i][part]), kWorkers / 32);
+        }
+        fence_mbar_init();
+        lost = give_up = 0;
+    }
+    if (tid < kMaxSegments) seg_acc[tid] = typename Op::Acc(0);
+    // rows that follow tensor 0 without counting are converted last, an equal share of them per block;
+    // those of a small call are on their way to L2 from the start
+    uint32_t f_lo = 0, f_hi = 0;
+    if (a.follow_vecs > 0 && !a.follow_counts) {
+        const uint32_t total = (uint32_t)(a.units / a.tensors) * a.follow_vecs;
+        const uint32_t each = total / gridDim.x, more = total - each * gridDim.x;
+        f_lo = each * blockIdx.x + min(blockIdx.x, more);
+        f_hi = f_lo + each + (blockIdx.x < more ? 1u : 0u);
+        if (f_lo + tid * 8 < f_hi) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.follow_x + f_lo + tid * 8));
+    }
+    __syncthreads();
+    const Share share_full((uint32_t)min(a.stage_units, a.units), vecs);
+    const Share share_last((uint32_t)(a.units - (stages - 1) * a.stage_units), vecs);
+
+    if (warp == kWorkers / 32) {
+        // ============================== loads ==============================
+        if (lane == 0) {
+            int issued = 0;     // stages
+            bool on = true;
+            auto pieces = [&](int stage, uint32_t part, auto to) {
+                half_share(a, stage + 1 < stages ? share_full : share_last, stage, part, to);
+            };
+            auto wait = [&](uint32_t bar, uint32_t parity) {
+                const int64_t t0 = clock64();
+                bool done = mbar_test_wait(bar, parity);
+                while (!done && !give_up && clock64() - t0 < kWaitClocks) done = mbar_try_wait(bar, parity);
+                return done;
+            };
+            auto load = [&](int stage, uint32_t part) {
+                const uint32_t buf = stage & 1, bar = smem_u32(&full[buf]);
+                if (part == 0) {
+                    mbar_arrive_expect_tx(bar, (stage + 1 < stages ? share_full : share_last).n * 16);
+                    issued = stage + 1;
+                }
+                pieces(stage, part, [&](uint32_t i0, const uint4* src, uint32_t n) {
+                    bulk_load(smem_u32(smem) + (buf * kBufVecs + i0) * 16, src, n * 16, bar);
+                });
+            };
+            // What is requested waits in line before the exchange's words: a stage is requested when
+            // the exchange of the stage two before it is over, and is in L2 by the next exchange.
+            load(0, 0);
+            load(0, 1);
+            if (stages > 1) {
+                on = wait(smem_u32(&full[0]), 0);
+                if (on) load(1, 0);
+                if (on) load(1, 1);
+            }
+            for (int stage = 2; stage < stages && on; ++stage) {
+                const uint32_t buf = stage & 1, parity = ((stage >> 1) - 1) & 1;
+                on = wait(smem_u32(&known[buf]), parity);
+                for (uint32_t part = 0; part < kParts && on; ++part)
+                    pieces(stage, part, [&](uint32_t, const uint4* src, uint32_t n) { bulk_prefetch(src, n * 16); });
+                for (uint32_t part = 0; part < kParts && on; ++part) {
+                    on = wait(smem_u32(&part_free[buf][part]), parity);
+                    if (on) load(stage, part);
+                }
+            }
+            if (!on) {
+                lost = 1;
+                // copies land before the block exits (bounded: an aborted stage's last part was never issued)
+                const int64_t t0 = clock64();
+                for (int stage = max(0, issued - 2); stage < issued; ++stage)
+                    while (clock64() - t0 < kWaitClocks / 4 && !mbar_try_wait(smem_u32(&full[stage & 1]), (stage >> 1) & 1)) {}
+            }
+        }
+        __syncwarp();
+    } else if (warp > kWorkers / 32) {
+        // ============================== exchange ==============================
+        for (int stage = 0; stage < stages; ++stage) {
+            const Share& s = stage + 1 < stages ? share_full : share_last;
+            const uint32_t u0 = (uint32_t)(stage * a.stage_units) + s.unit;
+            uint32_t* const slots =
+                a.slots + (stage + 1 == stages ? a.last_set : stage & 1) * a.slots_per_set * Op::kSlotWords;
+            const uint32_t tag = (uint32_t)stage + 1;
+            if (stage == 0 || (stage + 1 == stages && share_last.total != share_full.total)) {
+                for (uint32_t g = lane; g < s.segs; g += 32) {
+                    holders[g][0] = (uint16_t)s.holder((s.unit + g) * vecs);
+                    holders[g][1] = (uint16_t)s.holder((s.unit + g + 1) * vecs - 1);
+                }
+            }
+            sync_exchange();        // A: the share is reduced
+            // (block b and unit u of the stage meet at most once, and b + u names the meeting)
+            for (uint32_t g = lane; g < s.segs; g += 32) {
+                Op::publish(slots, a.slots_per_set, blockIdx.x + s.unit + g, tag, seg_acc[g]);
+                seg_acc[g] = typename Op::Acc(0);
+            }
+            __syncwarp();
+            // Collect the values of this share's units: `width` lanes per segment (where a share has
+            // more than four segments, its units span two blocks at most).
+            const uint32_t width = s.segs <= 1 ? 32 : s.segs == 2 ? 16 : s.segs <= 4 ? 8 : 1;
+            const bool none_empty = s.total >= 8 * gridDim.x;
+            bool there = !lost;
+            const int64_t t0 = clock64();
+            for (uint32_t g0 = 0; g0 < s.segs; g0 += 32 / width) {
+                const uint32_t g = g0 + lane / width;
+                typename Op::Acc v = typename Op::Acc(0);
+                if (g < s.segs) {
+                    constexpr int kBatch = 5;       // polls under way at a time: 148 blocks at 32 a row
+                    const uint32_t u = s.unit + g, b1 = holders[g][1];
+                    for (uint32_t b0 = holders[g][0] + lane % width; b0 <= b1; b0 += kBatch * width) {
+                        typename Op::Raw raw[kBatch];
+                        for (bool all = false; there && !all;) {
+#pragma unroll
+                            for (int k = 0; k < kBatch; ++k) raw[k] = Op::load(slots, a.slots_per_set, min(b0 + k * width, b1) + u);
+                            all = true;
+#pragma unroll
+                            for (int k = 0; k < kBatch; ++k) {
+                                const uint32_t b = min(b0 + k * width, b1);
+                                all &= Op::tagged(raw[k], tag) || (!none_empty && cut(s.total, b) == cut(s.total, b + 1));
+                            }
+                            if (!all) there = !lost && clock64() - t0 < kWaitClocks;
+                        }
+#pragma unroll
+                        for (int k = 0; k < kBatch; ++k)
+                            if (b0 + k * width <= b1 && there && Op::tagged(raw[k], tag)) v = Op::combine(v, Op::value(raw[k]));
+                    }
+                }
+                __syncwarp();
+                for (uint32_t o = width >> 1; o > 0; o >>= 1) v = Op::combine(v, Op::shuffle(v, o));
+                if (g < s.segs && lane % width == 0) {
+                    const uint32_t unit = u0 + g, head = unit / tensors, z = unit - head * tensors;
+                    Segment<Op>& seg = segment[stage & 1][g];
+                    seg.result = Op::result(a.op, v);
+                    seg.begin = s.begin(g, vecs);
+                    seg.end = s.end(g, vecs);
+                    seg.head = head;
+                    seg.at = (int32_t)(s.at(g) - seg.begin);
+                    seg.out = static_cast<uint8_t*>(a.out[z]) + ((int64_t)head * vecs + seg.at) * Op::kOutBytes;
+                    if (there && (g > 0 || s.skip == 0)) {      // the unit begins here
+                        if (a.result_out[z] != nullptr) a.result_out[z][head] = Op::output(seg.result);
+                        if (z == 0 && a.follow_vecs > 0 && !a.follow_counts) Op::publish(a.heads, 0, head, 1, v);
+                    }
+                }
+            }
+            if (!__all_sync(0xffffffffu, there) && lane == 0) {
+                if (atomicCAS(a.status, 0u, (uint32_t)FP8ATTN_ERR_TIMEOUT) == 0u)
+                    a.status[1] = (kDetailGridWait << 24) | (blockIdx.x & 0xFFFFFFu);
+                give_up = 1;
+            }
+            if (lane == 0) mbar_arrive(smem_u32(&known[stage & 1]));
+            sync_exchange();        // B: results are known
+            if (give_up) break;
+        }
+    } else {
+        // ============================== workers ==============================
+        // Rows that follow tensor 0 and count: a block takes them in proportion to its segment of the
+        // head (so that their values join the segment's).
+        auto follow_range = [&](const Share& s, uint32_t g, uint32_t u0, uint32_t& head, uint32_t& f0, uint32_t& f1) {
+            const uint32_t unit = u0 + s.unit + g, at = s.at(g);
+            head = unit / tensors;
+            if (unit - head * tensors != 0) return false;
+            f0 = (uint32_t)((uint64_t)at * a.follow_vecs / vecs);
+            f1 = (uint32_t)((uint64_t)(at + s.end(g, vecs) - s.begin(g, vecs)) * a.follow_vecs / vecs);
+            return true;
+        };
+        auto convert = [&](int stage, uint32_t part) {
+            const Share& s = stage + 1 < stages ? share_full : share_last;
+            const uint4* buf = reinterpret_cast<const uint4*>(smem) + (stage & 1) * kBufVecs;
+            const uint32_t p0 = part == 0 ? 0 : s.half(), p1 = part == 0 ? s.half() : s.n;
+            for (uint32_t g = 0; g < s.segs; ++g) {
+                const Segment<Op>& seg = segment[stage & 1][g];
+                const uint32_t i0 = max(p0, seg.begin), i1 = min(p1, seg.end);
+                if (i0 < i1) Op::template convert<false>(a.op, seg, buf, i0, i1, tid);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&part_free[stage & 1][part]));
+        };
+        for (int stage = 0; stage <= stages; ++stage) {
+            if (stage < stages) {
+                const Share& s = stage + 1 < stages ? share_full : share_last;
+                const uint4* buf = reinterpret_cast<const uint4*>(smem) + (stage & 1) * kBufVecs;
+                const uint32_t bar = smem_u32(&full[stage & 1]), parity = (stage >> 1) & 1;
+                bool landed = mbar_test_wait(bar, parity);
+                if (!landed) {
+                    const int64_t t0 = clock64();
+                    while (!landed && !lost && clock64() - t0 < kWaitClocks) landed = mbar_try_wait(bar, parity);
+                }
+                if (!__all_sync(0xffffffffu, landed)) lost = 1;
+                for (uint32_t g = 0; g < s.segs; ++g) {
+                    const uint32_t b = s.begin(g, vecs), e = s.end(g, vecs);
+                    if (b + (tid & ~31) >= e && !a.follow_counts) continue;      // (whole warps)
+                    typename Op::Acc v = typename Op::Acc(0);
+                    if (b + tid < e) v = Op::reduce(buf + b, e - b, tid);
+                    uint32_t head, f0, f1;
+                    if (a.follow_counts && follow_range(s, g, (uint32_t)(stage * a.stage_units), head, f0, f1) && f0 + tid < f1)
+                        v = Op::combine(v, Op::reduce(a.follow_x + (int64_t)head * a.follow_vecs + f0, f1 - f0, tid));
+                    v = Op::warp_combine(v);
+                    if (lane == 0) Op::merge(&seg_acc[g], v);
+                }
+                sync_exchange();    // A
+            }
+            if (stage > 0) {
+                convert(stage - 1, 1);
+                const Share& s = stage < stages ? share_full : share_last;
+                for (uint32_t g = 0; a.follow_counts && g < s.segs; ++g) {
+                    Segment<Op> seg = segment[(stage - 1) & 1][g];
+                    uint32_t head, f0, f1;
+                    if (!follow_range(s, g, (uint32_t)((stage - 1) * a.stage_units), head, f0, f1)) continue;
+                    const int64_t first = (int64_t)head * a.follow_vecs;
+                    seg.out = static_cast<uint8_t*>(a.follow_out) + first * Op::kOutBytes;
+                    Op::template convert<true>(a.op, seg, a.follow_x + first, f0, f1, tid);
+                }
+            }
+            if (stage < stages) {
+                sync_exchange();    // B
+                if (give_up) break;
+                convert(stage, 0);
+            }
+        }
+    }
+    __syncthreads();
+    // ---- rows that follow tensor 0 ----
+    if (!give_up) {
+        bool there = true;
+        const int64_t t0 = clock64();
+        Segment<Op> seg;
+        seg.at = 0;
+        seg.out = static_cast<uint8_t*>(a.follow_out);
+        for (uint32_t x = f_lo; x < f_hi && there;) {
+            seg.head = x / a.follow_vecs;
+            const uint32_t end = f_hi - seg.head * a.follow_vecs < a.follow_vecs ? f_hi : (seg.head + 1) * a.follow_vecs;
+            typename Op::Raw raw = Op::load(a.heads, 0, seg.head);
+            while (there && !Op::tagged(raw, 1)) {
+                there = clock64() - t0 < kWaitClocks;
+                raw = Op::load(a.heads, 0, seg.head);
+            }
+            seg.result = Op::result(a.op, Op::value(raw));
+            if (there && tid < kWorkers) Op::template convert<true>(a.op, seg, a.follow_x, x, end, tid);
+            x = end;
+        }
+        if (!there && atomicCAS(a.status, 0u, (uint32_t)FP8ATTN_ERR_TIMEOUT) == 0u)
+            a.status[1] = (kDetailGridWait << 24) | (blockIdx.x & 0xFFFFFFu);
+    }
+    // ---- the last block to finish leaves everything at zero for the next call ----
+    __syncthreads();
+    // (what a block has collected it has read: nothing to fence)
+    if (tid == 0) last = atomicAdd(a.counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (last) {
+        for (uint32_t i = tid; i < a.sets * a.slots_per_set * Op::kSlotWords; i += kThreads) a.slots[i] = 0u;
+        if (a.follow_vecs > 0)
+            for (int i = tid; i < a.units / a.tensors * Op::kSlotWords; i += kThreads) a.heads[i] = 0u;
+        if (tid == 0) *a.counter = 0u;
+    }
+}
+
+// Fills stage_units and the published words' places in `words` (n_words of them) and returns the grid, or 0
+// where this path does not take the call: a unit that does not fit one buffer of every SM, heads so
+// short that a share would have too many segments, or too little room.
+template <class Op>
+unsigned plan(Args<Op>& a, int sms, uint32_t* words, int64_t n_words) {
+    if (a.units <= 0 || a.vecs <= 0 || a.vecs % 8 != 0) return 0;     // (shares end on multiples of eight vectors)
+    if ((uint64_t)a.follow_vecs * (uint64_t)(a.units / a.tensors) > 0x7fffffffull) return 0;
+    // at least 1 KB per block
+    const int64_t all = a.vecs * a.units;
+    const int64_t grid = all / 64 < 1 ? 1 : all / 64 > sms ? sms : all / 64;
+    const int64_t room = grid * kBufVecs;
+    if (a.vecs > room) return 0;
+    // (stages as large as fit: half as large, calls of many short heads take a third longer, because
+    // a stage costs 3.5 us however short)
+    const int64_t fit = room / a.vecs;
+    int64_t stages = (a.units + fit - 1) / fit;
+    a.stage_units = (int)((a.units + stages - 1) / stages);
+    stages = (a.units + a.stage_units - 1) / a.stage_units;
+    const int64_t share = (a.stage_units * a.vecs + grid - 1) / grid + 7;
+    if (share / a.vecs + 2 > kMaxSegments || stages > 0xfff0) return 0;
+    const bool shorter = stages > 2 && stages * a.stage_units != a.units;
+    a.sets = shorter ? 3 : stages > 1 ? 2 : 1;
+    a.last_set = shorter ? 2 : (int)(stages - 1) & 1;
+    const int64_t per_set = grid + a.stage_units, used = a.sets * per_set * Op::kSlotWords;
+    a.slots = words;
+    a.slots_per_set = (uint32_t)per_set;
+    a.heads = words + used;
+    if (used + (a.follow_vecs > 0 ? a.units / a.tensors * Op::kSlotWords : 0) > n_words) return 0;
+    return (unsigned)grid;
+}
+
+template <class Op>
+int launch(const Args<Op>& a, unsigned grid, bool clear, uint32_t* words, int n_words, cudaStream_t stream) {
+    // (the opt-in to large dynamic shared memory is per device and context: set on every call)
+    if (cudaFuncSetAttribute(staged_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) !=
+        cudaSuccess)
+        return FP8ATTN_ERR_CUDA;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeCooperative;
+    attr.val.cooperative = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (clear) {
+        clear_and_fetch_kernel<Op><<<grid, 32, 0, stream>>>(a, words, n_words);
+        count_launch();
+    }
+    if (cudaLaunchKernelEx(&cfg, staged_kernel<Op>, a) != cudaSuccess) return FP8ATTN_ERR_CUDA;
+    count_launch();
+    return FP8ATTN_OK;
+}
+
+}  // namespace staged
+}  // namespace fp8attn

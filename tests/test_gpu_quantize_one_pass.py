@@ -1,0 +1,64 @@
+"""The one-pass quantizer (heads held on chip between the maximum and the conversion) against the
+two-launch form, which the other tests hold against the oracle: same codes and scales, bit for bit.
+Shapes at its edges: one stage and several, a shorter last stage, shares of one segment and of many,
+heads just below and above what fits, test rows that outnumber the train rows, every call twice on
+one workspace (it has to leave its words clean)."""
+import pytest
+import torch
+
+from paper_2609_13031_b200 import api
+
+pytestmark = pytest.mark.gpu
+
+
+def tensors(B, H, rows, d, dtype, seed):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    return [torch.empty((B, H, r, d), dtype=dtype, device="cuda").normal_(generator=g) if r else None for r in rows]
+
+
+@pytest.mark.parametrize("B,H,n,m,d,dtype,flags", [
+    (1, 1, 1, 0, 64, "bf16", 0),
+    (1, 3, 1, 5, 128, "fp16", 0),
+    (1, 2, 257, 31, 64, "bf16", 0),
+    (2, 5, 1000, 77, 128, "fp16", api.QUERY_SCALE_FROM_ALL_ROWS),
+    (4, 16, 63, 9, 64, "bf16", 0),                   # many segments per share
+    (1, 7, 9001, 300, 128, "bf16", 0),               # 21 units in two stages: a shorter last one
+    (1, 11, 12289, 64, 128, "bf16", api.QUERY_SCALE_FROM_ALL_ROWS),
+    (1, 7, 20011, 3001, 128, "bf16", 0),             # 21 units, three at a time
+    (1, 4, 30001, 0, 128, "fp16", 0),                # 12 units, two at a time
+    (1, 2, 65536, 1, 128, "bf16", 0),                # the largest head that fits
+    (1, 1, 65600, 100, 128, "bf16", 0),              # the first that does not
+    (1, 3, 300, 40000, 64, "bf16", 0),               # test rows outnumber the train rows
+    (1, 2, 500, 3000, 64, "bf16", api.QUERY_SCALE_FROM_ALL_ROWS),
+    (3, 100, 16, 4, 64, "bf16", 0),
+])
+def test_one_pass_matches_two_launches(B, H, n, m, d, dtype, flags):
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float16
+    ws = api.new_workspace(B, H)
+    for seed in (1, 2):
+        x = tensors(B, H, (n, n, n, m), d, tdt, seed)
+        got = api.quantize_qkv(*x, ws, flags=flags)
+        want = api.quantize_qkv(*x, ws, flags=flags | api.QKV_TWO_LAUNCHES)
+        again = api.quantize_qkv(*x, ws, flags=flags)
+        for name in ("q8", "k8", "v8", "t8", "sq", "sk", "sv"):
+            assert torch.equal(got[name], want[name]), name
+            assert torch.equal(again[name], want[name]), name
+        code, scale = api.quantize(x[1], ws)
+        assert torch.equal(code, want["k8"]) and torch.equal(scale, want["sk"])
+    assert api.last_device_status(ws) == (0, 0)
+
+
+def test_workspace_shared_with_other_calls():
+    """The words of the one-pass kernel are its own: perturbation, ordered quantization and the
+    two-launch form in between change nothing."""
+    x = tensors(1, 4, (3000, 3000, 3000, 100), 64, torch.bfloat16, 3)
+    ws = api.new_workspace(1, 4)
+    first = api.quantize_qkv(*x, ws)
+    api.perturb(x[1], 0.05, 1, 1, ws)
+    api.quantize_qkv(*x, ws, order_keys=True)
+    api.quantize_qkv(*x, ws, flags=api.QKV_TWO_LAUNCHES)
+    second = api.quantize_qkv(*x, ws)
+    for name in ("q8", "k8", "v8", "t8", "sq", "sk", "sv"):
+        assert torch.equal(first[name], second[name]), name
+    assert api.last_device_status(ws) == (0, 0)
