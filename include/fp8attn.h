@@ -219,19 +219,21 @@ int bf16attn_icl_forward(const void* q_train, const void* q_test, const void* k,
  * outputs of bf16attn_icl_forward_ex (which then is an fp16 kernel).
  *
  * FP8ATTN_SPLIT_TAIL balances the last, partly filled round of the launch.  The
- * grid is one CTA per 256 query rows of a head (per 384 at d = 64 in launches of
- * eight rounds and more, which the split does not apply to); when the number of CTAs is not
+ * grid is one CTA per 256 query rows of a head (384 in some launches at d = 64, see
+ * fp8attn_attention_rows_per_cta); when the number of CTAs is not
  * a multiple of the number of SMs, the CTAs left over after the last full
  * round would run alone on a fraction of the GPU.  With this flag each of them
- * is replaced by up to 16 CTAs that share its query rows and divide the train
+ * is replaced by up to 40 CTAs that share its query rows and divide the train
  * keys between them, followed by a small kernel that combines their partial
  * results (the online softmax of the paper's kernel, applied once more across
- * key ranges).  The workspace must then be at least
- * fp8attn_workspace_bytes(B, H, n_train, n_test, d) with n_train > 0, which
- * includes the scratch for the partial results, else
- * FP8ATTN_ERR_WORKSPACE.  The split is applied only where it was measured to
+ * key ranges).  The workspace must then include scratch for the partial results:
+ * at least 256 rows of d + 4 floats per SM beyond the size that
+ * fp8attn_workspace_bytes returns for n_train = 0, else FP8ATTN_ERR_WORKSPACE;
+ * fp8attn_workspace_bytes(B, H, n_train, n_test, d) with n_train > 0 includes all
+ * that the split can use.  The split is applied only where it was measured to
  * pay (launches of fewer than 8 CTAs per SM whose key ranges keep at least
- * four steps); elsewhere the flag changes nothing.  Results stay within the same tolerances, but which
+ * four steps); elsewhere the flag changes nothing but, at d = 64, the rows per CTA.
+ * Results stay within the same tolerances, but which
  * rows take the split path depends on the sizes of the call, so a row's result
  * is no longer bit-identical across calls with different n_test.
  *
@@ -265,9 +267,11 @@ int fp8attn_gate_use_fp8(int64_t n_train);
 /* Informational, host only (the paper has no counterpart): the number of query rows that
  * one CTA of the forward calls takes for a call of these sizes and flags on the current
  * device: 256 (two 128-row tiles), or 384 (three) at d = 64 when the grid of 384-row
- * blocks fills the SMs at least eight times over.  Without a device the SM count of a
- * B200 (148) is assumed.  0 for unsupported sizes.  Results do not depend on it beyond the
- * order of the online softmax (steps of 128 or 96 keys). */
+ * blocks fills the SMs at least eight times over or, with FP8ATTN_SPLIT_TAIL, when that of
+ * 256-row blocks does or when a launch of less than one round is over sooner that way.
+ * Without a device the SM count of a B200 (148) is assumed.  0 for unsupported sizes.
+ * Results do not depend on it beyond the order of the online softmax (steps of 128 or 96
+ * keys). */
 int fp8attn_attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d, uint32_t flags);
 
 /* Seeded Gaussian perturbation of Q, K or V (paper appendix, Eq. 3: the noise
@@ -376,8 +380,8 @@ int fp8attn_host_step_status(void* device_scratch, int B, int H, int64_t n_train
 
 /* Bytes of workspace the calls above need: a few KB for the status words and the
  * per-head accumulators (all that is returned for n_train = 0), plus, for
- * n_train > 0 and d in {64, 128}, the scratch of FP8ATTN_SPLIT_TAIL (about 13 MB
- * at d = 64, 26 MB at d = 128; independent of n_train and n_test).  A workspace
+ * n_train > 0 and d in {64, 128}, the scratch of FP8ATTN_SPLIT_TAIL (about 15 MB
+ * at d = 64, 20 MB at d = 128; independent of n_train and n_test).  A workspace
  * of the smaller size serves every call that does not set that flag. */
 size_t fp8attn_workspace_bytes(int B, int H, int64_t n_train, int64_t n_test, int d);
 

@@ -9,7 +9,7 @@ namespace fp8attn {
 static std::atomic<uint64_t> g_launches{0};
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
-size_t split_scratch_bytes(int d) {
+size_t split_scratch_bytes(int d, int rows) {
     // one unit per SM at most; without a device to ask (size queries on a host without
     // a GPU) the size assumes the largest sm_100 part
     constexpr int kSmsWithoutDevice = 160;
@@ -17,7 +17,7 @@ size_t split_scratch_bytes(int d) {
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
         sms = kSmsWithoutDevice;
-    return (size_t)sms * 256 * (size_t)(d + 4) * sizeof(float);
+    return (size_t)sms * (size_t)rows * (size_t)(d + 4) * sizeof(float);
 }
 
 namespace {
@@ -67,7 +67,7 @@ int forward(bool fp8, const void* q_train, const void* q_test, const void* k, co
     if (!(softmax_scale == softmax_scale) || isinf(softmax_scale)) return FP8ATTN_ERR_INVALID_ARG;
     rc = check_workspace(workspace, workspace_bytes_, B, H);
     if (rc != FP8ATTN_OK) return rc;
-    if ((flags & FP8ATTN_SPLIT_TAIL) && workspace_bytes_ < workspace_bytes(B, H) + split_scratch_bytes(d))
+    if ((flags & FP8ATTN_SPLIT_TAIL) && workspace_bytes_ < workspace_bytes(B, H) + split_scratch_bytes(d, 256))
         return FP8ATTN_ERR_WORKSPACE;
     rc = check_device();
     if (rc != FP8ATTN_OK) return rc;
@@ -289,7 +289,7 @@ int fp8attn_attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test
 size_t fp8attn_workspace_bytes(int B, int H, int64_t n_train, int64_t, int d) {
     if (B <= 0 || H <= 0) return 0;
     // with the size of an attention call: room for the tail split's partial results as well
-    if (n_train > 0 && (d == 64 || d == 128)) return workspace_bytes(B, H) + split_scratch_bytes(d);
+    if (n_train > 0 && (d == 64 || d == 128)) return workspace_bytes(B, H) + split_scratch_bytes(d, split_scratch_rows(d));
     return workspace_bytes(B, H);
 }
 

@@ -39,7 +39,6 @@ constexpr int kTileM = 128;           // query rows per tile
 // softmax warps per tile, then the Q K^T issuer, the TMA producer and two P V issuers (tiles
 // {0, 2} and {1}).
 template <int kT> constexpr int kRowsPerBlock = kT * kTileM;
-static_assert(kRowsPerBlock<2> == 256, "split_scratch_bytes() in api.cu sizes the scratch for blocks of 256 rows");
 template <int kT> constexpr int kNumThreads = (4 * kT + 4) * 32;
 // Register budgets after setmaxnreg.  The CTA's register pool is what it was launched with
 // (threads x registers at launch, as ptxas reports them for the launch bound);
@@ -51,7 +50,10 @@ template <int kT> constexpr bool kRegsFit =
     4 * kT * 32 * kRegsSoftmax<kT> + 4 * 32 * kRegsOther <= kNumThreads<kT> * kLaunchRegs<kT>;
 static_assert(kRegsFit<2> && kRegsFit<3>, "setmaxnreg budgets exceed the CTA's register pool");
 constexpr uint32_t kTmemCols = 512;
-constexpr int kMaxSplits = 16;        // key ranges a split query block is divided into, at most
+// Key ranges a split query block is divided into, at most.  (More would still be faster where a launch
+// has only a block or two, but every range rounds P against maxima of its own, and beyond this the
+// FP8 results move further from those of an unsplit launch than 3 %.)
+constexpr int kMaxSplits = 40;
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 
 // detail codes written next to FP8ATTN_ERR_TIMEOUT
@@ -95,11 +97,14 @@ struct Cfg {
     // (Layouts before this one, d = 128: FP8 with 96-key steps and an S region per tile,
     // 3.6 % more time; P written over S, where Q K^T has to wait for P V: the 16-bit kernel
     // took 10 % more time and 20 % more cycles that way.)
-    static constexpr uint32_t kColS = 0, kColO = 256;
-    static constexpr uint32_t kColP0 = kKeys, kPStride = kKeys / 2;   // P_t at kColP0 + t*kPStride
-    // FP8: P alternates between two buffers per tile (the second kPCols columns after the
-    // first), so that writing P of one step never waits for the P V of the step before.
-    static constexpr int kPBufs = kFp8 ? 2 : 1;
+    // 16 bits, d = 64, two tiles: room for two P buffers per tile as well (S | 2 x 2 x 64 | O0 | O1).
+    // (8 heads of 8,192 + 2,048 rows 236 -> 228 us)
+    static constexpr bool kRoomy = !kFp8 && kD == 64 && kT == 2;
+    static constexpr uint32_t kColS = 0, kColO = kRoomy ? 384 : 256;
+    static constexpr uint32_t kColP0 = kKeys, kPStride = kRoomy ? 128 : kKeys / 2;   // P_t at kColP0 + t*kPStride
+    // P alternates between two buffers per tile (the second kPCols columns after the first) where
+    // there is room, so that writing P of one step never waits for the P V of the step before.
+    static constexpr int kPBufs = kFp8 || kRoomy ? 2 : 1;
     // pairs of exponentials, out of every 16 pairs, that go to the FMA pipe (measured best)
     static constexpr int kPolyPer16 = kFp8 ? (kT == 3 ? 2 : 4) : 2;
     static_assert(kPBufs * kPCols <= (int)kPStride, "TMEM layout: P tiles overlap");
@@ -755,12 +760,14 @@ icl_attention_kernel(const __grid_constant__ CUtensorMap map_q_train,
 }
 
 // Combines the partial results of the split query blocks: with M = max_s c*m_s,
-// out = s_v * sum_s 2^(c*m_s - M) O_s / sum_s 2^(c*m_s - M) l_s.  One thread per row and
-// eight output columns.
+// out = s_v * sum_s 2^(c*m_s - M) O_s / sum_s 2^(c*m_s - M) l_s.  One thread per row and four output
+// columns.  Bound by the latency of its loads, which come from L2: eight ranges are under way at a
+// time (8 x 300 rows of d = 64 in 9 ranges: 6.9 us with one at a time).
 template <int kD, int kT>
 __global__ void __launch_bounds__(256)
 combine_split_kernel(const KernelArgs args, int units, int out_half, int fp8) {
-    const int per_row = kD / 8;
+    constexpr int kBatch = 8;
+    const int per_row = kD / 4;
     const int64_t tid = (int64_t)blockIdx.x * 256 + threadIdx.x;
     const int64_t unit = tid / (kRowsPerBlock<kT> * per_row);
     if (unit >= units) return;
@@ -776,33 +783,44 @@ combine_split_kernel(const KernelArgs args, int units, int out_half, int fp8) {
     const int bh_kv = (is_test && args.test_kv_head0) ? (bh / args.heads) * args.heads : bh;
     const float* base = args.partial + ((size_t)unit * args.splits * kRowsPerBlock<kT> + r) * kPartialStride<kD>;
     const size_t split_stride = (size_t)kRowsPerBlock<kT> * kPartialStride<kD>;
-    float mmax = -INFINITY;
-    for (int s = 0; s < args.splits; ++s) mmax = fmaxf(mmax, base[s * split_stride + kD]);
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    float lsum = 0.f;
-    for (int s = 0; s < args.splits; ++s) {
-        const float* ps = base + s * split_stride;
-        const float wgt = exp2f(ps[kD] - mmax);
-        lsum = fmaf(wgt, ps[kD + 1], lsum);
-        const float4 a = *reinterpret_cast<const float4*>(ps + g * 8);
-        const float4 b = *reinterpret_cast<const float4*>(ps + g * 8 + 4);
-        acc[0] = fmaf(wgt, a.x, acc[0]); acc[1] = fmaf(wgt, a.y, acc[1]);
-        acc[2] = fmaf(wgt, a.z, acc[2]); acc[3] = fmaf(wgt, a.w, acc[3]);
-        acc[4] = fmaf(wgt, b.x, acc[4]); acc[5] = fmaf(wgt, b.y, acc[5]);
-        acc[6] = fmaf(wgt, b.z, acc[6]); acc[7] = fmaf(wgt, b.w, acc[7]);
+    float m = -INFINITY, lsum = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < args.splits; s0 += kBatch) {
+        float2 ml[kBatch];
+        float4 o[kBatch];
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) {
+            const float* ps = base + (size_t)min(s0 + k, args.splits - 1) * split_stride;
+            ml[k] = *reinterpret_cast<const float2*>(ps + kD);
+            o[k] = *reinterpret_cast<const float4*>(ps + g * 4);
+        }
+        float m_new = m;
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) m_new = fmaxf(m_new, ml[k].x);     // (a repeated range changes no maximum)
+        const float f = exp2f(m - m_new);
+        m = m_new;
+        lsum *= f;
+        acc.x *= f; acc.y *= f; acc.z *= f; acc.w *= f;
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) {
+            const float wgt = s0 + k < args.splits ? exp2f(ml[k].x - m) : 0.f;
+            lsum = fmaf(wgt, ml[k].y, lsum);
+            acc.x = fmaf(wgt, o[k].x, acc.x); acc.y = fmaf(wgt, o[k].y, acc.y);
+            acc.z = fmaf(wgt, o[k].z, acc.z); acc.w = fmaf(wgt, o[k].w, acc.w);
+        }
     }
     const float inv = (fp8 ? args.scale_v[bh_kv] : 1.0f) / lsum;
-    uint4 v;
+    uint2 v;
     if (out_half) {
-        v.x = pack_f16x2(acc[0] * inv, acc[1] * inv); v.y = pack_f16x2(acc[2] * inv, acc[3] * inv);
-        v.z = pack_f16x2(acc[4] * inv, acc[5] * inv); v.w = pack_f16x2(acc[6] * inv, acc[7] * inv);
+        v.x = pack_f16x2(acc.x * inv, acc.y * inv);
+        v.y = pack_f16x2(acc.z * inv, acc.w * inv);
     } else {
-        v.x = pack_bf16x2(acc[0] * inv, acc[1] * inv); v.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
-        v.z = pack_bf16x2(acc[4] * inv, acc[5] * inv); v.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
+        v.x = pack_bf16x2(acc.x * inv, acc.y * inv);
+        v.y = pack_bf16x2(acc.z * inv, acc.w * inv);
     }
     __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(is_test ? args.out_test : args.out_train) +
                          ((int64_t)bh * q_rows + row) * kD;
-    *reinterpret_cast<uint4*>(out + g * 8) = v;
+    *reinterpret_cast<uint2*>(out + g * 4) = v;
 }
 
 template <bool kFp8, int kD, bool kHalf, int kT>
@@ -844,8 +862,7 @@ int launch(const AttnParams& p, cudaStream_t stream) {
     a.splits = 1;
     a.partial = nullptr;
     int units = 0;
-    // (three-tile launches have at least eight rounds, where the split does not pay)
-    if (kT == 2 && (p.flags & FP8ATTN_SPLIT_TAIL) && p.partial != nullptr) {
+    if ((p.flags & FP8ATTN_SPLIT_TAIL) && p.partial != nullptr) {
         int sms = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
             return FP8ATTN_ERR_CUDA;
@@ -870,7 +887,7 @@ int launch(const AttnParams& p, cudaStream_t stream) {
         }
     }
     auto kern = icl_attention_kernel<kFp8, kD, kHalf, kT, false>;
-    auto kern_split = icl_attention_kernel<kFp8, kD, kHalf, 2, true>;
+    auto kern_split = icl_attention_kernel<kFp8, kD, kHalf, kT, true>;
     // The opt-in to large dynamic shared memory is per device and per context; it is set on
     // every call (a cached flag would go stale when the context is destroyed).
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemBytes) !=
@@ -902,8 +919,8 @@ int launch(const AttnParams& p, cudaStream_t stream) {
         count_launch();
     }
     if (units > 0) {
-        const int64_t threads = (int64_t)units * kRowsPerBlock<kT> * (kD / 8);
-        combine_split_kernel<kD, 2><<<(unsigned)((threads + 255) / 256), 256, 0, stream>>>(
+        const int64_t threads = (int64_t)units * kRowsPerBlock<kT> * (kD / 4);
+        combine_split_kernel<kD, kT><<<(unsigned)((threads + 255) / 256), 256, 0, stream>>>(
             a, units, kHalf ? 1 : 0, kFp8 ? 1 : 0);
         count_launch();
     }
@@ -932,26 +949,52 @@ int launch_wait_timeout_selftest(uint32_t* status, uint64_t limit_ns, cudaStream
     return cudaGetLastError() == cudaSuccess ? FP8ATTN_OK : FP8ATTN_ERR_CUDA;
 }
 
-// d = 64: three tiles per CTA where the grid of 384-row blocks still fills the SMs at least
-// eight times over (there the last, partly filled round no longer matters, and neither does
-// the tail split); two tiles per CTA for smaller launches.
 template <bool kFp8, bool kHalf>
 int launch_d64(const AttnParams& p, cudaStream_t stream) {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
         return FP8ATTN_ERR_CUDA;
-    if (attention_rows_per_cta(p.B, p.H, p.n_train, p.n_test, 64, p.flags, sms) == kRowsPerBlock<3>)
+    if (attention_rows_per_cta(p.B, p.H, p.n_train, p.n_test, 64, p.flags, sms, p.partial_bytes) == kRowsPerBlock<3>)
         return launch<kFp8, 64, kHalf, 3>(p, stream);
     return launch<kFp8, 64, kHalf, 2>(p, stream);
 }
 
-int attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d, uint32_t flags, int sms) {
+// d = 64: two or three tiles per CTA.
+//  - Three where the grid of 384-row blocks fills the SMs at least eight times over: there the last,
+//    partly filled round no longer matters, and three softmax warps per scheduler are 4 % faster.
+//  - With FP8ATTN_SPLIT_TAIL, three from eight rounds of 256-row blocks on, where the split of
+//    two-tile launches ends: it takes care of the last round of these too (8 heads of 32,768 + 8,192
+//    rows, bf16: 3.27 -> 3.17 ms).
+//  - With FP8ATTN_SPLIT_TAIL, for a launch of less than one round (a few test rows against a long
+//    table, above all), whichever gives the shorter critical path: a block of T tiles takes kCost[T - 1]
+//    per key, and the more blocks there are the fewer key ranges each is split into.  300 rows of 8 heads
+//    against 262,144: two tiles 16 blocks in 9 ranges, 322 us; three tiles 8 blocks in 18, 236 us.
+//  - Two otherwise (small grids pay for coarse blocks in their last round).
+int attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d, uint32_t flags, int sms,
+                           size_t partial_bytes) {
     if (d != 64) return kRowsPerBlock<2>;
-    const int64_t rows3 = kRowsPerBlock<3>;
-    const int64_t blocks = ((flags & FP8ATTN_TEST_ROWS_ONLY) ? 0 : (n_train + rows3 - 1) / rows3) +
-                           (n_test + rows3 - 1) / rows3;
-    return (int64_t)B * H * blocks >= 8 * (int64_t)sms ? kRowsPerBlock<3> : kRowsPerBlock<2>;
+    const int64_t heads = (int64_t)B * H, train = (flags & FP8ATTN_TEST_ROWS_ONLY) ? 0 : n_train;
+    auto blocks = [&](int64_t rows) { return heads * ((train + rows - 1) / rows + (n_test + rows - 1) / rows); };
+    const int64_t blocks2 = blocks(kRowsPerBlock<2>), blocks3 = blocks(kRowsPerBlock<3>);
+    if (blocks3 >= 8 * (int64_t)sms) return kRowsPerBlock<3>;
+    if ((flags & FP8ATTN_SPLIT_TAIL) && blocks2 >= 8 * (int64_t)sms) return kRowsPerBlock<3>;
+    if ((flags & FP8ATTN_SPLIT_TAIL) && blocks2 > 0 && blocks2 < sms) {
+        constexpr float kCost[3] = {0.72f, 1.0f, 1.43f};     // time per key of one, two, three tiles
+        constexpr float kSplitSteps = 6.0f;                  // launch and combine, in steps of 128 keys
+        const float steps = (float)n_train / 128.0f;
+        const int64_t tiles = ((train > n_test ? train : n_test) + kTileM - 1) / kTileM;
+        auto time = [&](int t, int64_t n) {
+            const int64_t room = (int64_t)(partial_bytes / ((size_t)n * t * kTileM * kPartialStride<64> * sizeof(float)));
+            int64_t splits = sms / n < kMaxSplits ? sms / n : kMaxSplits;
+            if (splits > room) splits = room;
+            if (splits > steps / 4) splits = (int64_t)(steps / 4);
+            const float one = kCost[(tiles < t ? tiles : t) - 1] * steps;
+            return splits >= 2 ? one / (float)splits + kSplitSteps : one;
+        };
+        if (time(3, blocks3) < 0.97f * time(2, blocks2)) return kRowsPerBlock<3>;
+    }
+    return kRowsPerBlock<2>;
 }
 
 int launch_icl_attention(const AttnParams& p, bool fp8, cudaStream_t stream) {

@@ -37,8 +37,11 @@ inline size_t workspace_bytes(int B, int H) {
 }
 
 // Scratch of the tail split (FP8ATTN_SPLIT_TAIL), appended to the workspace: partial results
-// of fewer than one CTA per SM of the current device, 256 rows of d + 4 floats each (api.cu).
-size_t split_scratch_bytes(int d);
+// of fewer than one CTA per SM of the current device, `rows` rows of d + 4 floats each (api.cu).
+// A caller may bring scratch for CTAs of 256 rows; with 384 at d = 64 the split has all the room it
+// can use.
+size_t split_scratch_bytes(int d, int rows);
+inline int split_scratch_rows(int d) { return d == 64 ? 384 : 256; }
 
 void count_launch();
 
@@ -85,9 +88,10 @@ struct AttnParams {
     size_t partial_bytes;
 };
 int launch_icl_attention(const AttnParams& p, bool fp8, cudaStream_t stream);
-// Query rows per CTA that a forward call of these sizes uses on a device with `sms` SMs: 256, or
-// 384 at d = 64 where the grid of 384-row blocks fills the SMs at least eight times over.
-int attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d, uint32_t flags, int sms);
+// Query rows per CTA that a forward call of these sizes and flags uses on a device with `sms` SMs and
+// with that much scratch for the tail split: 256, or at d = 64 also 384 (attention.cu says when).
+int attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d, uint32_t flags, int sms,
+                           size_t partial_bytes = (size_t)1 << 40);
 int launch_wait_timeout_selftest(uint32_t* status, uint64_t limit_ns, cudaStream_t stream);
 
 }  // namespace fp8attn
