@@ -134,11 +134,12 @@ def launch_count() -> int:
 
 
 def _ptr(t: torch.Tensor | None):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream() -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+def _stream() -> int:
+    # the current device's current stream, without the 3 us of building a torch.cuda.Stream for it
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _check(fn: str, rc: int):
@@ -434,12 +435,32 @@ def icl_attention(q_train, q_test, k, v, workspace=None, softmax_scale: float = 
     B, H, n_train, d = _dims(k)
     if workspace is None:
         workspace = new_workspace(B, H, k.device, n_train=n_train if flags & SPLIT_TAIL else 0, d=d)
-    has_test = q_test is not None and q_test.shape[2] > 0
-    o = quantize_qkv(q_train, k, v, q_test if has_test else None, workspace)
-    q8, k8, v8, sq, sk, sv = o["q8"], o["k8"], o["v8"], o["sq"], o["sk"], o["sv"]
-    t8 = o["t8"] if has_test else None
-    return icl_forward_fp8(q8, t8, k8, v8, sq, sk, sv, workspace, softmax_scale, flags=flags,
-                           out_dtype=k.dtype)
+    n_test = 0 if q_test is None else q_test.shape[2]
+    for t in (q_train, k, v) + (() if n_test == 0 else (q_test,)):
+        assert t.dtype == k.dtype and _is16(t)
+    half = k.dtype == torch.float16
+    # The codes and scales stay inside this call: one allocation holds them all (nine tensors of their own
+    # cost a small call, whose kernels take 20 us, more time on the host than that).
+    train, test, heads = B * H * n_train * d, B * H * n_test * d, B * H
+    at = [0]
+    for nbytes in (train, train, train, test, 4 * heads, 4 * heads, 4 * heads):
+        at.append(at[-1] + (nbytes + 255) // 256 * 256)
+    codes = k.new_empty(at[-1], dtype=torch.uint8)
+    q8, k8, v8, t8, sq, sk, sv = (codes.data_ptr() + o for o in at[:-1])
+    out_train = None if flags & TEST_ROWS_ONLY else k.new_empty((B, H, n_train, d))
+    out_test = k.new_empty((B, H, n_test, d)) if n_test else None
+    lib, stream, ws, ws_bytes = load(), _stream(), workspace.data_ptr(), workspace.numel()
+    if n_test == 0:
+        q_test = t8 = None
+    rc = lib.fp8attn_quantize_qkv_ex(q_train.data_ptr(), k.data_ptr(), v.data_ptr(), _ptr(q_test), B, H, n_train,
+                                     n_test, d, q8, k8, v8, t8, sq, sk, sv, INPUT_FP16 if half else 0, ws, ws_bytes,
+                                     stream)
+    _check("fp8attn_quantize_qkv", rc)
+    rc = lib.fp8attn_icl_forward_ex(None if out_train is None else q8, t8, k8, v8, sq, sk, sv, B, H, n_train, n_test, d,
+                                    float(softmax_scale), int(flags) | (IO_FP16 if half else 0), _ptr(out_train),
+                                    _ptr(out_test), ws, ws_bytes, stream)
+    _check("fp8attn_icl_forward", rc)
+    return out_train, out_test
 
 
 def icl_attention_arms(q_train, q_test, k, v, fp8_train: bool, fp8_test: bool, workspace=None,
