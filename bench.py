@@ -521,7 +521,9 @@ def main():
         tf_attn = tf(ms_attn)
         peak_fp8 = NOMINAL_FP8_OVER_BF16 * peaks["bf16_tflops_sustained"]
         peak_fp8_burst = NOMINAL_FP8_OVER_BF16 * peaks["bf16_tflops"]
-        quant_bytes = w.B * w.H * w.d * (5 * 3 * w.n_train + 3 * w.n_test)
+        # heads that fit on chip are read once (3 bytes an element), others twice
+        one_pass = not order_keys and w.n_train * w.d * 2 <= 16 << 20
+        quant_bytes = w.B * w.H * w.d * ((3 if one_pass else 5) * 3 * w.n_train + 3 * w.n_test)
         if order_keys:
             # one more pass over K for the row norms, the norms written and read, the row map written and read twice
             quant_bytes += w.B * w.H * w.n_train * (2 * w.d + 4 * 5)
