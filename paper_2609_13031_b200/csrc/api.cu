@@ -122,7 +122,7 @@ int fp8attn_quantize_ex(const void* x_bf16, int B, int H, int64_t rows, int d, c
     return launch_quantize(x_bf16, (int64_t)B * H, rows * (int64_t)d, scale_in, x_fp8, scale_out, amax, flags,
                            reinterpret_cast<uint32_t*>(ws + kWsStatusOffset),
                            reinterpret_cast<uint32_t*>(ws + kWsCounterOffset),
-                           reinterpret_cast<uint32_t*>(ws + ws_words_offset(B, H)),
+                           reinterpret_cast<uint32_t*>(ws + kWsWordsOffset),
                            static_cast<cudaStream_t>(cuda_stream));
 }
 
@@ -160,7 +160,7 @@ int quantize_qkv_impl(const void* q_train, const void* k, const void* v, const v
                                n_test * (int64_t)d, q_train_fp8, k_fp8, v_fp8, q_test_fp8, scale_q, scale_k,
                                scale_v, amax, flags, reinterpret_cast<uint32_t*>(ws + kWsStatusOffset),
                                reinterpret_cast<uint32_t*>(ws + kWsCounterOffset),
-                               reinterpret_cast<uint32_t*>(ws + ws_words_offset(B, H)), stream, key_dest, d);
+                               reinterpret_cast<uint32_t*>(ws + kWsWordsOffset), stream, key_dest, d);
 }
 }  // namespace
 
@@ -301,8 +301,7 @@ int fp8attn_last_device_status(void* workspace, void* cuda_stream, uint32_t* det
     if (cudaMemcpy(words, workspace, sizeof(words), cudaMemcpyDeviceToHost) != cudaSuccess)
         return FP8ATTN_ERR_CUDA;
     if (detail) *detail = words[1];
-    // after an error: clear the status words, and the arrival counters a one-launch
-    // quantization that gave up may have left behind
+    // after an error: clear the status words, the counter and the words of the one-pass kernels
     if (words[0] != 0 && cudaMemset(workspace, 0, kWsAmaxOffset) != cudaSuccess) return FP8ATTN_ERR_CUDA;
     return (int)words[0];
 }

@@ -11,29 +11,30 @@ namespace fp8attn {
 // Workspace layout (device memory, caller-owned, zero-filled once):
 //   [0,4)    device status word (fp8attn_status_t, 0 = ok); first error wins
 //   [4,8)    detail code of that error (which wait expired, which CTA)
-//   [256, 256 + 12*B*H) three sets of per-(b,h) absmax accumulators (fp32 bit
-//                       patterns): one is used by fp8attn_quantize, all three (Q, K, V)
-//                       by fp8attn_quantize_qkv; cleared at the start of every call.
-//                       fp8attn_perturb keeps its per-head sums of squares (fp64) here too.
 //   [16,20)  blocks of a one-pass kernel that are done; zero between calls
-//   after the accumulators: the one-pass kernels' own words (values that their blocks publish to
-//                       one another), kOnePassWords + 4*B*H of them; zero between calls
+//   [256, 4352) the one-pass kernels' own words (values that their blocks publish to one another);
+//                       zero between calls.  Their place must not depend on B*H: one workspace
+//                       serves calls of all sizes up to its own, and nothing but these kernels
+//                       may ever write there.
+//   [4352, 4352 + 12*B*H) three sets of per-(b,h) absmax accumulators (fp32 bit
+//                       patterns): one is used by fp8attn_quantize, all three (Q, K, V)
+//                       by fp8attn_quantize_qkv; cleared at the start of every call that uses
+//                       them, left as they are at its end.  fp8attn_perturb keeps its per-head
+//                       sums of squares (fp64) here too.
 constexpr size_t kWsStatusOffset = 0;
 constexpr size_t kWsDetailOffset = 4;
 constexpr size_t kWsCounterOffset = 16;
-constexpr size_t kWsAmaxOffset = 256;
+constexpr size_t kWsWordsOffset = 256;
 constexpr int kOnePassWords = 1024;
+constexpr size_t kWsAmaxOffset = kWsWordsOffset + sizeof(uint32_t) * kOnePassWords;
 // detail code (bits 24..31 of the detail word) of an expired grid-wide wait of a one-pass kernel
 constexpr uint32_t kDetailGridWait = 32;
 
-inline size_t ws_amax_bytes(int B, int H) {
-    size_t amax = (size_t)12 * (size_t)B * (size_t)H;
-    return ((amax + 255) / 256) * 256;
-}
-inline size_t ws_words_offset(int B, int H) { return kWsAmaxOffset + ws_amax_bytes(B, H); }
+// (16 bytes per head beyond the accumulators are unused: the size that callers were told before)
 inline size_t workspace_bytes(int B, int H) {
-    size_t partial = sizeof(float) * ((size_t)kOnePassWords + (size_t)4 * (size_t)B * (size_t)H);
-    return ws_words_offset(B, H) + ((partial + 255) / 256) * 256;
+    const size_t heads = (size_t)B * (size_t)H;
+    auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+    return kWsWordsOffset + up(12 * heads) + up(sizeof(uint32_t) * kOnePassWords + 16 * heads);
 }
 
 // Scratch of the tail split (FP8ATTN_SPLIT_TAIL), appended to the workspace: partial results

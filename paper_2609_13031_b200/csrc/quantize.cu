@@ -239,10 +239,10 @@ struct QuantizeOp {
 constexpr int64_t kOneLaunchMaxBytes = 48ll << 20;
 
 // The one-pass kernel for tensors [0, tensors) of `b` and, if there is one, tensor 3 with the scale of
-// tensor 0.  *taken: whether it takes the call.
+// tensor 0.  *taken: whether it takes the call.  amax_bits: the accumulators of the two-pass form, free here.
 template <bool kHalf>
 int launch_staged(const QuantBatch& b, int tensors, int64_t n_heads, uint32_t* status, uint32_t* counters,
-                  uint32_t* words, int sms, bool* taken, cudaStream_t stream) {
+                  uint32_t* words, uint32_t* amax_bits, int sms, bool* taken, cudaStream_t stream) {
     using Op = QuantizeOp<kHalf>;
     staged::Args<Op> a = {};
     for (int z = 0; z < tensors; ++z) {
@@ -261,12 +261,11 @@ int launch_staged(const QuantBatch& b, int tensors, int64_t n_heads, uint32_t* s
     a.status = status;
     a.counter = counters;
     *taken = false;
-    const int n_words = (int)(kOnePassWords + 4 * n_heads);
-    const unsigned grid = follow > 0x7fffffffll ? 0u : staged::plan(a, sms, words, n_words);
+    const bool clear = (a.vecs * a.units + follow * n_heads) * 16 > kOneLaunchMaxBytes;
+    const unsigned grid = follow > 0x7fffffffll ? 0u : staged::plan(a, sms, words, clear ? amax_bits : nullptr);
     if (grid == 0) return FP8ATTN_OK;
     *taken = true;
-    const bool clear = (a.vecs * a.units + follow * n_heads) * 16 > kOneLaunchMaxBytes;
-    return staged::launch(a, grid, clear, words, n_words, stream);
+    return staged::launch(a, grid, clear, stream);
 }
 
 }  // namespace
@@ -309,8 +308,8 @@ int launch_quantize_qkv(const void* q_train, const void* k, const void* v, const
     const bool half = (flags & FP8ATTN_INPUT_FP16) != 0;
     if (!(flags & (FP8ATTN_SCALES_GIVEN | FP8ATTN_QKV_TWO_LAUNCHES)) && key_dest == nullptr && elems_train > 0) {
         bool taken = false;
-        const int rc = half ? launch_staged<true>(b, 3, n_heads, status, counters, words, sms, &taken, stream)
-                            : launch_staged<false>(b, 3, n_heads, status, counters, words, sms, &taken, stream);
+        const int rc = half ? launch_staged<true>(b, 3, n_heads, status, counters, words, amax_bits, sms, &taken, stream)
+                            : launch_staged<false>(b, 3, n_heads, status, counters, words, amax_bits, sms, &taken, stream);
         if (rc != FP8ATTN_OK || taken) return rc;
     }
     const int64_t want = ((int64_t)sms * 16 + n_heads * 3 - 1) / (n_heads * 3);
@@ -371,8 +370,8 @@ int launch_quantize(const void* x_bf16, int64_t n_heads, int64_t elems_per_head,
         b.pairs_per_head[0] = pairs;
         b.scale_out[0] = scale_out;
         bool taken = false;
-        const int rc = half ? launch_staged<true>(b, 1, n_heads, status, counters, words, sms, &taken, stream)
-                            : launch_staged<false>(b, 1, n_heads, status, counters, words, sms, &taken, stream);
+        const int rc = half ? launch_staged<true>(b, 1, n_heads, status, counters, words, amax_bits, sms, &taken, stream)
+                            : launch_staged<false>(b, 1, n_heads, status, counters, words, amax_bits, sms, &taken, stream);
         if (rc != FP8ATTN_OK || taken) return rc;
     }
     if (scale_in == nullptr) {

@@ -140,12 +140,15 @@ __device__ __forceinline__ void half_share(const Args<Op>& a, const Share& s, in
 // A launch of its own before large calls: clears the words and has the first stage fetched to L2
 // meanwhile (the launch then costs nothing).  One warp per block, the grid of staged_kernel.
 template <class Op>
-__global__ void clear_and_fetch_kernel(const __grid_constant__ Args<Op> a, uint32_t* words, int n_words) {
+__global__ void clear_and_fetch_kernel(const __grid_constant__ Args<Op> a) {
     const Share s((uint32_t)min(a.stage_units, a.units), (uint32_t)a.vecs);
     if (threadIdx.x == 0)
         for (uint32_t part = 0; part < kParts; ++part)
             half_share(a, s, 0, part, [](uint32_t, const uint4* src, uint32_t n) { bulk_prefetch(src, n * 16); });
-    for (int i = blockIdx.x * 32 + threadIdx.x; i < n_words; i += gridDim.x * 32) words[i] = 0u;
+    const uint32_t t = blockIdx.x * 32 + threadIdx.x, threads = gridDim.x * 32;
+    for (uint32_t i = t; i < a.sets * a.slots_per_set * Op::kSlotWords; i += threads) a.slots[i] = 0u;
+    if (a.follow_vecs > 0)
+        for (uint32_t i = t; i < (uint32_t)(a.units / a.tensors) * Op::kSlotWords; i += threads) a.heads[i] = 0u;
 }
 
 template <class Op>
@@ -417,11 +420,13 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
     }
 }
 
-// Fills stage_units and the published words' places in `words` (n_words of them) and returns the grid, or 0
-// where this path does not take the call: a unit that does not fit one buffer of every SM, heads so
-// short that a share would have too many segments, or too little room.
+// Fills stage_units and the published words' places and returns the grid, or 0 where this path does not
+// take the call: a unit that does not fit one buffer of every SM, heads so short that a share would
+// have too many segments, or too little room.  `words`: the workspace's kOnePassWords, which are zero
+// between calls; `cleared_heads`: one word per head that the call clears first (NULL: it clears
+// nothing, all its words are among `words`).
 template <class Op>
-unsigned plan(Args<Op>& a, int sms, uint32_t* words, int64_t n_words) {
+unsigned plan(Args<Op>& a, int sms, uint32_t* words, uint32_t* cleared_heads) {
     if (a.units <= 0 || a.vecs <= 0 || a.vecs % 8 != 0) return 0;     // (shares end on multiples of eight vectors)
     if ((uint64_t)a.follow_vecs * (uint64_t)(a.units / a.tensors) > 0x7fffffffull) return 0;
     // at least 8 KB per block: with fewer blocks there is less to exchange (2 heads of 512 + 128 rows x 64:
@@ -444,13 +449,14 @@ unsigned plan(Args<Op>& a, int sms, uint32_t* words, int64_t n_words) {
     const int64_t per_set = grid + a.stage_units, used = a.sets * per_set * Op::kSlotWords;
     a.slots = words;
     a.slots_per_set = (uint32_t)per_set;
-    a.heads = words + used;
-    if (used + (a.follow_vecs > 0 ? a.units / a.tensors * Op::kSlotWords : 0) > n_words) return 0;
+    a.heads = cleared_heads != nullptr ? cleared_heads : words + used;
+    const int64_t head_words = cleared_heads == nullptr && a.follow_vecs > 0 ? a.units / a.tensors * Op::kSlotWords : 0;
+    if (used + head_words > kOnePassWords) return 0;
     return (unsigned)grid;
 }
 
 template <class Op>
-int launch(const Args<Op>& a, unsigned grid, bool clear, uint32_t* words, int n_words, cudaStream_t stream) {
+int launch(const Args<Op>& a, unsigned grid, bool clear, cudaStream_t stream) {
     // (the opt-in to large dynamic shared memory is per device and context: set on every call)
     if (cudaFuncSetAttribute(staged_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) !=
         cudaSuccess)
@@ -466,7 +472,7 @@ int launch(const Args<Op>& a, unsigned grid, bool clear, uint32_t* words, int n_
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     if (clear) {
-        clear_and_fetch_kernel<Op><<<grid, 32, 0, stream>>>(a, words, n_words);
+        clear_and_fetch_kernel<Op><<<grid, 32, 0, stream>>>(a);
         count_launch();
     }
     if (cudaLaunchKernelEx(&cfg, staged_kernel<Op>, a) != cudaSuccess) return FP8ATTN_ERR_CUDA;
