@@ -274,6 +274,14 @@ int fp8attn_gate_use_fp8(int64_t n_train);
  * keys). */
 int fp8attn_attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d, uint32_t flags);
 
+/* Informational, host only (the paper has no counterpart): how a quantization of these sizes runs
+ * on the current device, without one on a B200 (148 SMs).  tensors = 3: fp8attn_quantize_qkv(_ex)
+ * with these flags; tensors = 1: fp8attn_quantize(_ex) of n_train rows without scale_in.
+ *   n > 0   one pass, the heads held on chip, in n stages of as many heads as fit
+ *   0       two passes (also for sizes and flags that the call itself refuses)
+ * Codes and scales do not depend on it. */
+int fp8attn_quantize_stages(int tensors, int B, int H, int64_t n_train, int64_t n_test, int d, uint32_t flags);
+
 /* Seeded Gaussian perturbation of Q, K or V (paper appendix, Eq. 3: the noise
  * experiment that replaces quantization by an explicit perturbation):
  *

@@ -27,7 +27,7 @@ EXPORTS = (
     "fp8attn_selftest_wait_timeout", "fp8attn_quantize_ex",
     "fp8attn_icl_step_host", "fp8attn_host_step_scratch_bytes", "fp8attn_host_step_chunks",
     "fp8attn_host_step_status", "fp8attn_attention_rows_per_cta",
-    "fp8attn_quantize_qkv_ordered", "fp8attn_reorder_rows",
+    "fp8attn_quantize_qkv_ordered", "fp8attn_reorder_rows", "fp8attn_quantize_stages",
 )
 # flags of fp8attn_quantize_ex / fp8attn_quantize_qkv_ex
 QUERY_SCALE_FROM_ALL_ROWS = 1
@@ -113,6 +113,8 @@ def load() -> ctypes.CDLL:
     lib.fp8attn_launch_count.argtypes = []
     lib.fp8attn_attention_rows_per_cta.restype = i32
     lib.fp8attn_attention_rows_per_cta.argtypes = [i32, i32, i64, i64, i32, u32]
+    lib.fp8attn_quantize_stages.restype = i32
+    lib.fp8attn_quantize_stages.argtypes = [i32, i32, i32, i64, i64, i32, u32]
     lib.fp8attn_host_step_scratch_bytes.restype = sz
     lib.fp8attn_host_step_scratch_bytes.argtypes = [i32, i32, i64, i64, i32, u32]
     lib.fp8attn_host_step_chunks.restype = i32
@@ -283,6 +285,12 @@ def selftest_wait_timeout(workspace: torch.Tensor, limit_us: int = 1000) -> None
 def attention_rows_per_cta(B: int, H: int, n_train: int, n_test: int, d: int, flags: int = 0) -> int:
     """fp8attn_attention_rows_per_cta: 256 or 384 query rows per CTA for a call of these sizes."""
     return int(load().fp8attn_attention_rows_per_cta(B, H, n_train, n_test, d, int(flags)))
+
+
+def quantize_stages(tensors: int, B: int, H: int, n_train: int, n_test: int, d: int, flags: int = 0) -> int:
+    """fp8attn_quantize_stages: stages of the one-pass form that a quantization of these sizes takes
+    (tensors = 3: quantize_qkv, 1: quantize), 0 = two passes."""
+    return int(load().fp8attn_quantize_stages(tensors, B, H, n_train, n_test, d, int(flags)))
 
 
 def gate_use_fp8(n_train: int) -> bool:

@@ -35,6 +35,15 @@ int check_workspace(const void* ws, size_t bytes, int B, int H) {
     return FP8ATTN_OK;
 }
 
+// SMs of the current device; without one to ask (a host without a GPU) those of a B200
+int sms_or_b200() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
+        return 148;
+    return sms;
+}
+
 // The kernels are built for sm_100a only.
 int check_device() {
     int dev = 0, major = 0;
@@ -278,12 +287,15 @@ int fp8attn_gate_use_fp8(int64_t n_train) { return n_train > FP8ATTN_GATE_TRAIN_
 
 int fp8attn_attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d, uint32_t flags) {
     if (B <= 0 || H <= 0 || n_train < 0 || n_test < 0 || (d != 64 && d != 128)) return 0;
-    // without a device to ask (a host without a GPU): the SM count of a B200
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
-        sms = 148;
-    return fp8attn::attention_rows_per_cta(B, H, n_train, n_test, d, flags, sms);
+    return fp8attn::attention_rows_per_cta(B, H, n_train, n_test, d, flags, sms_or_b200());
+}
+
+int fp8attn_quantize_stages(int tensors, int B, int H, int64_t n_train, int64_t n_test, int d, uint32_t flags) {
+    if (B <= 0 || H <= 0 || (int64_t)B * H > 65535 || n_train < 0 || n_test < 0 || (d != 64 && d != 128) ||
+        (tensors != 1 && tensors != 3))
+        return 0;
+    return fp8attn::quantize_stages(tensors, (int64_t)B * H, n_train * d, tensors == 3 ? n_test * d : 0, flags,
+                                    sms_or_b200());
 }
 
 size_t fp8attn_workspace_bytes(int B, int H, int64_t n_train, int64_t, int d) {

@@ -61,6 +61,9 @@ int launch_quantize_qkv(const void* q_train, const void* k, const void* v, const
                         uint32_t* counters, uint32_t* words, cudaStream_t stream,
                         int32_t* key_dest = nullptr, int d = 64);
 
+// Stages of the one-pass form that a quantization of these sizes takes (tensors: 1 or 3), 0: two passes.
+int quantize_stages(int tensors, int64_t n_heads, int64_t elems_train, int64_t elems_test, uint32_t flags, int sms);
+
 // key_order.cu
 // dest[b,h,r] = the row that key r of head (b,h) moves to: the keys of largest norm first.
 // norm_scratch: device memory for one fp32 per key (its squared norm), the heads

@@ -188,7 +188,7 @@ struct QuantizeOp {
     struct Static {};
     using Result = Divisor;
     static constexpr int kOutBytes = 8;     // per 16-byte input vector
-    static constexpr int kSlotWords = 1;    // a published value: tag << 16 | maximum
+    // a published value is one word: tag << 16 | maximum
 
     // thread `tid`'s part of `vecs` vectors
     static __device__ __forceinline__ Acc reduce(const uint4* x, int vecs, int tid) {
@@ -238,34 +238,46 @@ struct QuantizeOp {
 // (which also starts on the data); smaller ones rely on what the last call left.
 constexpr int64_t kOneLaunchMaxBytes = 48ll << 20;
 
-// The one-pass kernel for tensors [0, tensors) of `b` and, if there is one, tensor 3 with the scale of
-// tensor 0.  *taken: whether it takes the call.  amax_bits: the accumulators of the two-pass form, free here.
+// How a quantization runs: in one pass (grid > 0) or in two.
+struct Form {
+    unsigned grid;
+    staged::Shape shape;
+};
+Form quantize_form(int tensors, int64_t n_heads, int64_t elems_train, int64_t elems_test, uint32_t flags, int sms) {
+    Form f = {};
+    if ((flags & (FP8ATTN_SCALES_GIVEN | FP8ATTN_QKV_TWO_LAUNCHES)) || elems_train <= 0) return f;
+    const int64_t follow = elems_test / 8;
+    if (follow > 0x7fffffffll) return f;
+    staged::Shape& a = f.shape;
+    a.tensors = tensors;
+    a.units = (int)(tensors * n_heads);
+    a.vecs = elems_train / 8;
+    a.follow_vecs = (uint32_t)follow;
+    a.follow_counts = follow > 0 && (flags & FP8ATTN_QUERY_SCALE_FROM_ALL_ROWS);
+    a.cleared = (a.vecs * a.units + follow * n_heads) * 16 > kOneLaunchMaxBytes;
+    f.grid = staged::plan(a, sms);
+    return f;
+}
+
+// The one-pass kernel for the tensors of `b`: tensors [0, tensors) and, if there are test rows, tensor 3
+// with the scale of tensor 0.  amax_bits: the accumulators of the two-pass form, free here.
 template <bool kHalf>
-int launch_staged(const QuantBatch& b, int tensors, int64_t n_heads, uint32_t* status, uint32_t* counters,
-                  uint32_t* words, uint32_t* amax_bits, int sms, bool* taken, cudaStream_t stream) {
-    using Op = QuantizeOp<kHalf>;
-    staged::Args<Op> a = {};
-    for (int z = 0; z < tensors; ++z) {
+int launch_staged(const Form& f, const QuantBatch& b, uint32_t* status, uint32_t* counters, uint32_t* words,
+                  uint32_t* amax_bits, cudaStream_t stream) {
+    staged::Args<QuantizeOp<kHalf>> a = {};
+    static_cast<staged::Shape&>(a) = f.shape;
+    for (int z = 0; z < a.tensors; ++z) {
         a.x[z] = b.x[z];
         a.out[z] = b.out[z];
         a.result_out[z] = b.scale_out[z];
     }
-    a.tensors = tensors;
-    a.units = (int)(tensors * n_heads);
-    a.vecs = b.pairs_per_head[0] * 2;
-    const int64_t follow = b.pairs_per_head[3] * 2;
     a.follow_x = b.x[3];
     a.follow_out = b.out[3];
-    a.follow_vecs = (uint32_t)follow;
-    a.follow_counts = b.amax_acc[3] != nullptr;
     a.status = status;
     a.counter = counters;
-    *taken = false;
-    const bool clear = (a.vecs * a.units + follow * n_heads) * 16 > kOneLaunchMaxBytes;
-    const unsigned grid = follow > 0x7fffffffll ? 0u : staged::plan(a, sms, words, clear ? amax_bits : nullptr);
-    if (grid == 0) return FP8ATTN_OK;
-    *taken = true;
-    return staged::launch(a, grid, clear, stream);
+    a.slots = words;
+    a.heads = a.cleared ? amax_bits : words + a.sets * a.slots_per_set;
+    return staged::launch(a, f.grid, stream);
 }
 
 }  // namespace
@@ -306,11 +318,11 @@ int launch_quantize_qkv(const void* q_train, const void* k, const void* v, const
     const int sms = sm_count();
     if (sms <= 0) return FP8ATTN_ERR_CUDA;
     const bool half = (flags & FP8ATTN_INPUT_FP16) != 0;
-    if (!(flags & (FP8ATTN_SCALES_GIVEN | FP8ATTN_QKV_TWO_LAUNCHES)) && key_dest == nullptr && elems_train > 0) {
-        bool taken = false;
-        const int rc = half ? launch_staged<true>(b, 3, n_heads, status, counters, words, amax_bits, sms, &taken, stream)
-                            : launch_staged<false>(b, 3, n_heads, status, counters, words, amax_bits, sms, &taken, stream);
-        if (rc != FP8ATTN_OK || taken) return rc;
+    if (key_dest == nullptr) {
+        const Form f = quantize_form(3, n_heads, elems_train, elems_test, flags, sms);
+        if (f.grid > 0)
+            return half ? launch_staged<true>(f, b, status, counters, words, amax_bits, stream)
+                        : launch_staged<false>(f, b, status, counters, words, amax_bits, stream);
     }
     const int64_t want = ((int64_t)sms * 16 + n_heads * 3 - 1) / (n_heads * 3);
     const int64_t have = (elems_train / 16 + kThreads - 1) / kThreads;
@@ -363,16 +375,16 @@ int launch_quantize(const void* x_bf16, int64_t n_heads, int64_t elems_per_head,
         int64_t b = want < have ? want : have;
         return (unsigned)(b < 1 ? 1 : b);
     };
-    if (scale_in == nullptr && elems_per_head > 0 && status != nullptr) {
-        QuantBatch b = {};
-        b.x[0] = static_cast<const uint4*>(x_bf16);
-        b.out[0] = static_cast<uint4*>(x_fp8);
-        b.pairs_per_head[0] = pairs;
-        b.scale_out[0] = scale_out;
-        bool taken = false;
-        const int rc = half ? launch_staged<true>(b, 1, n_heads, status, counters, words, amax_bits, sms, &taken, stream)
-                            : launch_staged<false>(b, 1, n_heads, status, counters, words, amax_bits, sms, &taken, stream);
-        if (rc != FP8ATTN_OK || taken) return rc;
+    if (scale_in == nullptr && status != nullptr) {
+        const Form f = quantize_form(1, n_heads, elems_per_head, 0, flags, sms);
+        if (f.grid > 0) {
+            QuantBatch b = {};
+            b.x[0] = static_cast<const uint4*>(x_bf16);
+            b.out[0] = static_cast<uint4*>(x_fp8);
+            b.scale_out[0] = scale_out;
+            return half ? launch_staged<true>(f, b, status, counters, words, amax_bits, stream)
+                        : launch_staged<false>(f, b, status, counters, words, amax_bits, stream);
+        }
     }
     if (scale_in == nullptr) {
         if (cudaMemsetAsync(amax_bits, 0, sizeof(uint32_t) * n_heads, stream) != cudaSuccess)
@@ -396,6 +408,11 @@ int launch_quantize(const void* x_bf16, int64_t n_heads, int64_t elems_per_head,
         count_launch();
     }
     return cudaGetLastError() == cudaSuccess ? FP8ATTN_OK : FP8ATTN_ERR_CUDA;
+}
+
+int quantize_stages(int tensors, int64_t n_heads, int64_t elems_train, int64_t elems_test, uint32_t flags, int sms) {
+    const Form f = quantize_form(tensors, n_heads, elems_train, elems_test, flags, sms);
+    return f.grid > 0 ? f.shape.stages : 0;
 }
 
 }  // namespace fp8attn

@@ -46,27 +46,32 @@ constexpr size_t kSmemBytes = (size_t)2 * kBufVecs * 16;
 constexpr int kMaxSegments = 48;               // per share
 constexpr int64_t kWaitClocks = 4000000000ll;  // 2 s
 
+// The sizes of a call and how it is cut (host arithmetic only, see plan()).
+struct Shape {
+    int tensors, units;         // tensors that are reduced; their heads
+    int64_t vecs;               // 16-byte vectors per unit
+    uint32_t follow_vecs;       // per head, of a tensor that takes the results of tensor 0 as they are ...
+    int follow_counts;          // ... after entering its reduction
+    bool cleared;               // a launch before clears the published words
+    int stage_units;            // per stage (the last one may have fewer)
+    int stages;
+    // Published values: `sets` sets of slots_per_set.  Alternate stages use alternate sets: a block is in
+    // stage s + 2 only after every block that it shares a unit with has collected stage s.  A shorter
+    // last stage pairs other blocks with one another and has a set of its own.
+    uint32_t slots_per_set;
+    int sets, last_set;
+};
+
 template <class Op>
-struct Args {
+struct Args : Shape {
     const uint4* x[3];          // the tensors that are reduced: unit u is head u / tensors of tensor u % tensors
     void* out[3];
     float* result_out[3];       // per head (NULL: none)
-    int tensors, units;
-    int64_t vecs;               // 16-byte vectors per unit
-    int stage_units;            // per stage (the last one may have fewer)
-    // a tensor that takes the results of tensor 0 as they are (values may lie outside their range) ...
-    const uint4* follow_x;
+    const uint4* follow_x;      // values may lie outside the range of tensor 0
     void* follow_out;
-    uint32_t follow_vecs;       // per head
-    int follow_counts;          // ... after entering its reduction
     uint32_t* status;
     uint32_t* counter;          // blocks done
-    uint32_t* slots;            // published values, `sets` sets of slots_per_set
-    uint32_t slots_per_set;
-    // Alternate stages use alternate sets: a block is in stage s + 2 only after every block that it
-    // shares a unit with has collected stage s.  A shorter last stage pairs other blocks with one
-    // another and has a set of its own.
-    int sets, last_set;
+    uint32_t* slots;            // published values
     uint32_t* heads;            // published results of tensor 0, for the rows that follow it
     typename Op::Static op;
 };
@@ -146,9 +151,9 @@ __global__ void clear_and_fetch_kernel(const __grid_constant__ Args<Op> a) {
         for (uint32_t part = 0; part < kParts; ++part)
             half_share(a, s, 0, part, [](uint32_t, const uint4* src, uint32_t n) { bulk_prefetch(src, n * 16); });
     const uint32_t t = blockIdx.x * 32 + threadIdx.x, threads = gridDim.x * 32;
-    for (uint32_t i = t; i < a.sets * a.slots_per_set * Op::kSlotWords; i += threads) a.slots[i] = 0u;
+    for (uint32_t i = t; i < a.sets * a.slots_per_set ; i += threads) a.slots[i] = 0u;
     if (a.follow_vecs > 0)
-        for (uint32_t i = t; i < (uint32_t)(a.units / a.tensors) * Op::kSlotWords; i += threads) a.heads[i] = 0u;
+        for (uint32_t i = t; i < (uint32_t)(a.units / a.tensors) ; i += threads) a.heads[i] = 0u;
 }
 
 template <class Op>
@@ -162,7 +167,7 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
     __shared__ int last;
     static_assert(kSmemBytes + sizeof(segment) + sizeof(seg_acc) + 768 <= 232448, "shared memory of a block");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int stages = (a.units + a.stage_units - 1) / a.stage_units;
+    const int stages = a.stages;
     const uint32_t vecs = (uint32_t)a.vecs, tensors = (uint32_t)a.tensors;
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -246,7 +251,7 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
             const Share& s = stage + 1 < stages ? share_full : share_last;
             const uint32_t u0 = (uint32_t)(stage * a.stage_units) + s.unit;
             uint32_t* const slots =
-                a.slots + (stage + 1 == stages ? a.last_set : stage & 1) * a.slots_per_set * Op::kSlotWords;
+                a.slots + (stage + 1 == stages ? a.last_set : stage & 1) * a.slots_per_set ;
             const uint32_t tag = (uint32_t)stage + 1;
             if (stage == 0 || (stage + 1 == stages && share_last.total != share_full.total)) {
                 for (uint32_t g = lane; g < s.segs; g += 32) {
@@ -413,20 +418,17 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
     if (tid == 0) last = atomicAdd(a.counter, 1u) == gridDim.x - 1;
     __syncthreads();
     if (last) {
-        for (uint32_t i = tid; i < a.sets * a.slots_per_set * Op::kSlotWords; i += kThreads) a.slots[i] = 0u;
+        for (uint32_t i = tid; i < a.sets * a.slots_per_set ; i += kThreads) a.slots[i] = 0u;
         if (a.follow_vecs > 0)
-            for (int i = tid; i < a.units / a.tensors * Op::kSlotWords; i += kThreads) a.heads[i] = 0u;
+            for (int i = tid; i < a.units / a.tensors ; i += kThreads) a.heads[i] = 0u;
         if (tid == 0) *a.counter = 0u;
     }
 }
 
-// Fills stage_units and the published words' places and returns the grid, or 0 where this path does not
-// take the call: a unit that does not fit one buffer of every SM, heads so short that a share would
-// have too many segments, or too little room.  `words`: the workspace's kOnePassWords, which are zero
-// between calls; `cleared_heads`: one word per head that the call clears first (NULL: it clears
-// nothing, all its words are among `words`).
-template <class Op>
-unsigned plan(Args<Op>& a, int sms, uint32_t* words, uint32_t* cleared_heads) {
+// Fills what plan() does not get (stage_units and everything behind it) and returns the grid, or 0 where
+// this path does not take the call: a unit that does not fit one buffer of every SM, heads so short that
+// a share would have too many segments, or more words than the workspace has for them.
+inline unsigned plan(Shape& a, int sms) {
     if (a.units <= 0 || a.vecs <= 0 || a.vecs % 8 != 0) return 0;     // (shares end on multiples of eight vectors)
     if ((uint64_t)a.follow_vecs * (uint64_t)(a.units / a.tensors) > 0x7fffffffull) return 0;
     // at least 8 KB per block: with fewer blocks there is less to exchange (2 heads of 512 + 128 rows x 64:
@@ -443,20 +445,20 @@ unsigned plan(Args<Op>& a, int sms, uint32_t* words, uint32_t* cleared_heads) {
     stages = (a.units + a.stage_units - 1) / a.stage_units;
     const int64_t share = (a.stage_units * a.vecs + grid - 1) / grid + 7;
     if (share / a.vecs + 2 > kMaxSegments || stages > 0xfff0) return 0;
+    a.stages = (int)stages;
     const bool shorter = stages > 2 && stages * a.stage_units != a.units;
     a.sets = shorter ? 3 : stages > 1 ? 2 : 1;
     a.last_set = shorter ? 2 : (int)(stages - 1) & 1;
-    const int64_t per_set = grid + a.stage_units, used = a.sets * per_set * Op::kSlotWords;
-    a.slots = words;
+    const int64_t per_set = grid + a.stage_units;
+    // the words of the heads sit behind the slots, or where the call clears them first
+    const int64_t head_words = !a.cleared && a.follow_vecs > 0 ? a.units / a.tensors : 0;
+    if (a.sets * per_set + head_words > kOnePassWords) return 0;
     a.slots_per_set = (uint32_t)per_set;
-    a.heads = cleared_heads != nullptr ? cleared_heads : words + used;
-    const int64_t head_words = cleared_heads == nullptr && a.follow_vecs > 0 ? a.units / a.tensors * Op::kSlotWords : 0;
-    if (used + head_words > kOnePassWords) return 0;
     return (unsigned)grid;
 }
 
 template <class Op>
-int launch(const Args<Op>& a, unsigned grid, bool clear, cudaStream_t stream) {
+int launch(const Args<Op>& a, unsigned grid, cudaStream_t stream) {
     // (the opt-in to large dynamic shared memory is per device and context: set on every call)
     if (cudaFuncSetAttribute(staged_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) !=
         cudaSuccess)
@@ -471,7 +473,7 @@ int launch(const Args<Op>& a, unsigned grid, bool clear, cudaStream_t stream) {
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    if (clear) {
+    if (a.cleared) {
         clear_and_fetch_kernel<Op><<<grid, 32, 0, stream>>>(a);
         count_launch();
     }

@@ -138,20 +138,23 @@ def test_fused_qkv_quantize_matches_oracle(cfg, n, m):
 
 
 def test_fused_qkv_large_call_takes_two_launches():
-    """Above the one-launch size (48 MB of 16-bit input) the call is a maximum pass and a
-    conversion pass; bit-identical to the oracle all the same."""
+    """Above the one-launch size (48 MB of 16-bit input) the call takes two launches: one that starts on
+    the data and the one-pass kernel, or on request the maximum and the conversion; bit-identical to the
+    oracle either way."""
     w = W.CONFIGS["C3"].scaled(20000, 3000)      # 8 heads x 128 x (3 x 20000 + 3000) x 2 B = 129 MB
     g = W.generate(w)
     ws = api.new_workspace(w.B, w.H)
-    before = api.launch_count()
-    o = api.quantize_qkv(to_dev(g["q_train"]), to_dev(g["k"]), to_dev(g["v"]), to_dev(g["q_test"]), ws)
-    assert api.launch_count() - before == 2
     rq, rsq = oracle.quantize(g["q_train"])
     rt, _ = oracle.quantize(g["q_test"], scale_in=rsq)
     rv, rsv = oracle.quantize(g["v"])
-    assert np.array_equal(o["q8"].cpu().numpy(), rq) and np.array_equal(o["t8"].cpu().numpy(), rt)
-    assert np.array_equal(o["v8"].cpu().numpy(), rv) and np.array_equal(o["sv"].cpu().numpy(), rsv)
-    assert api.last_device_status(ws) == (0, 0)
+    for flags in (0, api.QKV_TWO_LAUNCHES):
+        assert (api.quantize_stages(3, w.B, w.H, 20000, 3000, w.d, flags) > 0) == (flags == 0)
+        before = api.launch_count()
+        o = api.quantize_qkv(to_dev(g["q_train"]), to_dev(g["k"]), to_dev(g["v"]), to_dev(g["q_test"]), ws, flags=flags)
+        assert api.launch_count() - before == 2
+        assert np.array_equal(o["q8"].cpu().numpy(), rq) and np.array_equal(o["t8"].cpu().numpy(), rt)
+        assert np.array_equal(o["v8"].cpu().numpy(), rv) and np.array_equal(o["sv"].cpu().numpy(), rsv)
+        assert api.last_device_status(ws) == (0, 0)
 
 
 @pytest.mark.parametrize("extra", [0, api.QKV_TWO_LAUNCHES])

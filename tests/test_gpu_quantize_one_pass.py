@@ -3,9 +3,11 @@ two-launch form, which the other tests hold against the oracle: same codes and s
 Shapes at its edges: one stage and several, a shorter last stage, shares of one segment and of many,
 heads just below and above what fits, test rows that outnumber the train rows, every call twice on
 one workspace (it has to leave its words clean)."""
+import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2609_13031_b200 import api
 
 pytestmark = pytest.mark.gpu
@@ -17,23 +19,25 @@ def tensors(B, H, rows, d, dtype, seed):
     return [torch.empty((B, H, r, d), dtype=dtype, device="cuda").normal_(generator=g) if r else None for r in rows]
 
 
-@pytest.mark.parametrize("B,H,n,m,d,dtype,flags", [
-    (1, 1, 1, 0, 64, "bf16", 0),
-    (1, 3, 1, 5, 128, "fp16", 0),
-    (1, 2, 257, 31, 64, "bf16", 0),
-    (2, 5, 1000, 77, 128, "fp16", api.QUERY_SCALE_FROM_ALL_ROWS),
-    (4, 16, 63, 9, 64, "bf16", 0),                   # many segments per share
-    (1, 7, 9001, 300, 128, "bf16", 0),               # 21 units in two stages: a shorter last one
-    (1, 11, 12289, 64, 128, "bf16", api.QUERY_SCALE_FROM_ALL_ROWS),
-    (1, 7, 20011, 3001, 128, "bf16", 0),             # 21 units, three at a time
-    (1, 4, 30001, 0, 128, "fp16", 0),                # 12 units, two at a time
-    (1, 2, 65536, 1, 128, "bf16", 0),                # the largest head that fits
-    (1, 1, 65600, 100, 128, "bf16", 0),              # the first that does not
-    (1, 3, 300, 40000, 64, "bf16", 0),               # test rows outnumber the train rows
-    (1, 2, 500, 3000, 64, "bf16", api.QUERY_SCALE_FROM_ALL_ROWS),
-    (3, 100, 16, 4, 64, "bf16", 0),
+@pytest.mark.parametrize("B,H,n,m,d,dtype,flags,stages", [
+    (1, 1, 1, 0, 64, "bf16", 0, 1),
+    (1, 3, 1, 5, 128, "fp16", 0, 1),
+    (1, 2, 257, 31, 64, "bf16", 0, 1),
+    (2, 5, 1000, 77, 128, "fp16", api.QUERY_SCALE_FROM_ALL_ROWS, 1),
+    (4, 16, 63, 9, 64, "bf16", 0, 1),                   # many segments per share
+    (1, 7, 9001, 300, 128, "bf16", 0, 3),               # 21 units, seven at a time
+    (1, 11, 12289, 64, 128, "bf16", api.QUERY_SCALE_FROM_ALL_ROWS, 7),    # 33 units, five at a time, then three
+    (1, 7, 20011, 3001, 128, "bf16", 0, 7),             # 21 units, three at a time
+    (1, 4, 30001, 0, 128, "fp16", 0, 6),                # 12 units, two at a time
+    (1, 2, 65536, 1, 128, "bf16", 0, 6),                # the largest head that fits
+    (1, 1, 65600, 100, 128, "bf16", 0, 0),              # the first that does not
+    (1, 3, 300, 40000, 64, "bf16", 0, 1),               # test rows outnumber the train rows
+    (1, 2, 500, 3000, 64, "bf16", api.QUERY_SCALE_FROM_ALL_ROWS, 1),
+    (3, 100, 16, 4, 64, "bf16", 0, 0),                  # heads too short for the shares' segments
 ])
-def test_one_pass_matches_two_launches(B, H, n, m, d, dtype, flags):
+def test_one_pass_matches_two_launches(B, H, n, m, d, dtype, flags, stages):
+    assert api.quantize_stages(3, B, H, n, m, d, flags) == stages
+    assert api.quantize_stages(3, B, H, n, m, d, flags | api.QKV_TWO_LAUNCHES) == 0
     tdt = torch.bfloat16 if dtype == "bf16" else torch.float16
     ws = api.new_workspace(B, H)
     for seed in (1, 2):
@@ -44,9 +48,25 @@ def test_one_pass_matches_two_launches(B, H, n, m, d, dtype, flags):
         for name in ("q8", "k8", "v8", "t8", "sq", "sk", "sv"):
             assert torch.equal(got[name], want[name]), name
             assert torch.equal(again[name], want[name]), name
+        assert (api.quantize_stages(1, B, H, n, 0, d) > 0) == (n <= 65536)
         code, scale = api.quantize(x[1], ws)
         assert torch.equal(code, want["k8"]) and torch.equal(scale, want["sk"])
     assert api.last_device_status(ws) == (0, 0)
+
+
+@pytest.mark.parametrize("H,n,m,stages", [(7, 9001, 300, 3), (2, 40000, 1000, 6)])
+def test_several_stages_match_oracle(H, n, m, stages):
+    assert api.quantize_stages(3, 1, H, n, m, 128) == stages
+    x = tensors(1, H, (n, n, n, m), 128, torch.bfloat16, 5)
+    ws = api.new_workspace(1, H)
+    o = api.quantize_qkv(*x, ws)
+    bits = [t.view(torch.int16).cpu().numpy().view(np.uint16) for t in x]
+    for i, (code, scale) in enumerate((("q8", "sq"), ("k8", "sk"), ("v8", "sv"))):
+        want, s = oracle.quantize(bits[i])
+        assert np.array_equal(o[code].cpu().numpy(), want) and np.array_equal(o[scale].cpu().numpy(), s)
+        if i == 0:
+            want_t, _ = oracle.quantize(bits[3], scale_in=s)
+    assert np.array_equal(o["t8"].cpu().numpy(), want_t)
 
 
 def test_workspace_shared_with_other_calls():
