@@ -80,13 +80,16 @@ int fp8attn_quantize_ex(const void* x_16bit, int B, int H, int64_t rows, int d,
  * Eq. 2), and Q_test quantized with the train-query scale (Method section, shared
  * query scale).  It removes most of the launch overhead that makes quantization
  * dominate at small train-row counts (the paper's latency tables below ~8k rows).
- * Heads of up to 16 MB per tensor are held on chip between the maximum and the
- * conversion, so that every element is read once: ONE launch, or two where the
+ * Heads of up to 128 KB per tensor (1,024 rows x 64) are held by one thread block
+ * each between the maximum and the conversion: ONE launch whose blocks do not wait
+ * for one another.  Heads of up to 16 MB per tensor are held by all SMs together,
+ * so that every element is read once as well: ONE launch, or two where the
  * 16-bit inputs total more than 48 MB (a small one first).  Its thread blocks (one
  * per SM) exchange the heads' maxima; they are launched cooperatively, so that all
  * are resident at once, and every wait is bounded (2 s), ending in
  * FP8ATTN_ERR_TIMEOUT in the workspace's status word.  Larger heads take two
- * launches that do not wait (maximum; conversion), as do all calls with
+ * launches that do not wait (maximum; conversion), as do short train heads with more
+ * than 128 KB of test rows that enter their maximum, and all calls with
  * FP8ATTN_QKV_TWO_LAUNCHES (the _ex call), e.g. of callers that share the GPU with
  * long-running kernels of other streams.
  *
@@ -277,7 +280,8 @@ int fp8attn_attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test
 /* Informational, host only (the paper has no counterpart): how a quantization of these sizes runs
  * on the current device, without one on a B200 (148 SMs).  tensors = 3: fp8attn_quantize_qkv(_ex)
  * with these flags; tensors = 1: fp8attn_quantize(_ex) of n_train rows without scale_in.
- *   n > 0   one pass, the heads held on chip, in n stages of as many heads as fit
+ *   n > 0   one pass, the heads held on chip by all SMs together, in n stages of as many heads as fit
+ *   -1      one pass, every head held by one thread block
  *   0       two passes (also for sizes and flags that the call itself refuses)
  * Codes and scales do not depend on it. */
 int fp8attn_quantize_stages(int tensors, int B, int H, int64_t n_train, int64_t n_test, int d, uint32_t flags);

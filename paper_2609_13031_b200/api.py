@@ -289,7 +289,7 @@ def attention_rows_per_cta(B: int, H: int, n_train: int, n_test: int, d: int, fl
 
 def quantize_stages(tensors: int, B: int, H: int, n_train: int, n_test: int, d: int, flags: int = 0) -> int:
     """fp8attn_quantize_stages: stages of the one-pass form that a quantization of these sizes takes
-    (tensors = 3: quantize_qkv, 1: quantize), 0 = two passes."""
+    (tensors = 3: quantize_qkv, 1: quantize), -1 = one block per head, 0 = two passes."""
     return int(load().fp8attn_quantize_stages(tensors, B, H, n_train, n_test, d, int(flags)))
 
 

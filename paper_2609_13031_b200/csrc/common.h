@@ -61,7 +61,8 @@ int launch_quantize_qkv(const void* q_train, const void* k, const void* v, const
                         uint32_t* counters, uint32_t* words, cudaStream_t stream,
                         int32_t* key_dest = nullptr, int d = 64);
 
-// Stages of the one-pass form that a quantization of these sizes takes (tensors: 1 or 3), 0: two passes.
+// The form that a quantization of these sizes takes (tensors: 1 or 3): stages of the staged kernel, -1: a
+// block per head, 0: two passes.
 int quantize_stages(int tensors, int64_t n_heads, int64_t elems_train, int64_t elems_test, uint32_t flags, int sms);
 
 // key_order.cu

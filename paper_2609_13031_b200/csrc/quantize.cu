@@ -1,8 +1,8 @@
 // Per-head absmax quantization of bf16 (or IEEE fp16) tensors to e4m3 (paper Eq. 2).
 //
-// Calls whose heads fit on chip take one pass (staged.cuh, QuantizeOp below): 2 B read + 1 B written
-// per element.  The others (heads of more than 16 MB, an order of the keys, scales given, or on
-// request) take two HBM-bound kernels:
+// Calls whose heads fit on chip take one pass: short heads a block each (quantize_heads_kernel), longer
+// ones all SMs together (staged.cuh, QuantizeOp below): 2 B read + 1 B written per element.  The others
+// (heads of more than 16 MB, an order of the keys, scales given, or on request) take two HBM-bound kernels:
 //   absmax_kernel    max |x| per head, packed bf16x2 max, one atomicMax per block
 //   quantize_kernel  s = amax/448, y = x/s (IEEE fp32), cvt.rn.satfinite.e4m3x2
 // Algorithmic traffic: 2 B read per element for the maximum, 2 B read + 1 B
@@ -238,25 +238,170 @@ struct QuantizeOp {
 // (which also starts on the data); smaller ones rely on what the last call left.
 constexpr int64_t kOneLaunchMaxBytes = 48ll << 20;
 
-// How a quantization runs: in one pass (grid > 0) or in two.
+// Short heads: one block per head holds it in registers between the maximum and the conversion.
+// Nothing is exchanged between blocks.  Test rows are cut into pieces with blocks of their own, each of
+// which takes the maximum of the train queries' head once more (from L2) instead of waiting for it; where
+// there are heads enough to fill the SMs, the block of the train queries converts them.
+// What bounds it: latency in small calls (one way in, one block-wide maximum, one way out); the
+// exchange of the staged kernel took half of such a call.  With many heads HBM.
+// Graph-replayed, staged kernel -> this one: 2 heads of 512 + 128 rows x 64 9.4 -> 3.5 us, 8 heads
+// 11.0 -> 3.7 us, 8 heads of 1,024 + 256 11.1 -> 4.7 us; two passes -> this one (where the staged kernel
+// took longer or did not take the call): 1,024 heads of 64 + 16 rows x 64 18.6 -> 9.3 us, 4,096 heads of
+// 128 + 32 rows x 64 88 -> 64 us.
+constexpr int kHeadPer = 8;                         // vectors per thread, at most
+constexpr int kHeadVecs = 1024 * kHeadPer;          // 131,072 bytes: 1,024 rows x 64, 512 x 128
+
+struct HeadArgs {
+    const uint4* x[4];
+    uint2* out[4];
+    float* scale_out[4];
+    int tensors, n_heads;
+    int vecs;                   // per head of the tensors that are reduced
+    int counts;                 // the test rows enter the maximum of tensor 0
+    int64_t test_vecs;          // per head
+    int pieces;                 // of the test rows of a head; 0: the block of tensor 0 converts them
+    int64_t piece_vecs;
+};
+
+template <bool kHalf>
+__device__ __forceinline__ Divisor block_divisor(typename In16<kHalf>::V2 m, uint32_t* warp_max) {
+    const uint32_t w = *reinterpret_cast<const uint32_t*>(&m);
+    uint32_t top = __reduce_max_sync(0xffffffffu, max(w & 0xffffu, w >> 16));
+    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = top;
+    __syncthreads();
+    top = __reduce_max_sync(0xffffffffu, (threadIdx.x & 31) < blockDim.x / 32 ? warp_max[threadIdx.x & 31] : 0u);
+    return divisor(head_scale(In16<kHalf>::lo(top)));
+}
+// (the per-element division stays out of the unrolled loops: small calls pay for the code they fetch)
+template <bool kHalf>
+__device__ __noinline__ void convert_direct(const uint4* x, uint2* out, int64_t n, Divisor dv) {
+#pragma unroll 1
+    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) out[i] = quant8_direct<kHalf>(ld_nc_v4(x + i), dv);
+}
+// `n` vectors, four loads of a thread under way at a time
+template <bool kHalf>
+__device__ __forceinline__ void convert_rows(const uint4* x, uint2* out, int64_t n, const Divisor& dv) {
+    if (dv.direct) return convert_direct<kHalf>(x, out, n, dv);
+    for (int64_t i = threadIdx.x; i < n; i += 4 * blockDim.x) {
+        uint4 v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i + k * blockDim.x < n) v[k] = ld_nc_v4(x + i + k * blockDim.x);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i + k * blockDim.x < n) out[i + k * blockDim.x] = quant8<kHalf, true>(v[k], dv);
+    }
+}
+
+template <bool kHalf>
+__global__ void __launch_bounds__(1024) quantize_heads_kernel(const __grid_constant__ HeadArgs a) {
+    using T = In16<kHalf>;
+    __shared__ uint32_t warp_max[32];
+    const int tid = threadIdx.x, mains = a.tensors * a.n_heads;
+    typename T::V2 m = T::as2(0u);
+    if ((int)blockIdx.x < mains) {
+        const int head = (int)blockIdx.x / a.tensors, z = (int)blockIdx.x - head * a.tensors;
+        const uint4* x = a.x[z] + (int64_t)head * a.vecs;
+        uint4 v[kHeadPer];
+#pragma unroll
+        for (int k = 0; k < kHeadPer; ++k) {
+            const int i = tid + k * (int)blockDim.x;
+            v[k] = i < a.vecs ? ld_nc_v4(x + i) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int k = 0; k < kHeadPer; ++k) m = absmax8<kHalf>(m, v[k]);
+        const uint4* test_x = a.x[3] + head * a.test_vecs;
+        if (a.counts && z == 0)
+            for (int64_t i = tid; i < a.test_vecs; i += blockDim.x) m = absmax8<kHalf>(m, ld_nc_v4(test_x + i));
+        const Divisor dv = block_divisor<kHalf>(m, warp_max);
+        if (tid == 0) a.scale_out[z][head] = dv.s;
+        uint2* out = a.out[z] + (int64_t)head * a.vecs;
+        if (dv.direct) convert_direct<kHalf>(x, out, a.vecs, dv);
+#pragma unroll
+        for (int k = 0; k < kHeadPer; ++k) {
+            const int i = tid + k * (int)blockDim.x;
+            if (i < a.vecs && !dv.direct) out[i] = quant8<kHalf, false>(v[k], dv);
+        }
+        if (z == 0 && a.pieces == 0) convert_rows<kHalf>(test_x, a.out[3] + head * a.test_vecs, a.test_vecs, dv);
+    } else {
+        const int item = (int)blockIdx.x - mains, head = item / a.pieces;
+        const int64_t first = (int64_t)(item - head * a.pieces) * a.piece_vecs;
+        const uint4* head_x = a.x[0] + (int64_t)head * a.vecs;
+        const uint4* test_x = a.x[3] + head * a.test_vecs;
+#pragma unroll 4
+        for (int i = tid; i < a.vecs; i += blockDim.x) m = absmax8<kHalf>(m, ld_nc_v4(head_x + i));
+        if (a.counts)
+            for (int64_t i = tid; i < a.test_vecs; i += blockDim.x) m = absmax8<kHalf>(m, ld_nc_v4(test_x + i));
+        const Divisor dv = block_divisor<kHalf>(m, warp_max);
+        convert_rows<kHalf>(test_x + first, a.out[3] + head * a.test_vecs + first, min(a.piece_vecs, a.test_vecs - first), dv);
+    }
+}
+
+// How a quantization runs.
 struct Form {
+    enum { kTwoPasses, kHeads, kStaged } kind;
     unsigned grid;
-    staged::Shape shape;
+    staged::Shape shape;        // kStaged
+    HeadArgs heads;             // kHeads: without its pointers
+    unsigned threads;           // kHeads
 };
 Form quantize_form(int tensors, int64_t n_heads, int64_t elems_train, int64_t elems_test, uint32_t flags, int sms) {
     Form f = {};
     if ((flags & (FP8ATTN_SCALES_GIVEN | FP8ATTN_QKV_TWO_LAUNCHES)) || elems_train <= 0) return f;
-    const int64_t follow = elems_test / 8;
+    const int64_t vecs = elems_train / 8, follow = elems_test / 8;
+    const bool counts = follow > 0 && (flags & FP8ATTN_QUERY_SCALE_FROM_ALL_ROWS);
+    if (vecs <= kHeadVecs) {
+        if (counts && follow > kHeadVecs) return f;
+        // Pieces of the test rows: two per SM, but none so small that reading the train queries again is
+        // most of its work.  None where the train heads fill the SMs by themselves.
+        // (16 heads of 300 + 20,000 x 128: 30 us, two passes 37 us; 4,096 heads of 128 + 32 x 64 with a block
+        // for the test rows of every head took 90 us)
+        int64_t piece = (follow * n_heads + 2 * sms - 1) / (2 * sms);
+        if (piece < vecs / 4) piece = vecs / 4;
+        if (piece < 1024) piece = 1024;
+        if (piece > follow) piece = follow;
+        const bool own = follow > 0 && !(tensors * n_heads >= 4 * sms && follow <= vecs);
+        const int64_t pieces = own ? (follow + piece - 1) / piece : 0;
+        if (n_heads * (tensors + pieces) > 0x7fffffffll) return f;
+        f.kind = Form::kHeads;
+        f.grid = (unsigned)(n_heads * (tensors + pieces));
+        HeadArgs& a = f.heads;
+        a.tensors = tensors;
+        a.n_heads = (int)n_heads;
+        a.vecs = (int)vecs;
+        a.counts = counts;
+        a.test_vecs = follow;
+        a.pieces = (int)pieces;
+        a.piece_vecs = piece;
+        // four vectors per thread, more where a block is full
+        const int64_t threads = (vecs + 4 * 32 - 1) / (4 * 32) * 32, least = pieces > 0 ? 256 : 64;
+        f.threads = (unsigned)(threads < least ? least : threads > 1024 ? 1024 : threads);
+        return f;
+    }
     if (follow > 0x7fffffffll) return f;
     staged::Shape& a = f.shape;
     a.tensors = tensors;
     a.units = (int)(tensors * n_heads);
-    a.vecs = elems_train / 8;
+    a.vecs = vecs;
     a.follow_vecs = (uint32_t)follow;
-    a.follow_counts = follow > 0 && (flags & FP8ATTN_QUERY_SCALE_FROM_ALL_ROWS);
+    a.follow_counts = counts;
     a.cleared = (a.vecs * a.units + follow * n_heads) * 16 > kOneLaunchMaxBytes;
     f.grid = staged::plan(a, sms);
+    if (f.grid > 0) f.kind = Form::kStaged;
     return f;
+}
+
+template <bool kHalf>
+int launch_heads(const Form& f, const QuantBatch& b, cudaStream_t stream) {
+    HeadArgs a = f.heads;
+    for (int z = 0; z < 4; ++z) {
+        a.x[z] = b.x[z];
+        a.out[z] = reinterpret_cast<uint2*>(b.out[z]);
+        a.scale_out[z] = b.scale_out[z];
+    }
+    quantize_heads_kernel<kHalf><<<f.grid, f.threads, 0, stream>>>(a);
+    count_launch();
+    return cudaGetLastError() == cudaSuccess ? FP8ATTN_OK : FP8ATTN_ERR_CUDA;
 }
 
 // The one-pass kernel for the tensors of `b`: tensors [0, tensors) and, if there are test rows, tensor 3
@@ -320,12 +465,16 @@ int launch_quantize_qkv(const void* q_train, const void* k, const void* v, const
     const bool half = (flags & FP8ATTN_INPUT_FP16) != 0;
     if (key_dest == nullptr) {
         const Form f = quantize_form(3, n_heads, elems_train, elems_test, flags, sms);
-        if (f.grid > 0)
+        if (f.kind == Form::kHeads) return half ? launch_heads<true>(f, b, stream) : launch_heads<false>(f, b, stream);
+        if (f.kind == Form::kStaged)
             return half ? launch_staged<true>(f, b, status, counters, words, amax_bits, stream)
                         : launch_staged<false>(f, b, status, counters, words, amax_bits, stream);
     }
     const int64_t want = ((int64_t)sms * 16 + n_heads * 3 - 1) / (n_heads * 3);
-    const int64_t have = (elems_train / 16 + kThreads - 1) / kThreads;
+    // (blocks for the train rows; more only where the test rows are many times as many: blocks with
+    // nothing to do cost 2 us in calls of 12 us, too few took 4 heads of 64 + 32,768 x 128 350 us, not 20)
+    const int64_t most = elems_test / 4 > elems_train ? elems_test / 4 : elems_train;
+    const int64_t have = (most / 16 + kThreads - 1) / kThreads;
     const unsigned bx = (unsigned)(want < have ? (want < 1 ? 1 : want) : (have < 1 ? 1 : have));
     if (!(flags & FP8ATTN_SCALES_GIVEN) &&
         cudaMemsetAsync(amax_bits, 0, sizeof(uint32_t) * 3 * n_heads, stream) != cudaSuccess)
@@ -377,11 +526,12 @@ int launch_quantize(const void* x_bf16, int64_t n_heads, int64_t elems_per_head,
     };
     if (scale_in == nullptr && status != nullptr) {
         const Form f = quantize_form(1, n_heads, elems_per_head, 0, flags, sms);
-        if (f.grid > 0) {
+        if (f.kind != Form::kTwoPasses) {
             QuantBatch b = {};
             b.x[0] = static_cast<const uint4*>(x_bf16);
             b.out[0] = static_cast<uint4*>(x_fp8);
             b.scale_out[0] = scale_out;
+            if (f.kind == Form::kHeads) return half ? launch_heads<true>(f, b, stream) : launch_heads<false>(f, b, stream);
             return half ? launch_staged<true>(f, b, status, counters, words, amax_bits, stream)
                         : launch_staged<false>(f, b, status, counters, words, amax_bits, stream);
         }
@@ -412,7 +562,7 @@ int launch_quantize(const void* x_bf16, int64_t n_heads, int64_t elems_per_head,
 
 int quantize_stages(int tensors, int64_t n_heads, int64_t elems_train, int64_t elems_test, uint32_t flags, int sms) {
     const Form f = quantize_form(tensors, n_heads, elems_train, elems_test, flags, sms);
-    return f.grid > 0 ? f.shape.stages : 0;
+    return f.kind == Form::kHeads ? -1 : f.kind == Form::kStaged ? f.shape.stages : 0;
 }
 
 }  // namespace fp8attn

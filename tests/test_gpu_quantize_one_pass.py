@@ -1,8 +1,8 @@
-"""The one-pass quantizer (heads held on chip between the maximum and the conversion) against the
-two-launch form, which the other tests hold against the oracle: same codes and scales, bit for bit.
-Shapes at its edges: one stage and several, a shorter last stage, shares of one segment and of many,
-heads just below and above what fits, test rows that outnumber the train rows, every call twice on
-one workspace (it has to leave its words clean)."""
+"""The one-pass forms of the quantizer (heads held on chip between the maximum and the conversion, by
+one block each or by all SMs together) against the two-launch form, which the other tests hold
+against the oracle: same codes and scales, bit for bit.  Shapes at their edges: one stage and several, a
+shorter last stage, heads just below and above what a block and what the chip holds, test rows that
+outnumber the train rows, every call twice on one workspace (it has to leave its words clean)."""
 import numpy as np
 import pytest
 import torch
@@ -20,20 +20,27 @@ def tensors(B, H, rows, d, dtype, seed):
 
 
 @pytest.mark.parametrize("B,H,n,m,d,dtype,flags,stages", [
-    (1, 1, 1, 0, 64, "bf16", 0, 1),
-    (1, 3, 1, 5, 128, "fp16", 0, 1),
-    (1, 2, 257, 31, 64, "bf16", 0, 1),
+    (1, 1, 1, 0, 64, "bf16", 0, -1),
+    (1, 3, 1, 5, 128, "fp16", 0, -1),
+    (1, 2, 257, 31, 64, "bf16", 0, -1),
     (2, 5, 1000, 77, 128, "fp16", api.QUERY_SCALE_FROM_ALL_ROWS, 1),
-    (4, 16, 63, 9, 64, "bf16", 0, 1),                   # many segments per share
+    (4, 16, 63, 9, 64, "bf16", 0, -1),
     (1, 7, 9001, 300, 128, "bf16", 0, 3),               # 21 units, seven at a time
     (1, 11, 12289, 64, 128, "bf16", api.QUERY_SCALE_FROM_ALL_ROWS, 7),    # 33 units, five at a time, then three
     (1, 7, 20011, 3001, 128, "bf16", 0, 7),             # 21 units, three at a time
     (1, 4, 30001, 0, 128, "fp16", 0, 6),                # 12 units, two at a time
     (1, 2, 65536, 1, 128, "bf16", 0, 6),                # the largest head that fits
     (1, 1, 65600, 100, 128, "bf16", 0, 0),              # the first that does not
-    (1, 3, 300, 40000, 64, "bf16", 0, 1),               # test rows outnumber the train rows
-    (1, 2, 500, 3000, 64, "bf16", api.QUERY_SCALE_FROM_ALL_ROWS, 1),
-    (3, 100, 16, 4, 64, "bf16", 0, 0),                  # heads too short for the shares' segments
+    (1, 3, 300, 40000, 64, "bf16", 0, -1),              # test rows outnumber the train rows
+    (3, 100, 16, 4, 64, "bf16", 0, -1),
+    (1, 2, 1024, 130, 64, "fp16", 0, -1),               # the longest head that one block holds
+    (1, 2, 1025, 130, 64, "fp16", 0, 1),                # the first that it does not
+    (1, 1, 1000, 70001, 64, "bf16", 0, -1),             # test rows in pieces, a shorter last one
+    (100, 8, 130, 3, 64, "bf16", 0, -1),                # heads fill the SMs: no pieces
+    (16, 16, 40, 41, 64, "fp16", 0, -1),                # more test rows than train rows: pieces again
+    (2, 3, 512, 512, 128, "bf16", api.QUERY_SCALE_FROM_ALL_ROWS, -1),     # the longest test head that enters the maximum
+    (2, 3, 512, 513, 128, "bf16", api.QUERY_SCALE_FROM_ALL_ROWS, 0),
+    (1, 2, 500, 3000, 64, "bf16", api.QUERY_SCALE_FROM_ALL_ROWS, 0),
 ])
 def test_one_pass_matches_two_launches(B, H, n, m, d, dtype, flags, stages):
     assert api.quantize_stages(3, B, H, n, m, d, flags) == stages
@@ -48,7 +55,7 @@ def test_one_pass_matches_two_launches(B, H, n, m, d, dtype, flags, stages):
         for name in ("q8", "k8", "v8", "t8", "sq", "sk", "sv"):
             assert torch.equal(got[name], want[name]), name
             assert torch.equal(again[name], want[name]), name
-        assert (api.quantize_stages(1, B, H, n, 0, d) > 0) == (n <= 65536)
+        assert (api.quantize_stages(1, B, H, n, 0, d) != 0) == (n <= 65536)
         code, scale = api.quantize(x[1], ws)
         assert torch.equal(code, want["k8"]) and torch.equal(scale, want["sk"])
     assert api.last_device_status(ws) == (0, 0)
