@@ -431,9 +431,10 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
 inline unsigned plan(Shape& a, int sms) {
     if (a.units <= 0 || a.vecs <= 0 || a.vecs % 8 != 0) return 0;     // (shares end on multiples of eight vectors)
     if ((uint64_t)a.follow_vecs * (uint64_t)(a.units / a.tensors) > 0x7fffffffull) return 0;
-    // at least 8 KB per block: with fewer blocks there is less to exchange (2 heads of 512 + 128 rows x 64:
-    // 9.1 us, with 1 KB each 10.3 us)
-    const int64_t all = a.vecs * a.units;
+    // at least 8 KB per block, test rows included: with fewer blocks there is less to exchange, but all of
+    // them share the test rows (1 head of 1,100 + 200,000 x 64 with the blocks that its train rows are worth:
+    // 19.4 us, with all of them 14.7)
+    const int64_t all = a.vecs * a.units + (int64_t)a.follow_vecs * (a.units / a.tensors);
     const int64_t grid = all / 512 < 1 ? 1 : all / 512 > sms ? sms : all / 512;
     const int64_t room = grid * kBufVecs;
     if (a.vecs > room) return 0;

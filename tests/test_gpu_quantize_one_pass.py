@@ -35,6 +35,7 @@ def tensors(B, H, rows, d, dtype, seed):
     (3, 100, 16, 4, 64, "bf16", 0, -1),
     (1, 2, 1024, 130, 64, "fp16", 0, -1),               # the longest head that one block holds
     (1, 2, 1025, 130, 64, "fp16", 0, 1),                # the first that it does not
+    (1, 1, 1100, 60001, 64, "bf16", 0, 1),              # test rows fill the SMs, shares of a few KB
     (1, 1, 1000, 70001, 64, "bf16", 0, -1),             # test rows in pieces, a shorter last one
     (100, 8, 130, 3, 64, "bf16", 0, -1),                # heads fill the SMs: no pieces
     (16, 16, 40, 41, 64, "fp16", 0, -1),                # more test rows than train rows: pieces again
