@@ -337,6 +337,24 @@ __global__ void __launch_bounds__(1024) quantize_heads_kernel(const __grid_const
     }
 }
 
+// Whether a call of more than kOneLaunchMaxBytes, two launches in either form, is faster in one pass.  Every
+// byte crosses the HBM interface once instead of twice, but a stage has a cost of its own, so small calls,
+// and heads that leave much of a stage empty (8.5 MB of the 16.8 MB that the SMs hold: one head per stage),
+// do better in two passes.  Both times in us, fitted to 80 measured sizes (50 .. 900 MB, 1 .. 64 heads, graph-
+// replayed, mean of inputs in L2 and not), within 15 % of each.  One pass / two: 8 heads of 12,289 + 3,000 x 128
+// 42 / 39 us, 4 heads of 33,000 + 5,000 56 / 49 us, 2 heads of 33,200 + 8,300 33 / 28 us, 8 heads of 35,000 +
+// 5,000 100 / 101 us, of 44,000 + 1,000 102 / 120 us, of 65,536 + 16,384 129 / 183 us.  Test rows that enter the
+// maximum of the train queries are read by the blocks that hold those: 8 heads of 20,011 + 3,001 x 128 76 /
+// 58 us, of 65,536 + 16,384 157 / 185 us.
+bool one_pass_pays(const staged::Shape& a) {
+    const double heads = a.units / a.tensors, mb = 16e-6;
+    const double train = mb * (double)a.vecs * a.units, test = mb * (double)a.follow_vecs * heads;
+    double one = 12.4 + 1.74 * a.stages + 0.175 * train;
+    if (a.follow_vecs > 0) one += 5.5 + 0.21 * test;
+    if (a.follow_counts) one += 3.3 * (a.stages < heads ? a.stages : heads);
+    return one < 6.3 + 0.407 * (train + test);
+}
+
 // How a quantization runs.
 struct Form {
     enum { kTwoPasses, kHeads, kStaged } kind;
@@ -387,7 +405,7 @@ Form quantize_form(int tensors, int64_t n_heads, int64_t elems_train, int64_t el
     a.follow_counts = counts;
     a.cleared = (a.vecs * a.units + follow * n_heads) * 16 > kOneLaunchMaxBytes;
     f.grid = staged::plan(a, sms);
-    if (f.grid > 0) f.kind = Form::kStaged;
+    if (f.grid > 0 && (!a.cleared || one_pass_pays(a))) f.kind = Form::kStaged;
     return f;
 }
 

@@ -58,6 +58,22 @@ def test_host_step_plan_is_host_only_arithmetic():
     assert api.host_step_scratch_bytes(1, 8, 0, 16, 64) == 0 and api.host_step_scratch_bytes(1, 8, 64, 16, 96) == 0
 
 
+def test_quantizer_form_is_host_only_arithmetic():
+    """On both sides of each line between a block per head (-1), one pass in stages and two passes."""
+    api.load()
+    both = api.QUERY_SCALE_FROM_ALL_ROWS
+    for tensors, H, n, m, d, flags, stages in (
+            (3, 8, 1024, 256, 64, 0, -1), (3, 8, 1025, 256, 64, 0, 1), (1, 8, 512, 0, 128, 0, -1), (1, 8, 513, 0, 128, 0, 1),
+            (3, 8, 512, 512, 128, both, -1), (3, 8, 512, 513, 128, both, 0),
+            (3, 8, 7500, 2048, 128, 0, 3), (3, 8, 8192, 2048, 128, 0, 0), (3, 2, 33203, 8300, 128, 0, 0), (3, 1, 33203, 8300, 128, 0, 3),
+            (3, 4, 33000, 5000, 128, 0, 0), (3, 8, 44000, 1000, 128, 0, 24), (1, 8, 33203, 0, 128, 0, 0), (1, 8, 32768, 0, 128, 0, 4),
+            (3, 8, 20011, 3001, 128, 0, 8), (3, 8, 20011, 3001, 128, both, 0), (3, 8, 65536, 16384, 128, both, 24),
+            (3, 1, 65536, 0, 128, 0, 3), (3, 1, 65600, 0, 128, 0, 0),
+            (3, 8, 8192, 2048, 128, api.QKV_TWO_LAUNCHES, 0), (3, 8, 8192, 2048, 128, api.SCALES_GIVEN, 0),
+            (2, 8, 512, 0, 64, 0, 0), (3, 8, 512, 0, 96, 0, 0), (3, 0, 512, 0, 64, 0, 0), (3, 8, 0, 0, 64, 0, 0)):
+        assert api.quantize_stages(tensors, 1, H, n, m, d, flags) == stages, (tensors, H, n, m, d, flags)
+
+
 def test_dispatch_gate_matches_the_paper_constant():
     import os
     from helpers import read_golden_table

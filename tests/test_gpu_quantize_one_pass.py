@@ -26,7 +26,10 @@ def tensors(B, H, rows, d, dtype, seed):
     (2, 5, 1000, 77, 128, "fp16", api.QUERY_SCALE_FROM_ALL_ROWS, 1),
     (4, 16, 63, 9, 64, "bf16", 0, -1),
     (1, 7, 9001, 300, 128, "bf16", 0, 3),               # 21 units, seven at a time
-    (1, 11, 12289, 64, 128, "bf16", api.QUERY_SCALE_FROM_ALL_ROWS, 7),    # 33 units, five at a time, then three
+    (1, 11, 12289, 64, 128, "bf16", 0, 7),              # 33 units, five at a time, then three
+    (1, 11, 12289, 64, 128, "bf16", api.QUERY_SCALE_FROM_ALL_ROWS, 0),    # too many heads whose rows enter the maximum
+    (1, 6, 8000, 1333, 128, "fp16", api.QUERY_SCALE_FROM_ALL_ROWS, 3),    # 18 units, six at a time
+    (1, 2, 33203, 77, 128, "bf16", 0, 0),               # 6 units, one at a time, half a stage empty
     (1, 7, 20011, 3001, 128, "bf16", 0, 7),             # 21 units, three at a time
     (1, 4, 30001, 0, 128, "fp16", 0, 6),                # 12 units, two at a time
     (1, 2, 65536, 1, 128, "bf16", 0, 6),                # the largest head that fits
@@ -62,7 +65,7 @@ def test_one_pass_matches_two_launches(B, H, n, m, d, dtype, flags, stages):
     assert api.last_device_status(ws) == (0, 0)
 
 
-@pytest.mark.parametrize("H,n,m,stages", [(7, 9001, 300, 3), (2, 40000, 1000, 6)])
+@pytest.mark.parametrize("H,n,m,stages", [(7, 9001, 300, 3), (2, 65000, 1000, 6)])
 def test_several_stages_match_oracle(H, n, m, stages):
     assert api.quantize_stages(3, 1, H, n, m, 128) == stages
     x = tensors(1, H, (n, n, n, m), 128, torch.bfloat16, 5)
