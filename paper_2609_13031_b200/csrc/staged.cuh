@@ -414,8 +414,11 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
     }
     // ---- the last block to finish leaves everything at zero for the next call ----
     __syncthreads();
-    // (what a block has collected it has read: nothing to fence)
-    if (tid == 0) last = atomicAdd(a.counter, 1u) == gridDim.x - 1;
+    if (tid == 0) {     // every block's stores and polls of the words come before the zeros
+        __threadfence();
+        last = atomicAdd(a.counter, 1u) == gridDim.x - 1;
+        __threadfence();
+    }
     __syncthreads();
     if (last) {
         for (uint32_t i = tid; i < a.sets * a.slots_per_set ; i += kThreads) a.slots[i] = 0u;
