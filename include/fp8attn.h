@@ -413,6 +413,14 @@ int fp8attn_last_device_status(void* workspace, void* cuda_stream, uint32_t* det
 int fp8attn_selftest_wait_timeout(void* workspace, size_t workspace_bytes, uint32_t limit_us,
                                   void* cuda_stream);
 
+/* The same for the waits of the one-pass quantizer: fp8attn_quantize of a bf16 tensor, every
+ * wait of which ends after limit_clocks SM clocks (1..10^8) instead of 2 s.  Waits that run out
+ * are recorded as above; codes and scales are then not valid.  FP8ATTN_ERR_UNSUPPORTED where a
+ * call of these sizes has no waits (fp8attn_quantize_stages(1, ...) <= 0). */
+int fp8attn_selftest_quantize_timeout(const void* x_bf16, int B, int H, int64_t rows, int d, void* x_fp8,
+                                      float* scale_out, uint32_t limit_clocks, void* workspace,
+                                      size_t workspace_bytes, void* cuda_stream);
+
 /* Static, human-readable name of a status code. */
 const char* fp8attn_status_string(int status);
 

@@ -24,7 +24,7 @@ EXPORTS = (
     "fp8attn_launch_count", "fp8attn_quantize_noalloc",
     "fp8attn_icl_forward_ex", "bf16attn_icl_forward_ex", "fp8attn_gate_use_fp8",
     "fp8attn_quantize_qkv", "fp8attn_quantize_qkv_ex", "fp8attn_perturb",
-    "fp8attn_selftest_wait_timeout", "fp8attn_quantize_ex",
+    "fp8attn_selftest_wait_timeout", "fp8attn_selftest_quantize_timeout", "fp8attn_quantize_ex",
     "fp8attn_icl_step_host", "fp8attn_host_step_scratch_bytes", "fp8attn_host_step_chunks",
     "fp8attn_host_step_status", "fp8attn_attention_rows_per_cta",
     "fp8attn_quantize_qkv_ordered", "fp8attn_reorder_rows", "fp8attn_quantize_stages",
@@ -98,6 +98,8 @@ def load() -> ctypes.CDLL:
     lib.fp8attn_perturb.argtypes = [vp, i32, i32, i64, i32, f32, ctypes.c_uint64, u32, vp, vp, vp, sz, vp]
     lib.fp8attn_selftest_wait_timeout.restype = i32
     lib.fp8attn_selftest_wait_timeout.argtypes = [vp, sz, u32, vp]
+    lib.fp8attn_selftest_quantize_timeout.restype = i32
+    lib.fp8attn_selftest_quantize_timeout.argtypes = [vp, i32, i32, i64, i32, vp, vp, u32, vp, sz, vp]
     lib.fp8attn_gate_use_fp8.restype = i32
     lib.fp8attn_gate_use_fp8.argtypes = [i64]
     lib.bf16attn_icl_forward.restype = i32
@@ -280,6 +282,17 @@ def selftest_wait_timeout(workspace: torch.Tensor, limit_us: int = 1000) -> None
     """fp8attn_selftest_wait_timeout: make one bounded device wait expire on purpose."""
     rc = load().fp8attn_selftest_wait_timeout(_ptr(workspace), workspace.numel(), int(limit_us), _stream())
     _check("fp8attn_selftest_wait_timeout", rc)
+
+
+def selftest_quantize_timeout(x: torch.Tensor, workspace: torch.Tensor, out: torch.Tensor, scale_out: torch.Tensor,
+                              limit_clocks: int = 1) -> None:
+    """fp8attn_selftest_quantize_timeout: a one-pass quantization whose waits end after that many clocks."""
+    B, H, rows, d = _dims(x)
+    assert x.dtype == torch.bfloat16 and out.dtype == torch.uint8 and out.shape == x.shape
+    assert scale_out.dtype == torch.float32 and scale_out.numel() == B * H
+    rc = load().fp8attn_selftest_quantize_timeout(_ptr(x), B, H, rows, d, _ptr(out), _ptr(scale_out), int(limit_clocks),
+                                                  _ptr(workspace), workspace.numel(), _stream())
+    _check("fp8attn_selftest_quantize_timeout", rc)
 
 
 def attention_rows_per_cta(B: int, H: int, n_train: int, n_test: int, d: int, flags: int = 0) -> int:

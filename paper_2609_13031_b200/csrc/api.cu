@@ -283,6 +283,28 @@ int fp8attn_selftest_wait_timeout(void* workspace, size_t workspace_bytes_, uint
                                         static_cast<cudaStream_t>(cuda_stream));
 }
 
+int fp8attn_selftest_quantize_timeout(const void* x_bf16, int B, int H, int64_t rows, int d, void* x_fp8,
+                                      float* scale_out, uint32_t limit_clocks, void* workspace,
+                                      size_t workspace_bytes_, void* cuda_stream) {
+    int rc = check_shape(B, H, d);
+    if (rc != FP8ATTN_OK) return rc;
+    if ((int64_t)B * H > 65535) return FP8ATTN_ERR_UNSUPPORTED;
+    if (limit_clocks == 0 || limit_clocks > 100000000u || rows < 1 || !x_bf16 || !x_fp8 || !scale_out)
+        return FP8ATTN_ERR_INVALID_ARG;
+    if (!aligned(x_bf16, 16) || !aligned(x_fp8, 16) || !aligned(scale_out, 4)) return FP8ATTN_ERR_INVALID_ARG;
+    rc = check_workspace(workspace, workspace_bytes_, B, H);
+    if (rc != FP8ATTN_OK) return rc;
+    rc = check_device();
+    if (rc != FP8ATTN_OK) return rc;
+    char* ws = static_cast<char*>(workspace);
+    return launch_quantize_timeout_selftest(x_bf16, (int64_t)B * H, rows * (int64_t)d, x_fp8, scale_out,
+                                            reinterpret_cast<uint32_t*>(ws + kWsAmaxOffset),
+                                            reinterpret_cast<uint32_t*>(ws + kWsStatusOffset),
+                                            reinterpret_cast<uint32_t*>(ws + kWsCounterOffset),
+                                            reinterpret_cast<uint32_t*>(ws + kWsWordsOffset), (int64_t)limit_clocks,
+                                            static_cast<cudaStream_t>(cuda_stream));
+}
+
 int fp8attn_gate_use_fp8(int64_t n_train) { return n_train > FP8ATTN_GATE_TRAIN_ROWS ? 1 : 0; }
 
 int fp8attn_attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d, uint32_t flags) {

@@ -65,6 +65,11 @@ int launch_quantize_qkv(const void* q_train, const void* k, const void* v, const
 // block per head, 0: two passes.
 int quantize_stages(int tensors, int64_t n_heads, int64_t elems_train, int64_t elems_test, uint32_t flags, int sms);
 
+// launch_quantize of a bf16 tensor by the staged kernel, every wait of which ends after that many clocks
+int launch_quantize_timeout_selftest(const void* x_bf16, int64_t n_heads, int64_t elems_per_head, void* x_fp8,
+                                     float* scale_out, uint32_t* amax_bits, uint32_t* status, uint32_t* counters,
+                                     uint32_t* words, int64_t wait_clocks, cudaStream_t stream);
+
 // key_order.cu
 // dest[b,h,r] = the row that key r of head (b,h) moves to: the keys of largest norm first.
 // norm_scratch: device memory for one fp32 per key (its squared norm), the heads

@@ -426,7 +426,7 @@ int launch_heads(const Form& f, const QuantBatch& b, cudaStream_t stream) {
 // with the scale of tensor 0.  amax_bits: the accumulators of the two-pass form, free here.
 template <bool kHalf>
 int launch_staged(const Form& f, const QuantBatch& b, uint32_t* status, uint32_t* counters, uint32_t* words,
-                  uint32_t* amax_bits, cudaStream_t stream) {
+                  uint32_t* amax_bits, cudaStream_t stream, int64_t wait_clocks = staged::kWaitClocks) {
     staged::Args<QuantizeOp<kHalf>> a = {};
     static_cast<staged::Shape&>(a) = f.shape;
     for (int z = 0; z < a.tensors; ++z) {
@@ -436,6 +436,7 @@ int launch_staged(const Form& f, const QuantBatch& b, uint32_t* status, uint32_t
     }
     a.follow_x = b.x[3];
     a.follow_out = b.out[3];
+    a.wait_clocks = wait_clocks;
     a.status = status;
     a.counter = counters;
     a.slots = words;
@@ -576,6 +577,20 @@ int launch_quantize(const void* x_bf16, int64_t n_heads, int64_t elems_per_head,
         count_launch();
     }
     return cudaGetLastError() == cudaSuccess ? FP8ATTN_OK : FP8ATTN_ERR_CUDA;
+}
+
+int launch_quantize_timeout_selftest(const void* x_bf16, int64_t n_heads, int64_t elems_per_head, void* x_fp8,
+                                     float* scale_out, uint32_t* amax_bits, uint32_t* status, uint32_t* counters,
+                                     uint32_t* words, int64_t wait_clocks, cudaStream_t stream) {
+    const int sms = sm_count();
+    if (sms <= 0) return FP8ATTN_ERR_CUDA;
+    const Form f = quantize_form(1, n_heads, elems_per_head, 0, 0u, sms);
+    if (f.kind != Form::kStaged) return FP8ATTN_ERR_UNSUPPORTED;
+    QuantBatch b = {};
+    b.x[0] = static_cast<const uint4*>(x_bf16);
+    b.out[0] = static_cast<uint4*>(x_fp8);
+    b.scale_out[0] = scale_out;
+    return launch_staged<false>(f, b, status, counters, words, amax_bits, stream, wait_clocks);
 }
 
 int quantize_stages(int tensors, int64_t n_heads, int64_t elems_train, int64_t elems_test, uint32_t flags, int sms) {

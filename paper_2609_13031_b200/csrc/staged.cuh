@@ -44,7 +44,7 @@ constexpr int kBufVecs = 7088;                 // 16-byte vectors per buffer: a 
 constexpr int kParts = 2;                      // a buffer is given up in halves
 constexpr size_t kSmemBytes = (size_t)2 * kBufVecs * 16;
 constexpr int kMaxSegments = 48;               // per share
-constexpr int64_t kWaitClocks = 4000000000ll;  // 2 s
+constexpr int64_t kWaitClocks = 4000000000ll;  // 2 s (Args::wait_clocks of every call but the self-test)
 
 // The sizes of a call and how it is cut (host arithmetic only, see plan()).
 struct Shape {
@@ -69,6 +69,7 @@ struct Args : Shape {
     float* result_out[3];       // per head (NULL: none)
     const uint4* follow_x;      // values may lie outside the range of tensor 0
     void* follow_out;
+    int64_t wait_clocks;        // limit of every wait
     uint32_t* status;
     uint32_t* counter;          // blocks done
     uint32_t* slots;            // published values
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
     const uint32_t vecs = (uint32_t)a.vecs, tensors = (uint32_t)a.tensors;
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
-            mbar_init(smem_u32(&full[i]), 1);
+            mbar_init(smem_u32(&full[i]), kParts);
             mbar_init(smem_u32(&known[i]), 1);
             for (int part = 0; part < kParts; ++part) mbar_init(smem_u32(&part_free[i][part]), kWorkers / 32);
         }
@@ -190,13 +191,13 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
         if (f_lo + tid * 8 < f_hi) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.follow_x + f_lo + tid * 8));
     }
     __syncthreads();
+    int parts = 0;      // halves of stages that the load thread has requested
     const Share share_full((uint32_t)min(a.stage_units, a.units), vecs);
     const Share share_last((uint32_t)(a.units - (stages - 1) * a.stage_units), vecs);
 
     if (warp == kWorkers / 32) {
         // ============================== loads ==============================
         if (lane == 0) {
-            int issued = 0;     // stages
             bool on = true;
             auto pieces = [&](int stage, uint32_t part, auto to) {
                 half_share(a, stage + 1 < stages ? share_full : share_last, stage, part, to);
@@ -204,15 +205,14 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
             auto wait = [&](uint32_t bar, uint32_t parity) {
                 const int64_t t0 = clock64();
                 bool done = mbar_test_wait(bar, parity);
-                while (!done && !give_up && clock64() - t0 < kWaitClocks) done = mbar_try_wait(bar, parity);
+                while (!done && !give_up && clock64() - t0 < a.wait_clocks) done = mbar_try_wait(bar, parity);
                 return done;
             };
             auto load = [&](int stage, uint32_t part) {
                 const uint32_t buf = stage & 1, bar = smem_u32(&full[buf]);
-                if (part == 0) {
-                    mbar_arrive_expect_tx(bar, (stage + 1 < stages ? share_full : share_last).n * 16);
-                    issued = stage + 1;
-                }
+                const Share& s = stage + 1 < stages ? share_full : share_last;
+                mbar_arrive_expect_tx(bar, (part == 0 ? s.half() : s.n - s.half()) * 16);
+                ++parts;
                 pieces(stage, part, [&](uint32_t i0, const uint4* src, uint32_t n) {
                     bulk_load(smem_u32(smem) + (buf * kBufVecs + i0) * 16, src, n * 16, bar);
                 });
@@ -236,13 +236,7 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
                     if (on) load(stage, part);
                 }
             }
-            if (!on) {
-                lost = 1;
-                // copies land before the block exits (bounded: an aborted stage's last part was never issued)
-                const int64_t t0 = clock64();
-                for (int stage = max(0, issued - 2); stage < issued; ++stage)
-                    while (clock64() - t0 < kWaitClocks / 4 && !mbar_try_wait(smem_u32(&full[stage & 1]), (stage >> 1) & 1)) {}
-            }
+            if (!on) lost = 1;
         }
         __syncwarp();
     } else if (warp > kWorkers / 32) {
@@ -260,8 +254,10 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
                 }
             }
             sync_exchange();        // A: the share is reduced
-            // (block b and unit u of the stage meet at most once, and b + u names the meeting)
-            for (uint32_t g = lane; g < s.segs; g += 32) {
+            // (block b and unit u of the stage meet at most once, and b + u names the meeting; what never
+            // landed is not published)
+            bool there = !lost;
+            for (uint32_t g = lane; g < s.segs && there; g += 32) {
                 Op::publish(slots, a.slots_per_set, blockIdx.x + s.unit + g, tag, seg_acc[g]);
                 seg_acc[g] = typename Op::Acc(0);
             }
@@ -270,7 +266,6 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
             // more than four segments, its units span two blocks at most).
             const uint32_t width = s.segs <= 1 ? 32 : s.segs == 2 ? 16 : s.segs <= 4 ? 8 : 1;
             const bool none_empty = s.total >= 8 * gridDim.x;
-            bool there = !lost;
             const int64_t t0 = clock64();
             for (uint32_t g0 = 0; g0 < s.segs; g0 += 32 / width) {
                 const uint32_t g = g0 + lane / width;
@@ -289,7 +284,7 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
                                 const uint32_t b = min(b0 + k * width, b1);
                                 all &= Op::tagged(raw[k], tag) || (!none_empty && cut(s.total, b) == cut(s.total, b + 1));
                             }
-                            if (!all) there = !lost && clock64() - t0 < kWaitClocks;
+                            if (!all) there = !lost && clock64() - t0 < a.wait_clocks;
                         }
 #pragma unroll
                         for (int k = 0; k < kBatch; ++k)
@@ -354,7 +349,7 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
                 bool landed = mbar_test_wait(bar, parity);
                 if (!landed) {
                     const int64_t t0 = clock64();
-                    while (!landed && !lost && clock64() - t0 < kWaitClocks) landed = mbar_try_wait(bar, parity);
+                    while (!landed && !lost && clock64() - t0 < a.wait_clocks) landed = mbar_try_wait(bar, parity);
                 }
                 if (!__all_sync(0xffffffffu, landed)) lost = 1;
                 for (uint32_t g = 0; g < s.segs; ++g) {
@@ -390,6 +385,13 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
         }
     }
     __syncthreads();
+    // ---- a block that gives up leaves when its copies have landed ----
+    if (give_up && tid == kWorkers) {
+        if (parts & 1) mbar_arrive(smem_u32(&full[parts >> 1 & 1]));      // for the half that was never requested
+        const int64_t t0 = clock64();
+        for (int n = (parts + 1) / 2, stage = max(0, n - 2); stage < n; ++stage)
+            while (!mbar_try_wait(smem_u32(&full[stage & 1]), (stage >> 1) & 1) && clock64() - t0 < kWaitClocks) {}
+    }
     // ---- rows that follow tensor 0 ----
     if (!give_up) {
         bool there = true;
@@ -402,7 +404,7 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
             const uint32_t end = f_hi - seg.head * a.follow_vecs < a.follow_vecs ? f_hi : (seg.head + 1) * a.follow_vecs;
             typename Op::Raw raw = Op::load(a.heads, 0, seg.head);
             while (there && !Op::tagged(raw, 1)) {
-                there = clock64() - t0 < kWaitClocks;
+                there = clock64() - t0 < a.wait_clocks;
                 raw = Op::load(a.heads, 0, seg.head);
             }
             seg.result = Op::result(a.op, Op::value(raw));

@@ -33,8 +33,46 @@ def test_expired_wait_is_reported_is_sticky_and_clears():
     assert not torch.all(out == 7.0) and torch.isfinite(out.float()).all()
 
 
+@pytest.mark.parametrize("H,n,d,stages", [(4, 3000, 64, 1), (8, 20011, 128, 3), (3, 40000, 128, 3)])
+@pytest.mark.parametrize("limit", [1, 2000, 6000, 20000])
+def test_one_pass_quantizer_gives_up_cleanly(H, n, d, stages, limit):
+    """Waits that run out (at once, or in the middle of a stage whose copies are under way): the call
+    comes back, says so, leaves its words at zero and writes nowhere else; the next call is right."""
+    assert api.quantize_stages(1, 1, H, n, 0, d) == stages
+    torch.manual_seed(n + limit)
+    x = torch.randn((1, H, n, d), device="cuda").to(torch.bfloat16)
+    want, want_scale = torch.empty_like(x, dtype=torch.uint8), torch.empty((1, H), device="cuda")
+    api.quantize_noalloc(x, want, want_scale)
+    ws = api.new_workspace(1, H)
+    guarded = torch.full((x.numel() + 8192,), 0x55, dtype=torch.uint8, device="cuda")
+    codes, scale = guarded[4096:-4096].view(x.shape), torch.zeros((1, H), device="cuda")
+    for _ in range(3):
+        api.selftest_quantize_timeout(x, ws, codes, scale, limit_clocks=limit)
+        torch.cuda.synchronize()
+        left = ws.clone()
+        assert not left[16:].any()                             # counter, words and accumulators
+        assert (guarded[:4096] == 0x55).all() and (guarded[-4096:] == 0x55).all()
+        status, detail = api.last_device_status(ws)
+        assert status in (api.OK, api.ERR_TIMEOUT) and (limit > 1 or status == api.ERR_TIMEOUT)
+        assert (detail >> 24) == (32 if status else 0)
+        if status == api.OK:
+            assert torch.equal(codes, want) and torch.equal(scale, want_scale)
+        got, got_scale = api.quantize(x, ws)
+        assert torch.equal(got, want) and torch.equal(got_scale, want_scale)
+        assert api.last_device_status(ws) == (0, 0)
+
+
 def test_selftest_argument_checks():
     lib = api.load()
     ws = api.new_workspace(1, 1)
     assert lib.fp8attn_selftest_wait_timeout(ws.data_ptr(), ws.numel(), 0, None) == api.ERR_INVALID_ARG
     assert lib.fp8attn_selftest_wait_timeout(None, ws.numel(), 10, None) == api.ERR_WORKSPACE
+    x = torch.zeros((1, 1, 1025, 64), dtype=torch.bfloat16, device="cuda")
+    o, s = torch.empty_like(x, dtype=torch.uint8), torch.empty((1, 1), device="cuda")
+    call = lambda rows, limit, w=ws.data_ptr(): lib.fp8attn_selftest_quantize_timeout(
+        x.data_ptr(), 1, 1, rows, 64, o.data_ptr(), s.data_ptr(), limit, w, ws.numel(), None)
+    assert call(1025, 0) == call(0, 10) == call(1025, 200000000) == api.ERR_INVALID_ARG
+    assert call(1024, 10) == api.ERR_UNSUPPORTED                # a block per head: no waits
+    assert call(1025, 10, None) == api.ERR_WORKSPACE
+    torch.cuda.synchronize()
+    assert api.last_device_status(ws) == (0, 0)
