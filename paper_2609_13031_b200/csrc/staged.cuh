@@ -19,8 +19,10 @@
 // the work).
 //
 // The blocks are launched cooperatively, i.e. resident together or not at all; the waits are
-// bounded all the same (kWaitClocks: FP8ATTN_ERR_TIMEOUT in the status word).  The last block to
-// finish leaves the published words and its counter at zero for the next call.
+// bounded all the same (kWaitClocks: FP8ATTN_ERR_TIMEOUT in the status word).  The last block whose
+// exchange warp has read all that it will read leaves the published words and the counter at zero for
+// the next call, while the workers convert.  (At the end of the kernel the fence that orders this waits
+// for the block's output stores: 1 us a call.)
 //
 // Measured, quantizer, 8 heads of 65,536 + 16,384 rows x 128 (654 MB in and out, 100 us at the copy
 // rate): 128 us, two passes 182 us; 16 heads of 30,011 x 64 62.6 / 89.1 us; 8 heads of 20,011 + 3,001 x
@@ -44,6 +46,7 @@ constexpr int kBufVecs = 7088;                 // 16-byte vectors per buffer: a 
 constexpr int kParts = 2;                      // a buffer is given up in halves
 constexpr size_t kSmemBytes = (size_t)2 * kBufVecs * 16;
 constexpr int kMaxSegments = 48;               // per share
+constexpr int kMaxFollowHeads = 32;            // whose rows follow in one block, in calls that clear nothing first
 constexpr int64_t kWaitClocks = 4000000000ll;  // 2 s (Args::wait_clocks of every call but the self-test)
 
 // The sizes of a call and how it is cut (host arithmetic only, see plan()).
@@ -164,9 +167,9 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
     __shared__ typename Op::Acc seg_acc[kMaxSegments];
     __shared__ Segment<Op> segment[2][kMaxSegments];
     __shared__ uint16_t holders[kMaxSegments][2];       // first and last block of every segment's unit
+    __shared__ typename Op::Acc follow_acc[kMaxFollowHeads];
     __shared__ volatile int lost, give_up;
-    __shared__ int last;
-    static_assert(kSmemBytes + sizeof(segment) + sizeof(seg_acc) + 768 <= 232448, "shared memory of a block");
+    static_assert(kSmemBytes + sizeof(segment) + sizeof(seg_acc) + sizeof(follow_acc) + 768 <= 232448, "shared memory of a block");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int stages = a.stages;
     const uint32_t vecs = (uint32_t)a.vecs, tensors = (uint32_t)a.tensors;
@@ -194,6 +197,11 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
     int parts = 0;      // halves of stages that the load thread has requested
     const Share share_full((uint32_t)min(a.stage_units, a.units), vecs);
     const Share share_last((uint32_t)(a.units - (stages - 1) * a.stage_units), vecs);
+
+    auto timed_out = [&] {
+        if (atomicCAS(a.status, 0u, (uint32_t)FP8ATTN_ERR_TIMEOUT) == 0u)
+            a.status[1] = (kDetailGridWait << 24) | (blockIdx.x & 0xFFFFFFu);
+    };
 
     if (warp == kWorkers / 32) {
         // ============================== loads ==============================
@@ -309,13 +317,46 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
                 }
             }
             if (!__all_sync(0xffffffffu, there) && lane == 0) {
-                if (atomicCAS(a.status, 0u, (uint32_t)FP8ATTN_ERR_TIMEOUT) == 0u)
-                    a.status[1] = (kDetailGridWait << 24) | (blockIdx.x & 0xFFFFFFu);
+                timed_out();
                 give_up = 1;
             }
             if (lane == 0) mbar_arrive(smem_u32(&known[stage & 1]));
             sync_exchange();        // B: results are known
             if (give_up) break;
+        }
+        // The heads that this block's following rows belong to (calls that cleared the words read them
+        // when they convert).
+        if (f_lo < f_hi && !a.cleared && !give_up) {
+            const uint32_t h = f_lo / a.follow_vecs + lane;
+            bool there = true;
+            if (h <= (f_hi - 1) / a.follow_vecs) {
+                const int64_t t0 = clock64();
+                typename Op::Raw raw = Op::load(a.heads, 0, h);
+                while (there && !Op::tagged(raw, 1)) {
+                    there = clock64() - t0 < a.wait_clocks;
+                    raw = Op::load(a.heads, 0, h);
+                }
+                follow_acc[lane] = Op::value(raw);
+            }
+            if (!__all_sync(0xffffffffu, there) && lane == 0) {
+                timed_out();
+                give_up = 1;
+            }
+        }
+        // The last warp to get here leaves everything at zero for the next call: its fence and those of the
+        // others put all stores and polls of the words before that.
+        __syncwarp();
+        uint32_t done = 0;
+        if (lane == 0) {
+            __threadfence();
+            done = atomicAdd(a.counter, 1u);
+            __threadfence();
+        }
+        if (__shfl_sync(0xffffffffu, done, 0) == gridDim.x - 1) {
+            for (uint32_t i = lane; i < a.sets * a.slots_per_set; i += 32) a.slots[i] = 0u;
+            if (a.follow_vecs > 0 && !a.cleared)
+                for (int i = lane; i < a.units / a.tensors; i += 32) a.heads[i] = 0u;
+            if (lane == 0) *a.counter = 0u;
         }
     } else {
         // ============================== workers ==============================
@@ -402,31 +443,20 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
         for (uint32_t x = f_lo; x < f_hi && there;) {
             seg.head = x / a.follow_vecs;
             const uint32_t end = f_hi - seg.head * a.follow_vecs < a.follow_vecs ? f_hi : (seg.head + 1) * a.follow_vecs;
-            typename Op::Raw raw = Op::load(a.heads, 0, seg.head);
-            while (there && !Op::tagged(raw, 1)) {
-                there = clock64() - t0 < a.wait_clocks;
-                raw = Op::load(a.heads, 0, seg.head);
+            typename Op::Acc v = follow_acc[a.cleared ? 0 : seg.head - f_lo / a.follow_vecs];
+            if (a.cleared) {
+                typename Op::Raw raw = Op::load(a.heads, 0, seg.head);
+                while (there && !Op::tagged(raw, 1)) {
+                    there = clock64() - t0 < a.wait_clocks;
+                    raw = Op::load(a.heads, 0, seg.head);
+                }
+                v = Op::value(raw);
             }
-            seg.result = Op::result(a.op, Op::value(raw));
+            seg.result = Op::result(a.op, v);
             if (there && tid < kWorkers) Op::template convert<true>(a.op, seg, a.follow_x, x, end, tid);
             x = end;
         }
-        if (!there && atomicCAS(a.status, 0u, (uint32_t)FP8ATTN_ERR_TIMEOUT) == 0u)
-            a.status[1] = (kDetailGridWait << 24) | (blockIdx.x & 0xFFFFFFu);
-    }
-    // ---- the last block to finish leaves everything at zero for the next call ----
-    __syncthreads();
-    if (tid == 0) {     // every block's stores and polls of the words come before the zeros
-        __threadfence();
-        last = atomicAdd(a.counter, 1u) == gridDim.x - 1;
-        __threadfence();
-    }
-    __syncthreads();
-    if (last) {
-        for (uint32_t i = tid; i < a.sets * a.slots_per_set ; i += kThreads) a.slots[i] = 0u;
-        if (a.follow_vecs > 0)
-            for (int i = tid; i < a.units / a.tensors ; i += kThreads) a.heads[i] = 0u;
-        if (tid == 0) *a.counter = 0u;
+        if (!there) timed_out();
     }
 }
 
@@ -458,7 +488,7 @@ inline unsigned plan(Shape& a, int sms) {
     const int64_t per_set = grid + a.stage_units;
     // the words of the heads sit behind the slots, or where the call clears them first
     const int64_t head_words = !a.cleared && a.follow_vecs > 0 ? a.units / a.tensors : 0;
-    if (a.sets * per_set + head_words > kOnePassWords) return 0;
+    if (a.sets * per_set + head_words > kOnePassWords || (head_words > 0 && head_words / grid + 2 > kMaxFollowHeads)) return 0;
     a.slots_per_set = (uint32_t)per_set;
     return (unsigned)grid;
 }
