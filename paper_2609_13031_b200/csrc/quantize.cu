@@ -189,6 +189,7 @@ struct QuantizeOp {
     using Result = Divisor;
     static constexpr int kOutBytes = 8;     // per 16-byte input vector
     // a published value is one word: tag << 16 | maximum
+    static constexpr Acc kLost = 0xffffffffu;   // published: no tag (tags are below 0xffff)
 
     // thread `tid`'s part of `vecs` vectors
     static __device__ __forceinline__ Acc reduce(const uint4* x, int vecs, int tid) {
@@ -424,9 +425,9 @@ int launch_heads(const Form& f, const QuantBatch& b, cudaStream_t stream) {
 
 // The one-pass kernel for the tensors of `b`: tensors [0, tensors) and, if there are test rows, tensor 3
 // with the scale of tensor 0.  amax_bits: the accumulators of the two-pass form, free here.
-template <bool kHalf>
+template <bool kHalf, bool kSelfTest = false>
 int launch_staged(const Form& f, const QuantBatch& b, uint32_t* status, uint32_t* counters, uint32_t* words,
-                  uint32_t* amax_bits, cudaStream_t stream, int64_t wait_clocks = staged::kWaitClocks) {
+                  uint32_t* amax_bits, cudaStream_t stream, int64_t wait_clocks = 0) {
     staged::Args<QuantizeOp<kHalf>> a = {};
     static_cast<staged::Shape&>(a) = f.shape;
     for (int z = 0; z < a.tensors; ++z) {
@@ -441,7 +442,7 @@ int launch_staged(const Form& f, const QuantBatch& b, uint32_t* status, uint32_t
     a.counter = counters;
     a.slots = words;
     a.heads = a.cleared ? amax_bits : words + a.sets * a.slots_per_set;
-    return staged::launch(a, f.grid, stream);
+    return staged::launch<kSelfTest>(a, f.grid, stream);
 }
 
 }  // namespace
@@ -590,7 +591,7 @@ int launch_quantize_timeout_selftest(const void* x_bf16, int64_t n_heads, int64_
     b.x[0] = static_cast<const uint4*>(x_bf16);
     b.out[0] = static_cast<uint4*>(x_fp8);
     b.scale_out[0] = scale_out;
-    return launch_staged<false>(f, b, status, counters, words, amax_bits, stream, wait_clocks);
+    return launch_staged<false, true>(f, b, status, counters, words, amax_bits, stream, wait_clocks);
 }
 
 int quantize_stages(int tensors, int64_t n_heads, int64_t elems_train, int64_t elems_test, uint32_t flags, int sms) {
