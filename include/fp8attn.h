@@ -19,8 +19,9 @@
  *     host before anything is launched.  Device-side problems (a bounded wait
  *     that ran out) are recorded in the workspace and read back with
  *     fp8attn_last_device_status(); the kernels never trap or spin forever.  A
- *     recorded device error is sticky: attention launches on that workspace do
- *     nothing until fp8attn_last_device_status() has read and cleared it.
+ *     recorded device error is sticky: attention launches on that workspace, and
+ *     fp8attn_quantize_qkv calls of up to 48 MB of 16-bit input that run in one
+ *     pass, write nothing until fp8attn_last_device_status() has read and cleared it.
  *   - Supported head dims: d = 64 and d = 128.  n_train >= 1, n_test >= 0, each
  *     below 2^31 - 256; B*H <= 65535.
  */

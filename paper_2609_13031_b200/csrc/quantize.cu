@@ -256,6 +256,7 @@ struct HeadArgs {
     const uint4* x[4];
     uint2* out[4];
     float* scale_out[4];
+    const uint32_t* status;     // write nothing while an error is recorded there (NULL: do not look)
     int tensors, n_heads;
     int vecs;                   // per head of the tensors that are reduced
     int counts;                 // the test rows enter the maximum of tensor 0
@@ -264,14 +265,18 @@ struct HeadArgs {
     int64_t piece_vecs;
 };
 
+__device__ __forceinline__ uint32_t recorded_error(const HeadArgs& a) {
+    return threadIdx.x == 0 && a.status != nullptr ? *reinterpret_cast<const volatile uint32_t*>(a.status) : 0u;
+}
 template <bool kHalf>
-__device__ __forceinline__ Divisor block_divisor(typename In16<kHalf>::V2 m, uint32_t* warp_max) {
+__device__ __forceinline__ bool block_divisor(typename In16<kHalf>::V2 m, uint32_t* warp_max, uint32_t error, Divisor& dv) {
     const uint32_t w = *reinterpret_cast<const uint32_t*>(&m);
     uint32_t top = __reduce_max_sync(0xffffffffu, max(w & 0xffffu, w >> 16));
     if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = top;
-    __syncthreads();
+    if (__syncthreads_or((int)error)) return false;
     top = __reduce_max_sync(0xffffffffu, (threadIdx.x & 31) < blockDim.x / 32 ? warp_max[threadIdx.x & 31] : 0u);
-    return divisor(head_scale(In16<kHalf>::lo(top)));
+    dv = divisor(head_scale(In16<kHalf>::lo(top)));
+    return true;
 }
 // (the per-element division stays out of the unrolled loops: small calls pay for the code they fetch)
 template <bool kHalf>
@@ -309,19 +314,24 @@ __global__ void __launch_bounds__(1024) quantize_heads_kernel(const __grid_const
             const int i = tid + k * (int)blockDim.x;
             v[k] = i < a.vecs ? ld_nc_v4(x + i) : make_uint4(0u, 0u, 0u, 0u);
         }
+        const uint32_t error = recorded_error(a);
 #pragma unroll
         for (int k = 0; k < kHeadPer; ++k) m = absmax8<kHalf>(m, v[k]);
         const uint4* test_x = a.x[3] + head * a.test_vecs;
         if (a.counts && z == 0)
             for (int64_t i = tid; i < a.test_vecs; i += blockDim.x) m = absmax8<kHalf>(m, ld_nc_v4(test_x + i));
-        const Divisor dv = block_divisor<kHalf>(m, warp_max);
+        Divisor dv;
+        if (!block_divisor<kHalf>(m, warp_max, error, dv)) return;
         if (tid == 0) a.scale_out[z][head] = dv.s;
         uint2* out = a.out[z] + (int64_t)head * a.vecs;
-        if (dv.direct) convert_direct<kHalf>(x, out, a.vecs, dv);
+        if (dv.direct) {
+            convert_direct<kHalf>(x, out, a.vecs, dv);
+        } else {
 #pragma unroll
-        for (int k = 0; k < kHeadPer; ++k) {
-            const int i = tid + k * (int)blockDim.x;
-            if (i < a.vecs && !dv.direct) out[i] = quant8<kHalf, false>(v[k], dv);
+            for (int k = 0; k < kHeadPer; ++k) {
+                const int i = tid + k * (int)blockDim.x;
+                if (i < a.vecs) out[i] = quant8<kHalf, false>(v[k], dv);
+            }
         }
         if (z == 0 && a.pieces == 0) convert_rows<kHalf>(test_x, a.out[3] + head * a.test_vecs, a.test_vecs, dv);
     } else {
@@ -329,11 +339,13 @@ __global__ void __launch_bounds__(1024) quantize_heads_kernel(const __grid_const
         const int64_t first = (int64_t)(item - head * a.pieces) * a.piece_vecs;
         const uint4* head_x = a.x[0] + (int64_t)head * a.vecs;
         const uint4* test_x = a.x[3] + head * a.test_vecs;
+        const uint32_t error = recorded_error(a);
 #pragma unroll 4
         for (int i = tid; i < a.vecs; i += blockDim.x) m = absmax8<kHalf>(m, ld_nc_v4(head_x + i));
         if (a.counts)
             for (int64_t i = tid; i < a.test_vecs; i += blockDim.x) m = absmax8<kHalf>(m, ld_nc_v4(test_x + i));
-        const Divisor dv = block_divisor<kHalf>(m, warp_max);
+        Divisor dv;
+        if (!block_divisor<kHalf>(m, warp_max, error, dv)) return;
         convert_rows<kHalf>(test_x + first, a.out[3] + head * a.test_vecs + first, min(a.piece_vecs, a.test_vecs - first), dv);
     }
 }
@@ -363,12 +375,15 @@ struct Form {
     staged::Shape shape;        // kStaged
     HeadArgs heads;             // kHeads: without its pointers
     unsigned threads;           // kHeads
+    bool heed_status;           // a fused call that is one launch writes nothing while an error is recorded
 };
 Form quantize_form(int tensors, int64_t n_heads, int64_t elems_train, int64_t elems_test, uint32_t flags, int sms) {
     Form f = {};
     if ((flags & (FP8ATTN_SCALES_GIVEN | FP8ATTN_QKV_TWO_LAUNCHES)) || elems_train <= 0) return f;
     const int64_t vecs = elems_train / 8, follow = elems_test / 8;
     const bool counts = follow > 0 && (flags & FP8ATTN_QUERY_SCALE_FROM_ALL_ROWS);
+    const bool large = (vecs * tensors + follow) * n_heads * 16 > kOneLaunchMaxBytes;
+    f.heed_status = tensors == 3 && !large;
     if (vecs <= kHeadVecs) {
         if (counts && follow > kHeadVecs) return f;
         // Pieces of the test rows: two per SM, but none so small that reading the train queries again is
@@ -404,15 +419,16 @@ Form quantize_form(int tensors, int64_t n_heads, int64_t elems_train, int64_t el
     a.vecs = vecs;
     a.follow_vecs = (uint32_t)follow;
     a.follow_counts = counts;
-    a.cleared = (a.vecs * a.units + follow * n_heads) * 16 > kOneLaunchMaxBytes;
+    a.cleared = large;
     f.grid = staged::plan(a, sms);
     if (f.grid > 0 && (!a.cleared || one_pass_pays(a))) f.kind = Form::kStaged;
     return f;
 }
 
 template <bool kHalf>
-int launch_heads(const Form& f, const QuantBatch& b, cudaStream_t stream) {
+int launch_heads(const Form& f, const QuantBatch& b, const uint32_t* status, cudaStream_t stream) {
     HeadArgs a = f.heads;
+    a.status = f.heed_status ? status : nullptr;
     for (int z = 0; z < 4; ++z) {
         a.x[z] = b.x[z];
         a.out[z] = reinterpret_cast<uint2*>(b.out[z]);
@@ -438,6 +454,7 @@ int launch_staged(const Form& f, const QuantBatch& b, uint32_t* status, uint32_t
     a.follow_x = b.x[3];
     a.follow_out = b.out[3];
     a.wait_clocks = wait_clocks;
+    a.heed_status = f.heed_status;
     a.status = status;
     a.counter = counters;
     a.slots = words;
@@ -485,7 +502,7 @@ int launch_quantize_qkv(const void* q_train, const void* k, const void* v, const
     const bool half = (flags & FP8ATTN_INPUT_FP16) != 0;
     if (key_dest == nullptr) {
         const Form f = quantize_form(3, n_heads, elems_train, elems_test, flags, sms);
-        if (f.kind == Form::kHeads) return half ? launch_heads<true>(f, b, stream) : launch_heads<false>(f, b, stream);
+        if (f.kind == Form::kHeads) return half ? launch_heads<true>(f, b, status, stream) : launch_heads<false>(f, b, status, stream);
         if (f.kind == Form::kStaged)
             return half ? launch_staged<true>(f, b, status, counters, words, amax_bits, stream)
                         : launch_staged<false>(f, b, status, counters, words, amax_bits, stream);
@@ -551,7 +568,7 @@ int launch_quantize(const void* x_bf16, int64_t n_heads, int64_t elems_per_head,
             b.x[0] = static_cast<const uint4*>(x_bf16);
             b.out[0] = static_cast<uint4*>(x_fp8);
             b.scale_out[0] = scale_out;
-            if (f.kind == Form::kHeads) return half ? launch_heads<true>(f, b, stream) : launch_heads<false>(f, b, stream);
+            if (f.kind == Form::kHeads) return half ? launch_heads<true>(f, b, status, stream) : launch_heads<false>(f, b, status, stream);
             return half ? launch_staged<true>(f, b, status, counters, words, amax_bits, stream)
                         : launch_staged<false>(f, b, status, counters, words, amax_bits, stream);
         }

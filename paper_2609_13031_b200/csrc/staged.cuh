@@ -73,6 +73,7 @@ struct Args : Shape {
     const uint4* follow_x;      // values may lie outside the range of tensor 0
     void* follow_out;
     int64_t wait_clocks;        // limit of every wait of the self-test
+    bool heed_status;           // write nothing while an error is recorded
     uint32_t* status;
     uint32_t* counter;          // blocks done
     uint32_t* slots;            // published values
@@ -253,6 +254,8 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
         __syncwarp();
     } else if (warp > kWorkers / 32) {
         // ============================== exchange ==============================
+        // (recorded before this launch, so all blocks decide alike; asked for under the first loads)
+        const bool pending = a.heed_status && *reinterpret_cast<volatile uint32_t*>(a.status) != 0u;
         for (int stage = 0; stage < stages; ++stage) {
             const Share& s = stage + 1 < stages ? share_full : share_last;
             const uint32_t u0 = (uint32_t)(stage * a.stage_units) + s.unit;
@@ -276,7 +279,7 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
             // more than four segments, its units span two blocks at most).
             const uint32_t width = s.segs <= 1 ? 32 : s.segs == 2 ? 16 : s.segs <= 4 ? 8 : 1;
             const bool none_empty = s.total >= 8 * gridDim.x;
-            bool there = !lost;
+            bool there = !lost && !pending;
             const int64_t t0 = clock64();
             for (uint32_t g0 = 0; g0 < s.segs; g0 += 32 / width) {
                 const uint32_t g = g0 + lane / width;
@@ -320,7 +323,7 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
                 }
             }
             if (!__all_sync(0xffffffffu, there) && lane == 0) {
-                timed_out();
+                if (!pending) timed_out();
                 give_up = 1;
             }
             if (lane == 0) mbar_arrive(smem_u32(&known[stage & 1]));

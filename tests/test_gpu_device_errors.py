@@ -33,6 +33,26 @@ def test_expired_wait_is_reported_is_sticky_and_clears():
     assert not torch.all(out == 7.0) and torch.isfinite(out.float()).all()
 
 
+@pytest.mark.parametrize("n,m,stages", [(512, 128, -1), (3000, 200, 1), (8192, 2048, 2)])
+def test_small_fused_quantization_writes_nothing_while_an_error_is_pending(n, m, stages):
+    assert api.quantize_stages(3, 1, 8, n, m, 64) == stages
+    q, k, v = (torch.randn((1, 8, n, 64), device="cuda").to(torch.bfloat16) for _ in range(3))
+    t = torch.randn((1, 8, m, 64), device="cuda").to(torch.bfloat16)
+    ws = api.new_workspace(1, 8)
+    want = api.quantize_qkv(q, k, v, t, ws, flags=api.QKV_TWO_LAUNCHES)
+    out = {name: torch.full_like(x, 7) for name, x in want.items()}
+    api.selftest_wait_timeout(ws, limit_us=500)
+    api.quantize_qkv(q, k, v, t, ws, out=out)
+    assert all((x == 7).all() for x in out.values())
+    code, scale = api.quantize(k, ws)                              # tensors by themselves are quantized all the same
+    assert torch.equal(code, want["k8"]) and torch.equal(scale, want["sk"])
+    status, detail = api.last_device_status(ws)
+    assert status == api.ERR_TIMEOUT and detail >> 24 == 11         # the self-test's, not one of the quantizer's
+    api.quantize_qkv(q, k, v, t, ws, out=out)
+    assert all(torch.equal(out[name], want[name]) for name in want)
+    assert api.last_device_status(ws) == (0, 0)
+
+
 @pytest.mark.parametrize("H,n,d,stages", [(4, 3000, 64, 1), (8, 20011, 128, 3), (3, 40000, 128, 3)])
 @pytest.mark.parametrize("limit", [1, 2000, 6000, 20000])
 def test_one_pass_quantizer_gives_up_cleanly(H, n, d, stages, limit):
