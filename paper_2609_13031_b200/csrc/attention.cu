@@ -20,6 +20,8 @@
 //
 // Scale placement (FP8 path): x = (alpha * s_q * s_k * log2 e) * S feeds exp2;
 // the V scale and 1/rowsum are applied to O in the epilogue.
+#include <type_traits>
+
 #include <cuda_bf16.h>
 
 #include "common.h"
@@ -760,14 +762,16 @@ icl_attention_kernel(const __grid_constant__ CUtensorMap map_q_train,
 }
 
 // Combines the partial results of the split query blocks: with M = max_s c*m_s,
-// out = s_v * sum_s 2^(c*m_s - M) O_s / sum_s 2^(c*m_s - M) l_s.  One thread per row and four output
-// columns.  Bound by the latency of its loads, which come from L2: eight ranges are under way at a
-// time (8 x 300 rows of d = 64 in 9 ranges: 6.9 us with one at a time).
-template <int kD, int kT>
+// out = s_v * sum_s 2^(c*m_s - M) O_s / sum_s 2^(c*m_s - M) l_s.  One thread per row and 4 * kVecs output
+// columns.  With few rows (kVecs = 1) it is bound by the latency of its loads, which come from L2: eight ranges
+// are under way at a time (8 x 300 rows of d = 64 in 9 ranges: 6.9 us with one at a time), the last of them
+// repeated where there are fewer.  With many rows (kVecs = 2) it is bound by the loads themselves: exactly
+// the ranges there are, eight columns per thread (8 x 2,048 rows of d = 64 in 3 ranges, whole call: 57.9 ->
+// 55.5 us; 16 x 700 rows of d = 128 52.6 -> 50.3 us; the other way round 2 x 300 rows in 37 ranges 53 -> 58 us).
+template <int kD, int kT, int kVecs>
 __global__ void __launch_bounds__(256)
 combine_split_kernel(const KernelArgs args, int units, int out_half, int fp8) {
-    constexpr int kBatch = 8;
-    const int per_row = kD / 4;
+    constexpr int per_row = kD / (4 * kVecs);
     const int64_t tid = (int64_t)blockIdx.x * 256 + threadIdx.x;
     const int64_t unit = tid / (kRowsPerBlock<kT> * per_row);
     if (unit >= units) return;
@@ -784,43 +788,59 @@ combine_split_kernel(const KernelArgs args, int units, int out_half, int fp8) {
     const float* base = args.partial + ((size_t)unit * args.splits * kRowsPerBlock<kT> + r) * kPartialStride<kD>;
     const size_t split_stride = (size_t)kRowsPerBlock<kT> * kPartialStride<kD>;
     float m = -INFINITY, lsum = 0.f;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s0 = 0; s0 < args.splits; s0 += kBatch) {
-        float2 ml[kBatch];
-        float4 o[kBatch];
+    float4 acc[kVecs] = {};
+    // kN ranges from `from` on, all their loads under way at a time
+    auto add = [&](auto n, int from) {
+        constexpr int kN = decltype(n)::value;
+        float2 ml[kN];
+        float4 o[kN][kVecs];
 #pragma unroll
-        for (int k = 0; k < kBatch; ++k) {
-            const float* ps = base + (size_t)min(s0 + k, args.splits - 1) * split_stride;
+        for (int k = 0; k < kN; ++k) {
+            const float* ps = base + (size_t)(kVecs == 1 ? min(from + k, args.splits - 1) : from + k) * split_stride;
             ml[k] = *reinterpret_cast<const float2*>(ps + kD);
-            o[k] = *reinterpret_cast<const float4*>(ps + g * 4);
+#pragma unroll
+            for (int i = 0; i < kVecs; ++i) o[k][i] = *reinterpret_cast<const float4*>(ps + (g * kVecs + i) * 4);
         }
         float m_new = m;
 #pragma unroll
-        for (int k = 0; k < kBatch; ++k) m_new = fmaxf(m_new, ml[k].x);     // (a repeated range changes no maximum)
+        for (int k = 0; k < kN; ++k) m_new = fmaxf(m_new, ml[k].x);
         const float f = exp2f(m - m_new);
         m = m_new;
         lsum *= f;
-        acc.x *= f; acc.y *= f; acc.z *= f; acc.w *= f;
 #pragma unroll
-        for (int k = 0; k < kBatch; ++k) {
-            const float wgt = s0 + k < args.splits ? exp2f(ml[k].x - m) : 0.f;
+        for (int i = 0; i < kVecs; ++i) { acc[i].x *= f; acc[i].y *= f; acc[i].z *= f; acc[i].w *= f; }
+#pragma unroll
+        for (int k = 0; k < kN; ++k) {
+            const float wgt = kVecs == 1 && from + k >= args.splits ? 0.f : exp2f(ml[k].x - m);
             lsum = fmaf(wgt, ml[k].y, lsum);
-            acc.x = fmaf(wgt, o[k].x, acc.x); acc.y = fmaf(wgt, o[k].y, acc.y);
-            acc.z = fmaf(wgt, o[k].z, acc.z); acc.w = fmaf(wgt, o[k].w, acc.w);
+#pragma unroll
+            for (int i = 0; i < kVecs; ++i) {
+                acc[i].x = fmaf(wgt, o[k][i].x, acc[i].x); acc[i].y = fmaf(wgt, o[k][i].y, acc[i].y);
+                acc[i].z = fmaf(wgt, o[k][i].z, acc[i].z); acc[i].w = fmaf(wgt, o[k][i].w, acc[i].w);
+            }
         }
+    };
+    int s = 0;
+    for (; s + (kVecs == 1 ? 1 : 8) <= args.splits; s += 8) add(std::integral_constant<int, 8>(), s);
+    if (kVecs > 1) {
+        if (args.splits & 4) { add(std::integral_constant<int, 4>(), s); s += 4; }
+        if (args.splits & 2) { add(std::integral_constant<int, 2>(), s); s += 2; }
+        if (args.splits & 1) add(std::integral_constant<int, 1>(), s);
     }
     const float inv = (fp8 ? args.scale_v[bh_kv] : 1.0f) / lsum;
-    uint2 v;
-    if (out_half) {
-        v.x = pack_f16x2(acc.x * inv, acc.y * inv);
-        v.y = pack_f16x2(acc.z * inv, acc.w * inv);
-    } else {
-        v.x = pack_bf16x2(acc.x * inv, acc.y * inv);
-        v.y = pack_bf16x2(acc.z * inv, acc.w * inv);
+    uint32_t v[2 * kVecs];
+#pragma unroll
+    for (int i = 0; i < kVecs; ++i) {
+        const float4& x = acc[i];
+        v[2 * i] = out_half ? pack_f16x2(x.x * inv, x.y * inv) : pack_bf16x2(x.x * inv, x.y * inv);
+        v[2 * i + 1] = out_half ? pack_f16x2(x.z * inv, x.w * inv) : pack_bf16x2(x.z * inv, x.w * inv);
     }
     __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(is_test ? args.out_test : args.out_train) +
-                         ((int64_t)bh * q_rows + row) * kD;
-    *reinterpret_cast<uint2*>(out + g * 4) = v;
+                         ((int64_t)bh * q_rows + row) * kD + g * kVecs * 4;
+    if constexpr (kVecs == 2)
+        *reinterpret_cast<uint4*>(out) = make_uint4(v[0], v[1], v[2], v[3]);
+    else
+        *reinterpret_cast<uint2*>(out) = make_uint2(v[0], v[1]);
 }
 
 template <bool kFp8, int kD, bool kHalf, int kT>
@@ -861,9 +881,8 @@ int launch(const AttnParams& p, cudaStream_t stream) {
     a.full_blocks = (int)grid;
     a.splits = 1;
     a.partial = nullptr;
-    int units = 0;
+    int units = 0, sms = 0;
     if ((p.flags & FP8ATTN_SPLIT_TAIL) && p.partial != nullptr) {
-        int sms = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
             return FP8ATTN_ERR_CUDA;
         const int64_t full = (grid / sms) * sms, left = grid - full;
@@ -919,9 +938,12 @@ int launch(const AttnParams& p, cudaStream_t stream) {
         count_launch();
     }
     if (units > 0) {
-        const int64_t threads = (int64_t)units * kRowsPerBlock<kT> * (kD / 4);
-        combine_split_kernel<kD, kT><<<(unsigned)((threads + 255) / 256), 256, 0, stream>>>(
-            a, units, kHalf ? 1 : 0, kFp8 ? 1 : 0);
+        // eight columns per thread from two blocks per SM on
+        const int64_t rows = (int64_t)units * kRowsPerBlock<kT>;
+        const bool wide = rows * (kD / 8) >= 2 * 256 * (int64_t)sms;
+        const unsigned blocks = (unsigned)((rows * (kD / (wide ? 8 : 4)) + 255) / 256);
+        if (wide) combine_split_kernel<kD, kT, 2><<<blocks, 256, 0, stream>>>(a, units, kHalf ? 1 : 0, kFp8 ? 1 : 0);
+        else combine_split_kernel<kD, kT, 1><<<blocks, 256, 0, stream>>>(a, units, kHalf ? 1 : 0, kFp8 ? 1 : 0);
         count_launch();
     }
     return cudaGetLastError() == cudaSuccess ? FP8ATTN_OK : FP8ATTN_ERR_CUDA;
