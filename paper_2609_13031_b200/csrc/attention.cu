@@ -990,8 +990,10 @@ int launch_d64(const AttnParams& p, cudaStream_t stream) {
 //    rows, bf16: 3.27 -> 3.17 ms).
 //  - With FP8ATTN_SPLIT_TAIL, for a launch of less than one round (a few test rows against a long
 //    table, above all), whichever gives the shorter critical path: a block of T tiles takes kCost[T - 1]
-//    per key, and the more blocks there are the fewer key ranges each is split into.  300 rows of 8 heads
-//    against 262,144: two tiles 16 blocks in 9 ranges, 322 us; three tiles 8 blocks in 18, 236 us.
+//    per key, the more blocks there are the fewer key ranges each is split into, and every range of a row is
+//    written and read once more.  300 rows of 8 heads against 262,144: two tiles 16 blocks in 9 ranges, 322 us;
+//    three tiles 8 blocks in 18, 236 us.  2,048 rows of 8 heads against 4,096: 34.2 us and 35.4 us; against
+//    8,192 55.8 and 55.5 us; against 30,011 173 and 164 us.
 //  - Two otherwise (small grids pay for coarse blocks in their last round).
 int attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d, uint32_t flags, int sms,
                            size_t partial_bytes) {
@@ -1004,6 +1006,8 @@ int attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d,
     if ((flags & FP8ATTN_SPLIT_TAIL) && blocks2 > 0 && blocks2 < sms) {
         constexpr float kCost[3] = {0.72f, 1.0f, 1.43f};     // time per key of one, two, three tiles
         constexpr float kSplitSteps = 6.0f;                  // launch and combine, in steps of 128 keys
+        constexpr float kRangeSteps = 0.8f / 16384.0f;       // per row and range
+        const int64_t rows = heads * (train + n_test);
         const float steps = (float)n_train / 128.0f;
         const int64_t tiles = ((train > n_test ? train : n_test) + kTileM - 1) / kTileM;
         auto time = [&](int t, int64_t n) {
@@ -1012,9 +1016,9 @@ int attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d,
             if (splits > room) splits = room;
             if (splits > steps / 4) splits = (int64_t)(steps / 4);
             const float one = kCost[(tiles < t ? tiles : t) - 1] * steps;
-            return splits >= 2 ? one / (float)splits + kSplitSteps : one;
+            return splits >= 2 ? one / (float)splits + kSplitSteps + kRangeSteps * (float)(rows * splits) : one;
         };
-        if (time(3, blocks3) < 0.97f * time(2, blocks2)) return kRowsPerBlock<3>;
+        if (time(3, blocks3) < 0.975f * time(2, blocks2)) return kRowsPerBlock<3>;
     }
     return kRowsPerBlock<2>;
 }
