@@ -61,6 +61,10 @@ typedef enum {
  *
  * rows may be 0 (nothing is written except scale_out when scale_in is given).
  * Inputs containing NaN or infinity are not supported.
+ * Without scale_in, heads of 128 KB to 16 MB are held on chip by thread blocks that
+ * wait for one another (one per SM, launched cooperatively; fp8attn_quantize_qkv
+ * describes this form): a wait that runs out after 2 s ends in FP8ATTN_ERR_TIMEOUT in
+ * the workspace's status word.
  */
 int fp8attn_quantize(const void* x_bf16, int B, int H, int64_t rows, int d,
                      const float* scale_in, void* x_fp8, float* scale_out,
@@ -68,7 +72,9 @@ int fp8attn_quantize(const void* x_bf16, int B, int H, int64_t rows, int d,
 
 /* fp8attn_quantize with a flags word.  FP8ATTN_INPUT_FP16: x holds IEEE fp16
  * instead of bf16 (the paper's kernel benchmark table runs in float16); the
- * arithmetic is the same, on the exact fp32 value of each input.  flags = 0 is
+ * arithmetic is the same, on the exact fp32 value of each input.
+ * FP8ATTN_QKV_TWO_LAUNCHES (8): never take the form whose blocks wait for one
+ * another, e.g. beside long-running kernels of other streams.  flags = 0 is
  * fp8attn_quantize.  Unknown flag bits return FP8ATTN_ERR_INVALID_ARG. */
 #define FP8ATTN_INPUT_FP16 2u
 int fp8attn_quantize_ex(const void* x_16bit, int B, int H, int64_t rows, int d,

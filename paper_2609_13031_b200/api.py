@@ -172,9 +172,10 @@ def _is16(t: torch.Tensor) -> bool:
 
 
 def quantize(x: torch.Tensor, workspace: torch.Tensor, scale_in: torch.Tensor | None = None,
-             out: torch.Tensor | None = None, scale_out: torch.Tensor | None = None):
+             out: torch.Tensor | None = None, scale_out: torch.Tensor | None = None, flags: int = 0):
     """fp8attn_quantize (bf16 input) / fp8attn_quantize_ex with FP8ATTN_INPUT_FP16 (fp16 input):
-    [B,H,rows,d] -> (e4m3 codes as uint8 [B,H,rows,d], fp32 scale [B,H])."""
+    [B,H,rows,d] -> (e4m3 codes as uint8 [B,H,rows,d], fp32 scale [B,H]).  ``flags``:
+    QKV_TWO_LAUNCHES, the form without waits."""
     B, H, rows, d = _dims(x)
     assert _is16(x)
     if out is None:
@@ -184,8 +185,10 @@ def quantize(x: torch.Tensor, workspace: torch.Tensor, scale_in: torch.Tensor | 
     if scale_in is not None:
         assert scale_in.dtype == torch.float32 and scale_in.is_contiguous() and scale_in.numel() == B * H
     if x.dtype == torch.float16:
+        flags |= INPUT_FP16
+    if flags:
         rc = load().fp8attn_quantize_ex(_ptr(x), B, H, rows, d, _ptr(scale_in), _ptr(out),
-                                        _ptr(scale_out), INPUT_FP16, _ptr(workspace),
+                                        _ptr(scale_out), int(flags), _ptr(workspace),
                                         workspace.numel(), _stream())
         _check("fp8attn_quantize_ex", rc)
         return out, scale_out

@@ -116,7 +116,7 @@ int fp8attn_quantize_ex(const void* x_bf16, int B, int H, int64_t rows, int d, c
                         size_t workspace_bytes_, void* cuda_stream) {
     int rc = check_shape(B, H, d);
     if (rc != FP8ATTN_OK) return rc;
-    if (flags & ~(uint32_t)FP8ATTN_INPUT_FP16) return FP8ATTN_ERR_INVALID_ARG;
+    if (flags & ~(uint32_t)(FP8ATTN_INPUT_FP16 | FP8ATTN_QKV_TWO_LAUNCHES)) return FP8ATTN_ERR_INVALID_ARG;
     if (rows < 0) return FP8ATTN_ERR_INVALID_ARG;
     if (rows > 0 && (!x_bf16 || !x_fp8)) return FP8ATTN_ERR_INVALID_ARG;
     if (!scale_in && !scale_out) return FP8ATTN_ERR_INVALID_ARG;

@@ -60,8 +60,11 @@ def test_one_pass_matches_two_launches(B, H, n, m, d, dtype, flags, stages):
             assert torch.equal(got[name], want[name]), name
             assert torch.equal(again[name], want[name]), name
         assert (api.quantize_stages(1, B, H, n, 0, d) != 0) == (n <= 65536)
-        code, scale = api.quantize(x[1], ws)
-        assert torch.equal(code, want["k8"]) and torch.equal(scale, want["sk"])
+        for extra in (0, api.QKV_TWO_LAUNCHES):
+            before = api.launch_count()
+            code, scale = api.quantize(x[1], ws, flags=extra)
+            assert not extra or api.launch_count() - before == 2
+            assert torch.equal(code, want["k8"]) and torch.equal(scale, want["sk"])
     assert api.last_device_status(ws) == (0, 0)
 
 
