@@ -94,7 +94,8 @@ int fp8attn_quantize_ex(const void* x_16bit, int B, int H, int64_t rows, int d,
  * 16-bit inputs total more than 48 MB (a small one first).  Its thread blocks (one
  * per SM) exchange the heads' maxima; they are launched cooperatively, so that all
  * are resident at once, and every wait is bounded (2 s), ending in
- * FP8ATTN_ERR_TIMEOUT in the workspace's status word.  Larger heads take two
+ * FP8ATTN_ERR_TIMEOUT in the workspace's status word.  Larger heads, and contexts that
+ * do not have all SMs of the device (where a cooperative launch is refused), take two
  * launches that do not wait (maximum; conversion), as do short train heads with more
  * than 128 KB of test rows that enter their maximum, and all calls with
  * FP8ATTN_QKV_TWO_LAUNCHES (the _ex call), e.g. of callers that share the GPU with

@@ -503,9 +503,11 @@ int launch_quantize_qkv(const void* q_train, const void* k, const void* v, const
     if (key_dest == nullptr) {
         const Form f = quantize_form(3, n_heads, elems_train, elems_test, flags, sms);
         if (f.kind == Form::kHeads) return half ? launch_heads<true>(f, b, status, stream) : launch_heads<false>(f, b, status, stream);
-        if (f.kind == Form::kStaged)
-            return half ? launch_staged<true>(f, b, status, counters, words, amax_bits, stream)
-                        : launch_staged<false>(f, b, status, counters, words, amax_bits, stream);
+        if (f.kind == Form::kStaged) {
+            const int rc = half ? launch_staged<true>(f, b, status, counters, words, amax_bits, stream)
+                                : launch_staged<false>(f, b, status, counters, words, amax_bits, stream);
+            if (rc != staged::kRefused) return rc;
+        }
     }
     const int64_t want = ((int64_t)sms * 16 + n_heads * 3 - 1) / (n_heads * 3);
     // (blocks for the train rows; more only where the test rows are many times as many: blocks with
@@ -569,8 +571,9 @@ int launch_quantize(const void* x_bf16, int64_t n_heads, int64_t elems_per_head,
             b.out[0] = static_cast<uint4*>(x_fp8);
             b.scale_out[0] = scale_out;
             if (f.kind == Form::kHeads) return half ? launch_heads<true>(f, b, status, stream) : launch_heads<false>(f, b, status, stream);
-            return half ? launch_staged<true>(f, b, status, counters, words, amax_bits, stream)
-                        : launch_staged<false>(f, b, status, counters, words, amax_bits, stream);
+            const int rc = half ? launch_staged<true>(f, b, status, counters, words, amax_bits, stream)
+                                : launch_staged<false>(f, b, status, counters, words, amax_bits, stream);
+            if (rc != staged::kRefused) return rc;
         }
     }
     if (scale_in == nullptr) {
@@ -608,7 +611,8 @@ int launch_quantize_timeout_selftest(const void* x_bf16, int64_t n_heads, int64_
     b.x[0] = static_cast<const uint4*>(x_bf16);
     b.out[0] = static_cast<uint4*>(x_fp8);
     b.scale_out[0] = scale_out;
-    return launch_staged<false, true>(f, b, status, counters, words, amax_bits, stream, wait_clocks);
+    const int rc = launch_staged<false, true>(f, b, status, counters, words, amax_bits, stream, wait_clocks);
+    return rc == staged::kRefused ? FP8ATTN_ERR_UNSUPPORTED : rc;
 }
 
 int quantize_stages(int tensors, int64_t n_heads, int64_t elems_train, int64_t elems_test, uint32_t flags, int sms) {

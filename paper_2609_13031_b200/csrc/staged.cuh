@@ -502,6 +502,10 @@ inline unsigned plan(Shape& a, int sms) {
     return (unsigned)grid;
 }
 
+// The device does not hold all blocks of a cooperative launch at once, as in a context that was given only
+// some of the SMs: nothing was launched that waits, the caller takes two passes.
+constexpr int kRefused = -1;
+
 template <bool kSelfTest, class Op>
 int launch(const Args<Op>& a, unsigned grid, cudaStream_t stream) {
     // (the opt-in to large dynamic shared memory is per device and context: set on every call)
@@ -521,9 +525,15 @@ int launch(const Args<Op>& a, unsigned grid, cudaStream_t stream) {
     cfg.numAttrs = 1;
     if (a.cleared) {
         clear_and_fetch_kernel<Op><<<grid, 32, 0, stream>>>(a);
+        if (cudaGetLastError() != cudaSuccess) return FP8ATTN_ERR_CUDA;
         count_launch();
     }
-    if (cudaLaunchKernelEx(&cfg, kernel, a) != cudaSuccess) return FP8ATTN_ERR_CUDA;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        cudaGetLastError();     // (reported here and nowhere else)
+        return kRefused;
+    }
+    if (e != cudaSuccess) return FP8ATTN_ERR_CUDA;
     count_launch();
     return FP8ATTN_OK;
 }
