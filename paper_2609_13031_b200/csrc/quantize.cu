@@ -1,7 +1,7 @@
 // Per-head absmax quantization of bf16 (or IEEE fp16) tensors to e4m3 (paper Eq. 2).
 //
 // Calls whose heads fit on chip take one pass: short heads a block each (quantize_heads_kernel), longer
-// ones all SMs together (staged.cuh, QuantizeOp below): 2 B read + 1 B written per element.  The others
+// ones all SMs together (staged.cuh): 2 B read + 1 B written per element.  The others
 // (heads of more than 16 MB, an order of the keys, scales given, or on request) take two HBM-bound kernels:
 //   absmax_kernel    max |x| per head, packed bf16x2 max, one atomicMax per block
 //   quantize_kernel  s = amax/448, y = x/s (IEEE fp32), cvt.rn.satfinite.e4m3x2
@@ -180,60 +180,6 @@ __global__ void __launch_bounds__(kThreads) quantize_batch_kernel(const QuantBat
                          b.row_dest[z], b.pairs_per_row_shift);
 }
 
-
-// The quantizer in one pass (staged.cuh): the reduction is the absmax, its result the scale.
-template <bool kHalf>
-struct QuantizeOp {
-    using Acc = uint32_t;       // bit pattern of max |x| in the 16-bit type, which orders like an integer
-    struct Static {};
-    using Result = Divisor;
-    static constexpr int kOutBytes = 8;     // per 16-byte input vector
-    // a published value is one word: tag << 16 | maximum
-    static constexpr Acc kLost = 0xffffffffu;   // published: no tag (tags are below 0xffff)
-
-    // thread `tid`'s part of `vecs` vectors
-    static __device__ __forceinline__ Acc reduce(const uint4* x, int vecs, int tid) {
-        typename In16<kHalf>::V2 m = In16<kHalf>::as2(0u);
-#pragma unroll 4
-        for (int i = tid; i < vecs; i += staged::kWorkers) m = absmax8<kHalf>(m, x[i]);
-        const uint32_t w = *reinterpret_cast<const uint32_t*>(&m);
-        return max(w & 0xffffu, w >> 16);
-    }
-    static __device__ __forceinline__ Acc combine(Acc a, Acc b) { return max(a, b); }
-    static __device__ __forceinline__ Acc shuffle(Acc v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
-    static __device__ __forceinline__ Acc warp_combine(Acc v) { return __reduce_max_sync(0xffffffffu, v); }
-    static __device__ __forceinline__ void merge(Acc* to, Acc v) { atomicMax(to, v); }
-    static __device__ __forceinline__ void publish(uint32_t* slots, uint32_t, uint32_t i, uint32_t tag, Acc v) {
-        *reinterpret_cast<volatile uint32_t*>(slots + i) = tag << 16 | v;
-    }
-    using Raw = uint32_t;
-    static __device__ __forceinline__ Raw load(const uint32_t* slots, uint32_t, uint32_t i) {
-        return *reinterpret_cast<const volatile uint32_t*>(slots + i);
-    }
-    static __device__ __forceinline__ bool tagged(Raw r, uint32_t tag) { return r >> 16 == tag; }
-    static __device__ __forceinline__ Acc value(Raw r) { return r & 0xffffu; }
-    static __device__ __forceinline__ Result result(const Static&, Acc v) { return divisor(head_scale(In16<kHalf>::lo(v))); }
-    static __device__ __forceinline__ float output(const Result& r) { return r.s; }
-    // positions [i0, i1); kFollows: the scale is another tensor's
-    template <bool kFollows>
-    static __device__ __forceinline__ void convert(const Static&, const staged::Segment<QuantizeOp>& seg, const uint4* x,
-                                                   uint32_t i0, uint32_t i1, int tid) {
-        constexpr uint32_t kStep = staged::kWorkers;
-        const Divisor dv = seg.result;
-        uint2* o = reinterpret_cast<uint2*>(seg.out);
-        if (dv.direct) {
-            for (uint32_t i = i0 + tid; i < i1; i += kStep) o[i] = quant8_direct<kHalf>(x[i], dv);
-            return;
-        }
-        uint32_t i = i0 + tid;
-        for (; i + kStep < i1; i += 2 * kStep) {    // two vectors under way at a time
-            const uint4 v0 = x[i], v1 = x[i + kStep];
-            o[i] = quant8<kHalf, kFollows>(v0, dv);
-            o[i + kStep] = quant8<kHalf, kFollows>(v1, dv);
-        }
-        if (i < i1) o[i] = quant8<kHalf, kFollows>(x[i], dv);
-    }
-};
 
 // Calls of more than this many 16-bit input bytes clear their words in a launch of their own first
 // (which also starts on the data); smaller ones rely on what the last call left.
@@ -444,7 +390,7 @@ int launch_heads(const Form& f, const QuantBatch& b, const uint32_t* status, cud
 template <bool kHalf, bool kSelfTest = false>
 int launch_staged(const Form& f, const QuantBatch& b, uint32_t* status, uint32_t* counters, uint32_t* words,
                   uint32_t* amax_bits, cudaStream_t stream, int64_t wait_clocks = 0) {
-    staged::Args<QuantizeOp<kHalf>> a = {};
+    staged::Args a = {};
     static_cast<staged::Shape&>(a) = f.shape;
     for (int z = 0; z < a.tensors; ++z) {
         a.x[z] = b.x[z];
@@ -459,7 +405,7 @@ int launch_staged(const Form& f, const QuantBatch& b, uint32_t* status, uint32_t
     a.counter = counters;
     a.slots = words;
     a.heads = a.cleared ? amax_bits : words + a.sets * a.slots_per_set;
-    return staged::launch<kSelfTest>(a, f.grid, stream);
+    return staged::launch<kHalf, kSelfTest>(a, f.grid, stream);
 }
 
 }  // namespace

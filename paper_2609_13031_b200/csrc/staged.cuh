@@ -1,6 +1,5 @@
-// One pass over tensors whose every element needs a reduction over its whole head first (the
-// absmax of the quantizer, the sum of squares of the perturbation): an element crosses the HBM
-// interface once on its way in and once on its way out.
+// The quantizer in one pass for heads that a block cannot hold by itself: an element crosses the HBM
+// interface once on its way in and once on its way out, although its head's maximum comes first.
 //
 // What bounds it: HBM.  Two kernels, one per pass, read every element twice (5 bytes per element
 // of the quantizer instead of 3), because a large call is more than L2 can hold between them.
@@ -33,6 +32,7 @@
 // Without the fetch to L2: 159 us.)
 #pragma once
 #include "common.h"
+#include "quantize_math.cuh"
 #include "sm100_ptx.cuh"
 
 namespace fp8attn {
@@ -45,7 +45,8 @@ constexpr int kWorkers = kThreads - 64;        // and one warp that issues the l
 constexpr int kBufVecs = 7088;                 // 16-byte vectors per buffer: a head of 65,536 x 128 over 148 SMs
 constexpr int kParts = 2;                      // a buffer is given up in halves
 constexpr size_t kSmemBytes = (size_t)2 * kBufVecs * 16;
-constexpr int kMaxSegments = 48;               // per share
+constexpr int kMinVecs = kBufVecs;             // heads are longer than that, so that ...
+constexpr int kMaxSegments = 2;                // ... a share is part of two at most
 constexpr int kMaxFollowHeads = 32;            // whose rows follow in one block, in calls that clear nothing first
 constexpr int64_t kWaitClocks = 4000000000ll;  // 2 s
 
@@ -65,7 +66,6 @@ struct Shape {
     int sets, last_set;
 };
 
-template <class Op>
 struct Args : Shape {
     const uint4* x[3];          // the tensors that are reduced: unit u is head u / tensors of tensor u % tensors
     void* out[3];
@@ -78,7 +78,6 @@ struct Args : Shape {
     uint32_t* counter;          // blocks done
     uint32_t* slots;            // published values
     uint32_t* heads;            // published results of tensor 0, for the rows that follow it
-    typename Op::Static op;
 };
 
 // the workers and the exchange warp (barrier 0 is __syncthreads)
@@ -123,19 +122,56 @@ struct Share {
     }
 };
 
+// A published value is one word: tag << 16 | maximum, the bit pattern of max |x| in the 16-bit type, which
+// orders like an integer.
+constexpr uint32_t kLost = 0xffffffffu;     // published: no tag (tags are below 0xffff)
+__device__ __forceinline__ void publish(uint32_t* word, uint32_t tag, uint32_t v) {
+    *reinterpret_cast<volatile uint32_t*>(word) = tag << 16 | v;
+}
+__device__ __forceinline__ uint32_t peek(const uint32_t* word) { return *reinterpret_cast<const volatile uint32_t*>(word); }
+__device__ __forceinline__ bool tagged(uint32_t word, uint32_t tag) { return word >> 16 == tag; }
+__device__ __forceinline__ uint32_t value(uint32_t word) { return word & 0xffffu; }
+
 // What the conversion needs to know about a segment.
-template <class Op>
 struct Segment {
-    typename Op::Result result;
+    Divisor divisor;
     uint8_t* out;               // where position 0 of the share would go
     uint32_t begin, end;        // positions
     uint32_t head;
     int32_t at;                 // vector of the unit = position + at
 };
 
+// thread `tid`'s part of max |x| over `vecs` vectors
+template <bool kHalf>
+__device__ __forceinline__ uint32_t reduce(const uint4* x, int vecs, int tid) {
+    typename In16<kHalf>::V2 m = In16<kHalf>::as2(0u);
+#pragma unroll 4
+    for (int i = tid; i < vecs; i += kWorkers) m = absmax8<kHalf>(m, x[i]);
+    const uint32_t w = *reinterpret_cast<const uint32_t*>(&m);
+    return max(w & 0xffffu, w >> 16);
+}
+// positions [i0, i1) of a segment; kFollows: the scale is another tensor's
+template <bool kHalf, bool kFollows>
+__device__ __forceinline__ void convert(const Segment& seg, const uint4* x, uint32_t i0, uint32_t i1, int tid) {
+    constexpr uint32_t kStep = kWorkers;
+    const Divisor dv = seg.divisor;
+    uint2* o = reinterpret_cast<uint2*>(seg.out);
+    if (dv.direct) {
+        for (uint32_t i = i0 + tid; i < i1; i += kStep) o[i] = quant8_direct<kHalf>(x[i], dv);
+        return;
+    }
+    uint32_t i = i0 + tid;
+    for (; i + kStep < i1; i += 2 * kStep) {    // two vectors under way at a time
+        const uint4 v0 = x[i], v1 = x[i + kStep];
+        o[i] = quant8<kHalf, kFollows>(v0, dv);
+        o[i + kStep] = quant8<kHalf, kFollows>(v1, dv);
+    }
+    if (i < i1) o[i] = quant8<kHalf, kFollows>(x[i], dv);
+}
+
 // every contiguous piece of half `part` of a share: to(first position, source, vectors)
-template <class Op, class To>
-__device__ __forceinline__ void half_share(const Args<Op>& a, const Share& s, int stage, uint32_t part, To to) {
+template <class To>
+__device__ __forceinline__ void half_share(const Args& a, const Share& s, int stage, uint32_t part, To to) {
     const uint32_t vecs = (uint32_t)a.vecs, tensors = (uint32_t)a.tensors;
     const uint32_t u0 = (uint32_t)(stage * a.stage_units) + s.unit;
     const uint32_t p0 = part == 0 ? 0 : s.half(), p1 = part == 0 ? s.half() : s.n;
@@ -149,8 +185,7 @@ __device__ __forceinline__ void half_share(const Args<Op>& a, const Share& s, in
 
 // A launch of its own before large calls: clears the words and has the first stage fetched to L2
 // meanwhile (the launch then costs nothing).  One warp per block, the grid of staged_kernel.
-template <class Op>
-__global__ void clear_and_fetch_kernel(const __grid_constant__ Args<Op> a) {
+__global__ void clear_and_fetch_kernel(const __grid_constant__ Args a) {
     const Share s((uint32_t)min(a.stage_units, a.units), (uint32_t)a.vecs);
     if (threadIdx.x == 0)
         for (uint32_t part = 0; part < kParts; ++part)
@@ -164,15 +199,15 @@ __global__ void clear_and_fetch_kernel(const __grid_constant__ Args<Op> a) {
 // kSelfTest: waits end after a.wait_clocks.  (A limit and checks that only an expired wait needs stay out of
 // the exchange's path in all other calls: a variable limit and a look at `lost` before a share is published
 // cost 0.4 us a stage, 89 -> 96 us for 16 heads of 20,011 + 3,001 x 128.)
-template <class Op, bool kSelfTest>
-__global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_constant__ Args<Op> a) {
+template <bool kHalf, bool kSelfTest>
+__global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_constant__ Args a) {
     const int64_t limit = kSelfTest ? a.wait_clocks : kWaitClocks;
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ uint64_t full[2], known[2], part_free[2][kParts];
-    __shared__ typename Op::Acc seg_acc[kMaxSegments];
-    __shared__ Segment<Op> segment[2][kMaxSegments];
+    __shared__ uint32_t seg_acc[kMaxSegments];
+    __shared__ Segment segment[2][kMaxSegments];
     __shared__ uint16_t holders[kMaxSegments][2];       // first and last block of every segment's unit
-    __shared__ typename Op::Acc follow_acc[kMaxFollowHeads];
+    __shared__ uint32_t follow_acc[kMaxFollowHeads];
     __shared__ volatile int lost, give_up;
     static_assert(kSmemBytes + sizeof(segment) + sizeof(seg_acc) + sizeof(follow_acc) + 768 <= 232448, "shared memory of a block");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -187,7 +222,7 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
         fence_mbar_init();
         lost = give_up = 0;
     }
-    if (tid < kMaxSegments) seg_acc[tid] = typename Op::Acc(0);
+    if (tid < kMaxSegments) seg_acc[tid] = 0u;
     // rows that follow tensor 0 without counting are converted last, an equal share of them per block;
     // those of a small call are on their way to L2 from the start
     uint32_t f_lo = 0, f_hi = 0;
@@ -271,54 +306,53 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
             sync_exchange();        // A: the share is reduced
             // (block b and unit u of the stage meet at most once, and b + u names the meeting)
             for (uint32_t g = lane; g < s.segs; g += 32) {
-                Op::publish(slots, a.slots_per_set, blockIdx.x + s.unit + g, tag, seg_acc[g]);
-                seg_acc[g] = typename Op::Acc(0);
+                publish(slots + blockIdx.x + s.unit + g, tag, seg_acc[g]);
+                seg_acc[g] = 0u;
             }
             __syncwarp();
-            // Collect the values of this share's units: `width` lanes per segment (where a share has
-            // more than four segments, its units span two blocks at most).
-            const uint32_t width = s.segs <= 1 ? 32 : s.segs == 2 ? 16 : s.segs <= 4 ? 8 : 1;
+            // Collect the values of this share's units: `width` lanes per segment.
+            const uint32_t width = s.segs <= 1 ? 32 : 16;
             const bool none_empty = s.total >= 8 * gridDim.x;
             bool there = !lost && !pending;
             const int64_t t0 = clock64();
             for (uint32_t g0 = 0; g0 < s.segs; g0 += 32 / width) {
                 const uint32_t g = g0 + lane / width;
-                typename Op::Acc v = typename Op::Acc(0);
+                uint32_t v = 0u;
                 if (g < s.segs) {
                     constexpr int kBatch = 5;       // polls under way at a time: 148 blocks at 32 a row
                     const uint32_t u = s.unit + g, b1 = holders[g][1];
                     for (uint32_t b0 = holders[g][0] + lane % width; b0 <= b1; b0 += kBatch * width) {
-                        typename Op::Raw raw[kBatch];
+                        uint32_t raw[kBatch];
                         for (bool all = false; there && !all;) {
 #pragma unroll
-                            for (int k = 0; k < kBatch; ++k) raw[k] = Op::load(slots, a.slots_per_set, min(b0 + k * width, b1) + u);
+                            for (int k = 0; k < kBatch; ++k) raw[k] = peek(slots + min(b0 + k * width, b1) + u);
                             all = true;
 #pragma unroll
                             for (int k = 0; k < kBatch; ++k) {
                                 const uint32_t b = min(b0 + k * width, b1);
-                                all &= Op::tagged(raw[k], tag) || (!none_empty && cut(s.total, b) == cut(s.total, b + 1));
+                                all &= tagged(raw[k], tag) || (!none_empty && cut(s.total, b) == cut(s.total, b + 1));
                             }
                             if (!all) there = !lost && clock64() - t0 < limit;
                         }
 #pragma unroll
                         for (int k = 0; k < kBatch; ++k)
-                            if (b0 + k * width <= b1 && there && Op::tagged(raw[k], tag)) v = Op::combine(v, Op::value(raw[k]));
+                            if (b0 + k * width <= b1 && there && tagged(raw[k], tag)) v = max(v, value(raw[k]));
                     }
                 }
                 __syncwarp();
-                for (uint32_t o = width >> 1; o > 0; o >>= 1) v = Op::combine(v, Op::shuffle(v, o));
+                for (uint32_t o = width >> 1; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
                 if (g < s.segs && lane % width == 0) {
                     const uint32_t unit = u0 + g, head = unit / tensors, z = unit - head * tensors;
-                    Segment<Op>& seg = segment[stage & 1][g];
-                    seg.result = Op::result(a.op, v);
+                    Segment& seg = segment[stage & 1][g];
+                    seg.divisor = divisor(head_scale(In16<kHalf>::lo(v)));
                     seg.begin = s.begin(g, vecs);
                     seg.end = s.end(g, vecs);
                     seg.head = head;
                     seg.at = (int32_t)(s.at(g) - seg.begin);
-                    seg.out = static_cast<uint8_t*>(a.out[z]) + ((int64_t)head * vecs + seg.at) * Op::kOutBytes;
+                    seg.out = static_cast<uint8_t*>(a.out[z]) + ((int64_t)head * vecs + seg.at) * 8;
                     if (there && (g > 0 || s.skip == 0)) {      // the unit begins here
-                        if (a.result_out[z] != nullptr) a.result_out[z][head] = Op::output(seg.result);
-                        if (z == 0 && a.follow_vecs > 0 && !a.follow_counts) Op::publish(a.heads, 0, head, 1, v);
+                        if (a.result_out[z] != nullptr) a.result_out[z][head] = seg.divisor.s;
+                        if (z == 0 && a.follow_vecs > 0 && !a.follow_counts) publish(a.heads + head, 1, v);
                     }
                 }
             }
@@ -337,12 +371,12 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
             bool there = true;
             if (h <= (f_hi - 1) / a.follow_vecs) {
                 const int64_t t0 = clock64();
-                typename Op::Raw raw = Op::load(a.heads, 0, h);
-                while (there && !Op::tagged(raw, 1)) {
+                uint32_t raw = peek(a.heads + h);
+                while (there && !tagged(raw, 1)) {
                     there = clock64() - t0 < limit;
-                    raw = Op::load(a.heads, 0, h);
+                    raw = peek(a.heads + h);
                 }
-                follow_acc[lane] = Op::value(raw);
+                follow_acc[lane] = value(raw);
             }
             if (!__all_sync(0xffffffffu, there) && lane == 0) {
                 timed_out();
@@ -376,14 +410,14 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
             f1 = (uint32_t)((uint64_t)(at + s.end(g, vecs) - s.begin(g, vecs)) * a.follow_vecs / vecs);
             return true;
         };
-        auto convert = [&](int stage, uint32_t part) {
+        auto convert_half = [&](int stage, uint32_t part) {
             const Share& s = stage + 1 < stages ? share_full : share_last;
             const uint4* buf = reinterpret_cast<const uint4*>(smem) + (stage & 1) * kBufVecs;
             const uint32_t p0 = part == 0 ? 0 : s.half(), p1 = part == 0 ? s.half() : s.n;
             for (uint32_t g = 0; g < s.segs; ++g) {
-                const Segment<Op>& seg = segment[stage & 1][g];
+                const Segment& seg = segment[stage & 1][g];
                 const uint32_t i0 = max(p0, seg.begin), i1 = min(p1, seg.end);
-                if (i0 < i1) Op::template convert<false>(a.op, seg, buf, i0, i1, tid);
+                if (i0 < i1) convert<kHalf, false>(seg, buf, i0, i1, tid);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&part_free[stage & 1][part]));
@@ -400,37 +434,37 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
                 }
                 if (!__all_sync(0xffffffffu, landed)) {     // what is published then bears no tag
                     lost = 1;
-                    for (uint32_t g = lane; g < s.segs; g += 32) Op::merge(&seg_acc[g], Op::kLost);
+                    for (uint32_t g = lane; g < s.segs; g += 32) atomicMax(&seg_acc[g], kLost);
                 }
                 for (uint32_t g = 0; g < s.segs; ++g) {
                     const uint32_t b = s.begin(g, vecs), e = s.end(g, vecs);
                     if (b + (tid & ~31) >= e && !a.follow_counts) continue;      // (whole warps)
-                    typename Op::Acc v = typename Op::Acc(0);
-                    if (b + tid < e) v = Op::reduce(buf + b, e - b, tid);
+                    uint32_t v = 0u;
+                    if (b + tid < e) v = reduce<kHalf>(buf + b, e - b, tid);
                     uint32_t head, f0, f1;
                     if (a.follow_counts && follow_range(s, g, (uint32_t)(stage * a.stage_units), head, f0, f1) && f0 + tid < f1)
-                        v = Op::combine(v, Op::reduce(a.follow_x + (int64_t)head * a.follow_vecs + f0, f1 - f0, tid));
-                    v = Op::warp_combine(v);
-                    if (lane == 0) Op::merge(&seg_acc[g], v);
+                        v = max(v, reduce<kHalf>(a.follow_x + (int64_t)head * a.follow_vecs + f0, f1 - f0, tid));
+                    v = __reduce_max_sync(0xffffffffu, v);
+                    if (lane == 0) atomicMax(&seg_acc[g], v);
                 }
                 sync_exchange();    // A
             }
             if (stage > 0) {
-                convert(stage - 1, 1);
+                convert_half(stage - 1, 1);
                 const Share& s = stage < stages ? share_full : share_last;
                 for (uint32_t g = 0; a.follow_counts && g < s.segs; ++g) {
-                    Segment<Op> seg = segment[(stage - 1) & 1][g];
+                    Segment seg = segment[(stage - 1) & 1][g];
                     uint32_t head, f0, f1;
                     if (!follow_range(s, g, (uint32_t)((stage - 1) * a.stage_units), head, f0, f1)) continue;
                     const int64_t first = (int64_t)head * a.follow_vecs;
-                    seg.out = static_cast<uint8_t*>(a.follow_out) + first * Op::kOutBytes;
-                    Op::template convert<true>(a.op, seg, a.follow_x + first, f0, f1, tid);
+                    seg.out = static_cast<uint8_t*>(a.follow_out) + first * 8;
+                    convert<kHalf, true>(seg, a.follow_x + first, f0, f1, tid);
                 }
             }
             if (stage < stages) {
                 sync_exchange();    // B
                 if (give_up) break;
-                convert(stage, 0);
+                convert_half(stage, 0);
             }
         }
     }
@@ -446,23 +480,23 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
     if (!give_up) {
         bool there = true;
         const int64_t t0 = clock64();
-        Segment<Op> seg;
+        Segment seg;
         seg.at = 0;
         seg.out = static_cast<uint8_t*>(a.follow_out);
         for (uint32_t x = f_lo; x < f_hi && there;) {
             seg.head = x / a.follow_vecs;
             const uint32_t end = f_hi - seg.head * a.follow_vecs < a.follow_vecs ? f_hi : (seg.head + 1) * a.follow_vecs;
-            typename Op::Acc v = follow_acc[a.cleared ? 0 : seg.head - f_lo / a.follow_vecs];
+            uint32_t v = follow_acc[a.cleared ? 0 : seg.head - f_lo / a.follow_vecs];
             if (a.cleared) {
-                typename Op::Raw raw = Op::load(a.heads, 0, seg.head);
-                while (there && !Op::tagged(raw, 1)) {
+                uint32_t raw = peek(a.heads + seg.head);
+                while (there && !tagged(raw, 1)) {
                     there = clock64() - t0 < limit;
-                    raw = Op::load(a.heads, 0, seg.head);
+                    raw = peek(a.heads + seg.head);
                 }
-                v = Op::value(raw);
+                v = value(raw);
             }
-            seg.result = Op::result(a.op, v);
-            if (there && tid < kWorkers) Op::template convert<true>(a.op, seg, a.follow_x, x, end, tid);
+            seg.divisor = divisor(head_scale(In16<kHalf>::lo(v)));
+            if (there && tid < kWorkers) convert<kHalf, true>(seg, a.follow_x, x, end, tid);
             x = end;
         }
         if (!there) timed_out();
@@ -470,10 +504,10 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
 }
 
 // Fills what plan() does not get (stage_units and everything behind it) and returns the grid, or 0 where
-// this path does not take the call: a unit that does not fit one buffer of every SM, heads so short that
-// a share would have too many segments, or more words than the workspace has for them.
+// this path does not take the call: a unit that does not fit one buffer of every SM or is no longer than a
+// share, or more words than the workspace has for them.
 inline unsigned plan(Shape& a, int sms) {
-    if (a.units <= 0 || a.vecs <= 0 || a.vecs % 8 != 0) return 0;     // (shares end on multiples of eight vectors)
+    if (a.units <= 0 || a.vecs <= kMinVecs || a.vecs % 8 != 0) return 0;     // (shares end on multiples of eight vectors)
     if ((uint64_t)a.follow_vecs * (uint64_t)(a.units / a.tensors) > 0x7fffffffull) return 0;
     // at least 8 KB per block, test rows included: with fewer blocks there is less to exchange, but all of
     // them share the test rows (1 head of 1,100 + 200,000 x 64 with the blocks that its train rows are worth:
@@ -488,8 +522,7 @@ inline unsigned plan(Shape& a, int sms) {
     int64_t stages = (a.units + fit - 1) / fit;
     a.stage_units = (int)((a.units + stages - 1) / stages);
     stages = (a.units + a.stage_units - 1) / a.stage_units;
-    const int64_t share = (a.stage_units * a.vecs + grid - 1) / grid + 7;
-    if (share / a.vecs + 2 > kMaxSegments || stages > 0xfff0) return 0;
+    if (stages > 0xfff0) return 0;
     a.stages = (int)stages;
     const bool shorter = stages > 2 && stages * a.stage_units != a.units;
     a.sets = shorter ? 3 : stages > 1 ? 2 : 1;
@@ -506,10 +539,10 @@ inline unsigned plan(Shape& a, int sms) {
 // some of the SMs: nothing was launched that waits, the caller takes two passes.
 constexpr int kRefused = -1;
 
-template <bool kSelfTest, class Op>
-int launch(const Args<Op>& a, unsigned grid, cudaStream_t stream) {
+template <bool kHalf, bool kSelfTest>
+int launch(const Args& a, unsigned grid, cudaStream_t stream) {
     // (the opt-in to large dynamic shared memory is per device and context: set on every call)
-    auto kernel = staged_kernel<Op, kSelfTest>;
+    auto kernel = staged_kernel<kHalf, kSelfTest>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) !=
         cudaSuccess)
         return FP8ATTN_ERR_CUDA;
@@ -524,7 +557,7 @@ int launch(const Args<Op>& a, unsigned grid, cudaStream_t stream) {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     if (a.cleared) {
-        clear_and_fetch_kernel<Op><<<grid, 32, 0, stream>>>(a);
+        clear_and_fetch_kernel<<<grid, 32, 0, stream>>>(a);
         if (cudaGetLastError() != cudaSuccess) return FP8ATTN_ERR_CUDA;
         count_launch();
     }
