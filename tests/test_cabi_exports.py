@@ -74,6 +74,16 @@ def test_quantizer_form_is_host_only_arithmetic():
         assert api.quantize_stages(tensors, 1, H, n, m, d, flags) == stages, (tensors, H, n, m, d, flags)
 
 
+def test_tiles_per_cta_of_split_launches():
+    """Both sides of the choice between two and three tiles for test rows against a table (d = 64)."""
+    api.load()
+    flags = api.SPLIT_TAIL | api.TEST_ROWS_ONLY
+    for H, n, m, rows in ((8, 4096, 2048, 256), (8, 8192, 2048, 256), (8, 30011, 2048, 384), (4, 30011, 2048, 384),
+                          (8, 131072, 700, 384), (8, 262144, 300, 384), (2, 131072, 300, 256), (16, 8192, 700, 256)):
+        assert api.attention_rows_per_cta(1, H, n, m, 64, flags) == rows, (H, n, m)
+    assert api.attention_rows_per_cta(1, 8, 30011, 2048, 64, api.TEST_ROWS_ONLY) == 256
+
+
 def test_dispatch_gate_matches_the_paper_constant():
     import os
     from helpers import read_golden_table

@@ -115,9 +115,9 @@ def test_argument_errors_are_reported_on_the_host():
                                       ("C5", 1, 0)])
 def test_fused_qkv_quantize_matches_oracle(cfg, n, m):
     """fp8attn_quantize_qkv is bit-identical to the oracle, including the shared train-query
-    scale for the test queries: as one launch (these sizes are small calls), and as two launches
-    when asked for.  Twice in a row on one workspace: the one-launch path must leave its
-    counters clean."""
+    scale for the test queries: as one launch (these sizes are small calls: a block per head, or one
+    pass in stages), and as two launches when asked for.  Twice in a row on one workspace: the
+    one-pass form must leave its words clean."""
     w = W.CONFIGS[cfg].scaled(n, m)
     g = W.generate(w)
     ws = api.new_workspace(w.B, w.H)
@@ -180,8 +180,8 @@ def test_fused_qkv_query_scale_from_all_rows(extra):
 
 @pytest.mark.parametrize("scale", [1e-38, 3e-31, 1e-30, 7.3e-12, 1.0, 6.5e11, 1e30, 3e30, 2.9e38])
 def test_given_scales_across_the_exponent_range(scale):
-    """A given scale anywhere in the fp32 range (the conversion takes its quotients from a
-    per-mantissa table inside a safe scale range and divides per element outside it): codes
+    """A given scale anywhere in the fp32 range (the conversion multiplies and corrects inside a safe
+    scale range and divides per element outside it): codes
     equal the oracle's, for inputs that span the whole bf16 exponent range, subnormals, zeros
     and both signs included."""
     rng = np.random.default_rng(17)
