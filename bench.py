@@ -317,8 +317,8 @@ def main():
         buf["key_dest"] = torch.empty((w.B, w.H, w.n_train), dtype=torch.int32, device="cuda")
 
     def quantize_all():
-        # all four quantizations (Q_train, K, V with their own scales; Q_test with Q_train's) in two
-        # launches; with the key order, two more small launches and K8, V8 written in that order
+        # all four quantizations (Q_train, K, V with their own scales; Q_test with Q_train's), one pass in
+        # two launches; with the key order, maximum, order and conversion, K8 and V8 in that order
         api.quantize_qkv(dev["q_train"], dev["k"], dev["v"], dev["q_test"], ws, out=buf, order_keys=order_keys)
 
     # the 16-bit comparison kernel runs on K, V in the same key order (reordered once, outside its timing)

@@ -215,8 +215,8 @@ def quantize_noalloc(x: torch.Tensor, out: torch.Tensor, scale_out: torch.Tensor
 
 
 def quantize_qkv(q_train, k, v, q_test, workspace, out=None, flags: int = 0, order_keys: bool = False):
-    """fp8attn_quantize_qkv: all four quantizations of one attention call in two
-    launches.  Returns dict(q8, k8, v8, t8, sq, sk, sv); ``out`` may supply those
+    """fp8attn_quantize_qkv: all four quantizations of one attention call, in one or two
+    launches (``quantize_stages``).  Returns dict(q8, k8, v8, t8, sq, sk, sv); ``out`` may supply those
     tensors preallocated.  With SCALES_GIVEN, ``out`` must hold sq, sk, sv and they
     are read instead of written (one launch).  ``order_keys``:
     fp8attn_quantize_qkv_ordered, K8 and V8 come out with the keys of largest norm first and

@@ -986,8 +986,8 @@ int launch_d64(const AttnParams& p, cudaStream_t stream) {
 //  - Three where the grid of 384-row blocks fills the SMs at least eight times over: there the last,
 //    partly filled round no longer matters, and three softmax warps per scheduler are 4 % faster.
 //  - With FP8ATTN_SPLIT_TAIL, three from eight rounds of 256-row blocks on, where the split of
-//    two-tile launches ends: it takes care of the last round of these too (8 heads of 32,768 + 8,192
-//    rows, bf16: 3.27 -> 3.17 ms).
+//    two-tile launches ends: it takes care of the last round of these too (8 heads of 30,011 + 8,000 to
+//    45,000 + 11,000 rows: FP8 0.89 .. 0.97 of the time, bf16 0.94 .. 0.98, fp16 0.93 .. 1.00).
 //  - With FP8ATTN_SPLIT_TAIL, for a launch of less than one round (a few test rows against a long
 //    table, above all), whichever gives the shorter critical path: a block of T tiles takes kCost[T - 1]
 //    per key, the more blocks there are the fewer key ranges each is split into, and every range of a row is

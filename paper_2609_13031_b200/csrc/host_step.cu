@@ -100,8 +100,8 @@ extern "C" int fp8attn_icl_step_host(const void* q_train, const void* k, const v
         device_scratch_bytes < p.set_bytes * (size_t)p.sets)
         return FP8ATTN_ERR_WORKSPACE;
     cudaStream_t user = static_cast<cudaStream_t>(cuda_stream);
-    // the two-launch quantizer: host steps of different streams may share the GPU, and the blocks
-    // of the one-launch form wait for one another
+    // the two-launch quantizer: host steps of different streams share the GPU, and the one-pass form needs
+    // every SM free at once
     const uint32_t qflags = FP8ATTN_QKV_TWO_LAUNCHES | ((flags & FP8ATTN_HOST_FP16) ? FP8ATTN_INPUT_FP16 : 0u);
     const uint32_t fflags = FP8ATTN_SPLIT_TAIL | ((flags & FP8ATTN_HOST_FP16) ? FP8ATTN_IO_FP16 : 0u);
 

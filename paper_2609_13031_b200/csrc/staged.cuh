@@ -23,10 +23,10 @@
 // the next call, while the workers convert.  (At the end of the kernel the fence that orders this waits
 // for the block's output stores: 1 us a call.)
 //
-// Measured, quantizer, 8 heads of 65,536 + 16,384 rows x 128 (654 MB in and out, 100 us at the copy
-// rate): 128 us, two passes 182 us; 16 heads of 30,011 x 64 62.6 / 89.1 us; 8 heads of 20,011 + 3,001 x
-// 128 57.0 / 55.7 us; 8,192 + 2,048 x 64 17.4 / 20.3 us.  About 10 us go before the second stage:
-// launch, the first stage's way in, and its exchange under the second's loads.
+// Measured, graph-replayed, one pass / two passes: 8 heads of 65,536 + 16,384 rows x 128 (654 MB in and
+// out, 100 us at the copy rate) 126-130 / 183 us; x 64 72 / 94 us; 16 heads of 20,011 + 3,001 x 128 92-97 / 115 us;
+// 8 heads 52-57 / 56 us; 8,192 + 2,048 x 64 15.8 / 20.5 us.  About 10 us go before the second stage: launch,
+// the first stage's way in, and its exchange under the second's loads.
 // (Tried before: 24 KB chunks handed out by tickets to a control thread and worker warps: 2.5 us per
 // chunk for the hand-overs.  Accumulators and a grid-wide counter instead of tagged words: 154 us.
 // Without the fetch to L2: 159 us.)
@@ -191,9 +191,9 @@ __global__ void clear_and_fetch_kernel(const __grid_constant__ Args a) {
         for (uint32_t part = 0; part < kParts; ++part)
             half_share(a, s, 0, part, [](uint32_t, const uint4* src, uint32_t n) { bulk_prefetch(src, n * 16); });
     const uint32_t t = blockIdx.x * 32 + threadIdx.x, threads = gridDim.x * 32;
-    for (uint32_t i = t; i < a.sets * a.slots_per_set ; i += threads) a.slots[i] = 0u;
+    for (uint32_t i = t; i < a.sets * a.slots_per_set; i += threads) a.slots[i] = 0u;
     if (a.follow_vecs > 0)
-        for (uint32_t i = t; i < (uint32_t)(a.units / a.tensors) ; i += threads) a.heads[i] = 0u;
+        for (uint32_t i = t; i < (uint32_t)(a.units / a.tensors); i += threads) a.heads[i] = 0u;
 }
 
 // kSelfTest: waits end after a.wait_clocks.  (A limit and checks that only an expired wait needs stay out of
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
             const Share& s = stage + 1 < stages ? share_full : share_last;
             const uint32_t u0 = (uint32_t)(stage * a.stage_units) + s.unit;
             uint32_t* const slots =
-                a.slots + (stage + 1 == stages ? a.last_set : stage & 1) * a.slots_per_set ;
+                a.slots + (stage + 1 == stages ? a.last_set : stage & 1) * a.slots_per_set;
             const uint32_t tag = (uint32_t)stage + 1;
             if (stage == 0 || (stage + 1 == stages && share_last.total != share_full.total)) {
                 for (uint32_t g = lane; g < s.segs; g += 32) {
