@@ -230,8 +230,8 @@ int bf16attn_icl_forward(const void* q_train, const void* q_test, const void* k,
  * outputs of bf16attn_icl_forward_ex (which then is an fp16 kernel).
  *
  * FP8ATTN_SPLIT_TAIL balances the last, partly filled round of the launch.  The
- * grid is one CTA per 256 query rows of a head (384 in some launches at d = 64, see
- * fp8attn_attention_rows_per_cta); when the number of CTAs is not
+ * grid is one CTA per 256 query rows of a head (384 in some launches at d = 64, 128 in small
+ * ones, see fp8attn_attention_rows_per_cta); when the number of CTAs is not
  * a multiple of the number of SMs, the CTAs left over after the last full
  * round would run alone on a fraction of the GPU.  With this flag each of them
  * is replaced by up to 40 CTAs that share its query rows and divide the train
@@ -279,7 +279,9 @@ int fp8attn_gate_use_fp8(int64_t n_train);
  * one CTA of the forward calls takes for a call of these sizes and flags on the current
  * device: 256 (two 128-row tiles), or 384 (three) at d = 64 when the grid of 384-row
  * blocks fills the SMs at least eight times over or, with FP8ATTN_SPLIT_TAIL, when that of
- * 256-row blocks does or when a launch of less than one round is over sooner that way.
+ * 256-row blocks does or when a launch of less than one round is over sooner that way,
+ * or 128 (one) up to 16,384 train rows when even the grid of 128-row blocks leaves SMs
+ * free and the keys are not split instead.
  * Without a device the SM count of a B200 (148) is assumed.  0 for unsupported sizes.
  * Results do not depend on it beyond the order of the online softmax (steps of 128 or 96
  * keys). */

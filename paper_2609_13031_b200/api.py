@@ -299,7 +299,7 @@ def selftest_quantize_timeout(x: torch.Tensor, workspace: torch.Tensor, out: tor
 
 
 def attention_rows_per_cta(B: int, H: int, n_train: int, n_test: int, d: int, flags: int = 0) -> int:
-    """fp8attn_attention_rows_per_cta: 256 or 384 query rows per CTA for a call of these sizes."""
+    """fp8attn_attention_rows_per_cta: 128, 256 or 384 query rows per CTA for a call of these sizes."""
     return int(load().fp8attn_attention_rows_per_cta(B, H, n_train, n_test, d, int(flags)))
 
 

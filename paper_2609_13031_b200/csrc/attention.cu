@@ -1,7 +1,7 @@
 // Fused ICL attention for sm_100a: train->train and test->train in one launch.
 //
 // One CTA owns the query rows of up to T 128-row tiles of one (b,h) (T = 3 at d = 64, 2 at
-// d = 128) and walks over all train keys in steps of kKeys keys.  Warp roles:
+// d = 128, 1 in small launches) and walks over all train keys in steps of kKeys keys.  Warp roles:
 //   warps 4t .. 4t+3   softmax of query tile t, one row per thread
 //   warp  4T           issues the Q K^T tcgen05.mma of all tiles (one elected lane)
 //   warp  4T+1         TMA producer for Q, K and V tiles
@@ -37,7 +37,8 @@ constexpr int kTileM = 128;           // query rows per tile
 // Query tiles per CTA (kT): two, or at d = 64 three for launches of many rounds (tensor memory
 // holds 512 columns and every tile's O takes d of them).  Three tiles put a third softmax warp
 // on every scheduler, at the price of a smaller register budget per thread (96-key steps) and
-// coarser blocks (384 rows), which small grids pay for in their last round.  Warps: four
+// coarser blocks (384 rows), which small grids pay for in their last round.  One tile where even that
+// many CTAs fit on the SMs at once: a step of one tile takes 1.1 us, of two 1.45 us.  Warps: four
 // softmax warps per tile, then the Q K^T issuer, the TMA producer and two P V issuers (tiles
 // {0, 2} and {1}).
 template <int kT> constexpr int kRowsPerBlock = kT * kTileM;
@@ -48,6 +49,7 @@ template <int kT> constexpr int kNumThreads = (4 * kT + 4) * 32;
 template <int kT> constexpr int kLaunchRegs = kT == 3 ? 128 : 168;
 template <int kT> constexpr int kRegsSoftmax = kT == 3 ? 152 : 224;
 constexpr int kRegsOther = 56;
+// (one tile: no more than 255 registers for 256 threads, nothing to redistribute)
 template <int kT> constexpr bool kRegsFit =
     4 * kT * 32 * kRegsSoftmax<kT> + 4 * 32 * kRegsOther <= kNumThreads<kT> * kLaunchRegs<kT>;
 static_assert(kRegsFit<2> && kRegsFit<3>, "setmaxnreg budgets exceed the CTA's register pool");
@@ -70,7 +72,7 @@ enum : uint32_t {
 // d = 64 through register allocation, hence a template parameter.)
 template <bool kFp8, int kD, bool kHalf, int kT>
 struct Cfg {
-    static_assert(kT == 2 || (kT == 3 && kD == 64), "tiles per CTA");
+    static_assert(kT == 1 || kT == 2 || (kT == 3 && kD == 64), "tiles per CTA");
     static constexpr int kES = kFp8 ? 1 : 2;                    // element bytes
     static constexpr int kRowBytes = kD * kES;
     static constexpr int kBoxBytes = kRowBytes > 128 ? 128 : kRowBytes;  // swizzle span
@@ -100,9 +102,9 @@ struct Cfg {
     // 3.6 % more time; P written over S, where Q K^T has to wait for P V: the 16-bit kernel
     // took 10 % more time and 20 % more cycles that way.)
     // 16 bits, d = 64, two tiles: room for two P buffers per tile as well (S | 2 x 2 x 64 | O0 | O1).
-    // (8 heads of 8,192 + 2,048 rows 236 -> 228 us)
-    static constexpr bool kRoomy = !kFp8 && kD == 64 && kT == 2;
-    static constexpr uint32_t kColS = 0, kColO = kRoomy ? 384 : 256;
+    // (8 heads of 8,192 + 2,048 rows 236 -> 228 us)  One tile: the same without the second (S | 2 x 64 | O).
+    static constexpr bool kRoomy = !kFp8 && (kT == 1 || (kD == 64 && kT == 2));
+    static constexpr uint32_t kColS = 0, kColO = kRoomy && kT == 2 ? 384 : 256;
     static constexpr uint32_t kColP0 = kKeys, kPStride = kRoomy ? 128 : kKeys / 2;   // P_t at kColP0 + t*kPStride
     // P alternates between two buffers per tile (the second kPCols columns after the first) where
     // there is room, so that writing P of one step never waits for the P V of the step before.
@@ -111,7 +113,10 @@ struct Cfg {
     static constexpr int kPolyPer16 = kFp8 ? (kT == 3 ? 2 : 4) : 2;
     static_assert(kPBufs * kPCols <= (int)kPStride, "TMEM layout: P tiles overlap");
     static_assert(kColP0 + kTiles * kPStride <= kColO && kColO + kTiles * kD <= 512, "TMEM layout");
-    static constexpr size_t kSmemBytes = (size_t)kTiles * kQTileBytes + (size_t)2 * kStages * kKVTileBytes + 1024;
+    static constexpr size_t kSmemUsed = (size_t)kTiles * kQTileBytes + (size_t)2 * kStages * kKVTileBytes + 1024;
+    // One CTA per SM, since it takes all of the tensor memory and a second one would wait for it: with two or
+    // three tiles the register file sees to that, with one it asks for more than half of the shared memory.
+    static constexpr size_t kSmemBytes = kT == 1 && kSmemUsed < 120 * 1024 ? 120 * 1024 : kSmemUsed;
 };
 
 struct Barriers {
@@ -415,7 +420,7 @@ icl_attention_kernel(const __grid_constant__ CUtensorMap map_q_train,
     Waiter w{args.status, false};
 
     if (warp == kTmaWarp) {
-        setmaxnreg_dec<kRegsOther>();
+        if (kT > 1) setmaxnreg_dec<kRegsOther>();
         // =========================== TMA producer ===========================
         // The whole warp walks the loop (waits included); one elected lane issues.
         if (elect_one()) {
@@ -454,7 +459,7 @@ icl_attention_kernel(const __grid_constant__ CUtensorMap map_q_train,
             }
         }
     } else if (warp == kQkWarp) {
-        setmaxnreg_dec<kRegsOther>();
+        if (kT > 1) setmaxnreg_dec<kRegsOther>();
         // ====================== Q K^T issuer (all query tiles) ======================
         // The whole warp walks the loop (waits included); one elected lane issues the
         // MMAs and commits.  Q K^T and P V are issued from different warps because one
@@ -511,7 +516,7 @@ icl_attention_kernel(const __grid_constant__ CUtensorMap map_q_train,
             __syncwarp();
         }
     } else if (warp >= kPvWarp0) {
-        setmaxnreg_dec<kRegsOther>();
+        if (kT > 1) setmaxnreg_dec<kRegsOther>();
         // ============ P V issuers: the first takes tiles 0 and 2, the second tile 1 ============
         // (the tiles' P become ready in the order of the rotation, so the tiles of one issuer
         // never wait for each other)
@@ -543,7 +548,7 @@ icl_attention_kernel(const __grid_constant__ CUtensorMap map_q_train,
         }
     } else {
         // ========================= softmax + epilogue =========================
-        setmaxnreg_inc<kRegsSoftmax<kT>>();
+        if (kT > 1) setmaxnreg_inc<kRegsSoftmax<kT>>();
         const int t = warp >> 2;                       // query tile
         if (t < ntiles) {
             const int row_in_tile = (warp & 3) * 32 + lane;
@@ -882,7 +887,7 @@ int launch(const AttnParams& p, cudaStream_t stream) {
     a.splits = 1;
     a.partial = nullptr;
     int units = 0, sms = 0;
-    if ((p.flags & FP8ATTN_SPLIT_TAIL) && p.partial != nullptr) {
+    if (kT > 1 && (p.flags & FP8ATTN_SPLIT_TAIL) && p.partial != nullptr) {
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
             return FP8ATTN_ERR_CUDA;
         const int64_t full = (grid / sms) * sms, left = grid - full;
@@ -906,7 +911,7 @@ int launch(const AttnParams& p, cudaStream_t stream) {
         }
     }
     auto kern = icl_attention_kernel<kFp8, kD, kHalf, kT, false>;
-    auto kern_split = icl_attention_kernel<kFp8, kD, kHalf, kT, true>;
+    auto kern_split = icl_attention_kernel<kFp8, kD, kHalf, kT == 1 ? 2 : kT, true>;     // (one tile: never split)
     // The opt-in to large dynamic shared memory is per device and per context; it is set on
     // every call (a cached flag would go stale when the context is destroyed).
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemBytes) !=
@@ -972,15 +977,26 @@ int launch_wait_timeout_selftest(uint32_t* status, uint64_t limit_ns, cudaStream
 }
 
 template <bool kFp8, bool kHalf>
-int launch_d64(const AttnParams& p, cudaStream_t stream) {
+int launch_tiles(const AttnParams& p, cudaStream_t stream) {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
         return FP8ATTN_ERR_CUDA;
-    if (attention_rows_per_cta(p.B, p.H, p.n_train, p.n_test, 64, p.flags, sms, p.partial_bytes) == kRowsPerBlock<3>)
-        return launch<kFp8, 64, kHalf, 3>(p, stream);
+    const int rows = attention_rows_per_cta(p.B, p.H, p.n_train, p.n_test, p.d, p.flags, sms, p.partial_bytes);
+    if (p.d == 128)
+        return rows == kRowsPerBlock<1> ? launch<kFp8, 128, kHalf, 1>(p, stream) : launch<kFp8, 128, kHalf, 2>(p, stream);
+    if (rows == kRowsPerBlock<1>) return launch<kFp8, 64, kHalf, 1>(p, stream);
+    if (rows == kRowsPerBlock<3>) return launch<kFp8, 64, kHalf, 3>(p, stream);
     return launch<kFp8, 64, kHalf, 2>(p, stream);
 }
+
+// One tile per CTA where all of a launch's tiles fit on the SMs at once and its keys are not split instead: the
+// CTA's steps are what the launch takes.  The same results bit for bit as with two tiles (a tile's rows see the
+// same keys in the same steps), so the choice may depend on the number of test rows.  Two tiles / one: 2 heads of
+// 512 + 128 x 64 10.1 / 8.1 us; 8 heads of 1,024 + 256 x 64 16.2 / 13.0, x 128 18.6 / 14.4 (bf16 20.3 / 15.3);
+// 2 heads of 8,192 + 1,000 x 128 101 / 77 (bf16 112 / 81); 1 head of 16,000 + 2,000 x 64 174 / 137.  Up to
+// kOneTileKeys keys, as measured: every K and V tile is fetched for half as many rows.
+constexpr int64_t kOneTileKeys = 16384;
 
 // d = 64: two or three tiles per CTA.
 //  - Three where the grid of 384-row blocks fills the SMs at least eight times over: there the last,
@@ -997,10 +1013,12 @@ int launch_d64(const AttnParams& p, cudaStream_t stream) {
 //  - Two otherwise (small grids pay for coarse blocks in their last round).
 int attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d, uint32_t flags, int sms,
                            size_t partial_bytes) {
-    if (d != 64) return kRowsPerBlock<2>;
     const int64_t heads = (int64_t)B * H, train = (flags & FP8ATTN_TEST_ROWS_ONLY) ? 0 : n_train;
     auto blocks = [&](int64_t rows) { return heads * ((train + rows - 1) / rows + (n_test + rows - 1) / rows); };
     const int64_t blocks2 = blocks(kRowsPerBlock<2>), blocks3 = blocks(kRowsPerBlock<3>);
+    const bool keys_split = (flags & FP8ATTN_SPLIT_TAIL) && n_train > 15 * 128 && 2 * blocks2 <= sms;
+    if (blocks(kRowsPerBlock<1>) <= sms && n_train <= kOneTileKeys && !keys_split) return kRowsPerBlock<1>;
+    if (d != 64) return kRowsPerBlock<2>;
     if (blocks3 >= 8 * (int64_t)sms) return kRowsPerBlock<3>;
     if ((flags & FP8ATTN_SPLIT_TAIL) && blocks2 >= 8 * (int64_t)sms) return kRowsPerBlock<3>;
     if ((flags & FP8ATTN_SPLIT_TAIL) && blocks2 > 0 && blocks2 < sms) {
@@ -1025,12 +1043,8 @@ int attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d,
 
 int launch_icl_attention(const AttnParams& p, bool fp8, cudaStream_t stream) {
     const bool half = (p.flags & FP8ATTN_IO_FP16) != 0;
-    if (fp8) {
-        if (half) return p.d == 64 ? launch_d64<true, true>(p, stream) : launch<true, 128, true, 2>(p, stream);
-        return p.d == 64 ? launch_d64<true, false>(p, stream) : launch<true, 128, false, 2>(p, stream);
-    }
-    if (half) return p.d == 64 ? launch_d64<false, true>(p, stream) : launch<false, 128, true, 2>(p, stream);
-    return p.d == 64 ? launch_d64<false, false>(p, stream) : launch<false, 128, false, 2>(p, stream);
+    if (fp8) return half ? launch_tiles<true, true>(p, stream) : launch_tiles<true, false>(p, stream);
+    return half ? launch_tiles<false, true>(p, stream) : launch_tiles<false, false>(p, stream);
 }
 
 }  // namespace fp8attn

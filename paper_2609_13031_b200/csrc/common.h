@@ -99,7 +99,7 @@ struct AttnParams {
 };
 int launch_icl_attention(const AttnParams& p, bool fp8, cudaStream_t stream);
 // Query rows per CTA that a forward call of these sizes and flags uses on a device with `sms` SMs and
-// with that much scratch for the tail split: 256, or at d = 64 also 384 (attention.cu says when).
+// with that much scratch for the tail split: 256, 128 in small launches, or at d = 64 also 384 (attention.cu says when).
 int attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d, uint32_t flags, int sms,
                            size_t partial_bytes = (size_t)1 << 40);
 int launch_wait_timeout_selftest(uint32_t* status, uint64_t limit_ns, cudaStream_t stream);
