@@ -1,7 +1,8 @@
 """Python binding of libfp8attn.so (declared in ``include/fp8attn.h``).
 
 Argument marshalling only: every function hands device pointers, sizes and the
-current CUDA stream to the C-ABI entry point of the same name.  torch is used
+current CUDA stream to the C-ABI entry point of the same name (``icl_attention`` through a
+CPython module, ``csrc/binding.cpp``, the others through ctypes).  torch is used
 for device memory and streams.  There is no fallback: if the CUDA library has
 not been built, loading raises.
 """
@@ -46,6 +47,7 @@ HOST_FP16 = 2
 HOST_ORDER_KEYS = 4
 
 _lib = None
+_native = None      # csrc/binding.cpp
 
 
 class Fp8AttnError(RuntimeError):
@@ -57,7 +59,7 @@ class Fp8AttnError(RuntimeError):
 def load() -> ctypes.CDLL:
     """Load the CUDA library; raises if it is missing (build it with
     ``python -m paper_2609_13031_b200.build`` or ``__graft_entry__.build()``)."""
-    global _lib
+    global _lib, _native
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -125,7 +127,13 @@ def load() -> ctypes.CDLL:
     lib.fp8attn_icl_step_host.argtypes = [vp, vp, vp, vp, i32, i32, i64, i64, i32, f32, u32, vp, vp, vp, sz, vp]
     lib.fp8attn_host_step_status.restype = i32
     lib.fp8attn_host_step_status.argtypes = [vp, i32, i32, i64, i64, i32, u32, vp, ctypes.POINTER(ctypes.c_uint32)]
-    _lib = lib
+    try:
+        from . import _binding
+    except ImportError as e:
+        raise RuntimeError("the native half of the binding has not been built.  Run "
+                           "`python -m paper_2609_13031_b200.build`.") from e
+    _binding.bind(ctypes.cast(lib.fp8attn_quantize_qkv_ex, vp).value, ctypes.cast(lib.fp8attn_icl_forward_ex, vp).value)
+    _native, _lib = _binding, lib
     return lib
 
 
@@ -456,34 +464,14 @@ def icl_attention(q_train, q_test, k, v, workspace=None, softmax_scale: float = 
     """The whole hot path on bf16 inputs: quantize Q_train, K, V per head, quantize
     Q_test with the train-query scale, then the fused FP8 attention (``flags``: forward
     flags, e.g. SPLIT_TAIL)."""
-    B, H, n_train, d = _dims(k)
     if workspace is None:
+        B, H, n_train, d = _dims(k)
         workspace = new_workspace(B, H, k.device, n_train=n_train if flags & SPLIT_TAIL else 0, d=d)
-    n_test = 0 if q_test is None else q_test.shape[2]
-    for t in (q_train, k, v) + (() if n_test == 0 else (q_test,)):
-        assert t.dtype == k.dtype and _is16(t)
-    half = k.dtype == torch.float16
-    # The codes and scales stay inside this call: one allocation holds them all (nine tensors of their own
-    # cost a small call, whose kernels take 20 us, more time on the host than that).
-    train, test, heads = B * H * n_train * d, B * H * n_test * d, B * H
-    at = [0]
-    for nbytes in (train, train, train, test, 4 * heads, 4 * heads, 4 * heads):
-        at.append(at[-1] + (nbytes + 255) // 256 * 256)
-    codes = k.new_empty(at[-1], dtype=torch.uint8)
-    q8, k8, v8, t8, sq, sk, sv = (codes.data_ptr() + o for o in at[:-1])
-    out_train = None if flags & TEST_ROWS_ONLY else k.new_empty((B, H, n_train, d))
-    out_test = k.new_empty((B, H, n_test, d)) if n_test else None
-    lib, stream, ws, ws_bytes = load(), _stream(), workspace.data_ptr(), workspace.numel()
-    if n_test == 0:
-        q_test = t8 = None
-    rc = lib.fp8attn_quantize_qkv_ex(q_train.data_ptr(), k.data_ptr(), v.data_ptr(), _ptr(q_test), B, H, n_train,
-                                     n_test, d, q8, k8, v8, t8, sq, sk, sv, INPUT_FP16 if half else 0, ws, ws_bytes,
-                                     stream)
-    _check("fp8attn_quantize_qkv", rc)
-    rc = lib.fp8attn_icl_forward_ex(None if out_train is None else q8, t8, k8, v8, sq, sk, sv, B, H, n_train, n_test, d,
-                                    float(softmax_scale), int(flags) | (IO_FP16 if half else 0), _ptr(out_train),
-                                    _ptr(out_test), ws, ws_bytes, stream)
-    _check("fp8attn_icl_forward", rc)
+    if _native is None:
+        load()
+    quantized, forward, out_train, out_test = _native.icl_attention(q_train, q_test, k, v, workspace, softmax_scale, flags)
+    _check("fp8attn_quantize_qkv", quantized)
+    _check("fp8attn_icl_forward", forward)
     return out_train, out_test
 
 

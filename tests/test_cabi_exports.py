@@ -138,3 +138,15 @@ def test_argument_checks_run_on_the_host_before_anything_touches_a_gpu():
     # arguments in order, but no GPU: the call reports it; nothing falls back to the CPU
     assert f(*ok) in (api.ERR_CUDA, api.ERR_UNSUPPORTED)
     assert q(P, 1, 2, 8, 64, None, P, P, WS, ws_bytes, None) in (api.ERR_CUDA, api.ERR_UNSUPPORTED)
+
+
+def test_native_binding_refuses_what_the_call_does_not_take():
+    import pytest
+    import torch
+    api.load()
+    ok = torch.zeros((1, 1, 4, 64), dtype=torch.bfloat16)
+    for args in ((ok, ok, ok, ok), (None, ok, ok, ok), (ok, ok, None, ok), (ok, ok, ok.view(1, 4, 64), ok)):
+        with pytest.raises(AssertionError):
+            api.icl_attention(*args, workspace=torch.zeros(4096, dtype=torch.uint8))
+    with pytest.raises(TypeError):
+        api.icl_attention(ok, 3, ok, ok, workspace=torch.zeros(4096, dtype=torch.uint8))
