@@ -109,6 +109,12 @@ struct Cfg {
     // P alternates between two buffers per tile (the second kPCols columns after the first) where
     // there is room, so that writing P of one step never waits for the P V of the step before.
     static constexpr int kPBufs = kFp8 || kRoomy ? 2 : 1;
+    // A softmax thread asks whether P V of the step before is done before it starts on the exponentials, and only
+    // waits at the end of the step, or where it needs the one P buffer, if it was not.  With two buffers the wait at
+    // the end never lasts, but the look alone is 140 of 2,011 cycles of a step of one tile (FP8, d = 64): 2 heads
+    // of 8,192 + 1,000 rows 73.4 -> 70.9 us, with two tiles 8 heads of 8,192 + 2,048 214 -> 210, three tiles 9,408 ->
+    // 9,339 (8 heads of 65,536 + 1,000); bf16 at d = 64 224 -> 221.  (bf16, one tile, d = 128: 15.7 -> 16.0, so not there.)
+    static constexpr bool kAskEarly = kPBufs == 1 || kFp8 || kD == 64;
     // pairs of exponentials, out of every 16 pairs, that go to the FMA pipe (measured best)
     static constexpr int kPolyPer16 = kFp8 ? (kT == 3 ? 2 : 4) : 2;
     static_assert(kPBufs * kPCols <= (int)kPStride, "TMEM layout: P tiles overlap");
@@ -603,7 +609,7 @@ icl_attention_kernel(const __grid_constant__ CUtensorMap map_q_train,
                 const float m_new = fmaxf(m, m_tile);
                 // P V of the previous step must be done before O is rescaled or P rewritten
                 bool pv_done = j == 0;
-                if (C::kPBufs == 1 && !pv_done && !w.dead) {
+                if (C::kAskEarly && !pv_done && !w.dead) {
                     // ask now, use the answer a chunk of exponentials later: the usual case
                     // (P V long done) then costs no stall in the middle of the chunk
                     pv_done = mbar_test_wait(smem_u32(&bars.p_free[t]), (j - 1) & 1);
@@ -675,7 +681,7 @@ icl_attention_kernel(const __grid_constant__ CUtensorMap map_q_train,
                     // That write comes after the next step's fence behind its wait for S.
                     w.wait(smem_u32(&bars.p_free[t]), (j - 1) & 1, kWaitPFree);
                     pv_done = true;
-                    if (rescale) tc_fence_after_sync();
+                    tc_fence_after_sync();
                 }
                 if (rescale) {
                     if (!pv_done) {
