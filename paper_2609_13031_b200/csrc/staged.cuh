@@ -25,7 +25,7 @@
 //
 // Measured, graph-replayed, one pass / two passes: 8 heads of 65,536 + 16,384 rows x 128 (654 MB in and
 // out, 100 us at the copy rate) 126-130 / 183 us; x 64 72 / 94 us; 16 heads of 20,011 + 3,001 x 128 92-97 / 115 us;
-// 8 heads 52-57 / 56 us; 8,192 + 2,048 x 64 15.8 / 20.5 us.  About 10 us go before the second stage: launch,
+// 8 heads 52-57 / 56 us; 8,192 + 2,048 x 64 14.5 / 20.5 us.  About 10 us go before the second stage: launch,
 // the first stage's way in, and its exchange under the second's loads.
 // (Tried before: 24 KB chunks handed out by tickets to a control thread and worker warps: 2.5 us per
 // chunk for the hand-overs.  Accumulators and a grid-wide counter instead of tagged words: 154 us.
@@ -503,6 +503,271 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
     }
 }
 
+// Two stages fill both buffers and wait for no room: they are loaded at once and exchanged together, so that the
+// workers stand still once, under the second load, instead of twice (2 us each, 3 us where the words wait behind loads
+// from HBM).  Graph-replayed, inputs not in L2 / in L2: 16 heads of 12,289 x 64 19.1 -> 17.8 / 13.1 -> 12.5 us, 8 heads of
+// 16,384 x 128 22.2 -> 20.1 / 13.7 -> 13.6, 8 heads of 8,192 + 2,048 x 64, three tensors, 21.4 -> 19.5 / 16.1 -> 14.5.  Rows
+// that count in the maximum stay with the general form.  (A kernel of its own: as a template parameter of the general
+// one it moved that by up to 3 % through its schedule.)
+template <bool kHalf, bool kSelfTest>
+__global__ void __launch_bounds__(kThreads, 1) staged_pair_kernel(const __grid_constant__ Args a) {
+    const int64_t limit = kSelfTest ? a.wait_clocks : kWaitClocks;
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ uint64_t full[2];
+    __shared__ uint32_t seg_acc[2][kMaxSegments];
+    __shared__ Segment segment[2][kMaxSegments];
+    __shared__ uint16_t holders[2][kMaxSegments][2];    // first and last block of every segment's unit
+    __shared__ uint32_t follow_acc[kMaxFollowHeads];
+    __shared__ volatile int lost, give_up;
+    static_assert(kSmemBytes + sizeof(segment) + sizeof(seg_acc) + sizeof(follow_acc) + 768 <= 232448, "shared memory of a block");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int stages = 2;
+    const uint32_t vecs = (uint32_t)a.vecs, tensors = (uint32_t)a.tensors;
+    if (tid == 0) {
+        for (int i = 0; i < 2; ++i) mbar_init(smem_u32(&full[i]), kParts);
+        fence_mbar_init();
+        lost = give_up = 0;
+    }
+    if (tid < (int)(sizeof(seg_acc) / sizeof(uint32_t))) (&seg_acc[0][0])[tid] = 0u;
+    // rows that follow tensor 0 without counting are converted last, an equal share of them per block;
+    // those of a small call are on their way to L2 from the start
+    uint32_t f_lo = 0, f_hi = 0;
+    if (a.follow_vecs > 0) {
+        const uint32_t total = (uint32_t)(a.units / a.tensors) * a.follow_vecs;
+        const uint32_t each = total / gridDim.x, more = total - each * gridDim.x;
+        f_lo = each * blockIdx.x + min(blockIdx.x, more);
+        f_hi = f_lo + each + (blockIdx.x < more ? 1u : 0u);
+        if (f_lo + tid * 8 < f_hi) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.follow_x + f_lo + tid * 8));
+    }
+    __syncthreads();
+    const Share share_full((uint32_t)min(a.stage_units, a.units), vecs);
+    const Share share_last((uint32_t)(a.units - (stages - 1) * a.stage_units), vecs);
+
+    auto timed_out = [&] {
+        if (atomicCAS(a.status, 0u, (uint32_t)FP8ATTN_ERR_TIMEOUT) == 0u)
+            a.status[1] = (kDetailGridWait << 24) | (blockIdx.x & 0xFFFFFFu);
+    };
+
+    if (warp == kWorkers / 32) {
+        // ============================== loads ==============================
+        if (lane == 0) {
+            for (int stage = 0; stage < stages; ++stage) {
+                const Share& s = stage == 0 ? share_full : share_last;
+                const uint32_t bar = smem_u32(&full[stage]);
+                for (uint32_t part = 0; part < kParts; ++part) {
+                    mbar_arrive_expect_tx(bar, (part == 0 ? s.half() : s.n - s.half()) * 16);
+                    half_share(a, s, stage, part, [&](uint32_t i0, const uint4* src, uint32_t n) {
+                        bulk_load(smem_u32(smem) + (stage * kBufVecs + i0) * 16, src, n * 16, bar);
+                    });
+                }
+            }
+        }
+        __syncwarp();
+    } else if (warp > kWorkers / 32) {
+        // ============================== exchange ==============================
+        // (recorded before this launch, so all blocks decide alike; asked for under the first loads)
+        const bool pending = a.heed_status && *reinterpret_cast<volatile uint32_t*>(a.status) != 0u;
+        // One stage's exchange: what of it can be known before the share is reduced (the barrier comes between).
+        struct Round {
+            const Share& s;
+            uint32_t u0, *slots, tag;
+            uint16_t (*holders)[2];
+            int stage;
+        };
+        auto round = [&](int stage) {
+            const Share& s = stage + 1 < stages ? share_full : share_last;
+            uint16_t (*const h)[2] = holders[stage];
+            for (uint32_t g = lane; g < s.segs; g += 32) {
+                h[g][0] = (uint16_t)s.holder((s.unit + g) * vecs);
+                h[g][1] = (uint16_t)s.holder((s.unit + g + 1) * vecs - 1);
+            }
+            return Round{s, (uint32_t)(stage * a.stage_units) + s.unit,
+                         a.slots + stage * a.slots_per_set, (uint32_t)stage + 1, h, stage};
+        };
+        auto put = [&](const Round& r) {
+            const Share& s = r.s;
+            // (block b and unit u of the stage meet at most once, and b + u names the meeting)
+            for (uint32_t g = lane; g < s.segs; g += 32) {
+                publish(r.slots + blockIdx.x + s.unit + g, r.tag, seg_acc[r.stage][g]);
+                seg_acc[r.stage][g] = 0u;
+            }
+            __syncwarp();
+        };
+        // true: this lane's values are there
+        auto collect = [&](const Round& r) {
+            const Share& s = r.s;
+            uint32_t* const slots = r.slots;
+            const uint32_t tag = r.tag, u0 = r.u0;
+            const int stage = r.stage;
+            // Collect the values of this share's units: `width` lanes per segment.
+            const uint32_t width = s.segs <= 1 ? 32 : 16;
+            const bool none_empty = s.total >= 8 * gridDim.x;
+            bool there = !lost && !pending;
+            const int64_t t0 = clock64();
+            for (uint32_t g0 = 0; g0 < s.segs; g0 += 32 / width) {
+                const uint32_t g = g0 + lane / width;
+                uint32_t v = 0u;
+                if (g < s.segs) {
+                    constexpr int kBatch = 5;       // polls under way at a time: 148 blocks at 32 a row
+                    const uint32_t u = s.unit + g, b1 = r.holders[g][1];
+                    for (uint32_t b0 = r.holders[g][0] + lane % width; b0 <= b1; b0 += kBatch * width) {
+                        uint32_t raw[kBatch];
+                        for (bool all = false; there && !all;) {
+#pragma unroll
+                            for (int k = 0; k < kBatch; ++k) raw[k] = peek(slots + min(b0 + k * width, b1) + u);
+                            all = true;
+#pragma unroll
+                            for (int k = 0; k < kBatch; ++k) {
+                                const uint32_t b = min(b0 + k * width, b1);
+                                all &= tagged(raw[k], tag) || (!none_empty && cut(s.total, b) == cut(s.total, b + 1));
+                            }
+                            if (!all) there = !lost && clock64() - t0 < limit;
+                        }
+#pragma unroll
+                        for (int k = 0; k < kBatch; ++k)
+                            if (b0 + k * width <= b1 && there && tagged(raw[k], tag)) v = max(v, value(raw[k]));
+                    }
+                }
+                __syncwarp();
+                for (uint32_t o = width >> 1; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+                if (g < s.segs && lane % width == 0) {
+                    const uint32_t unit = u0 + g, head = unit / tensors, z = unit - head * tensors;
+                    Segment& seg = segment[stage & 1][g];
+                    seg.divisor = divisor(head_scale(In16<kHalf>::lo(v)));
+                    seg.begin = s.begin(g, vecs);
+                    seg.end = s.end(g, vecs);
+                    seg.head = head;
+                    seg.at = (int32_t)(s.at(g) - seg.begin);
+                    seg.out = static_cast<uint8_t*>(a.out[z]) + ((int64_t)head * vecs + seg.at) * 8;
+                    if (there && (g > 0 || s.skip == 0)) {      // the unit begins here
+                        if (a.result_out[z] != nullptr) a.result_out[z][head] = seg.divisor.s;
+                        if (z == 0 && a.follow_vecs > 0) publish(a.heads + head, 1, v);
+                    }
+                }
+            }
+            return there;
+        };
+        const Round r0 = round(0), r1 = round(1);
+        sync_exchange();        // A: both shares are reduced
+        put(r0);
+        put(r1);
+        bool there = collect(r0);
+        there = collect(r1) && there;
+        if (!__all_sync(0xffffffffu, there) && lane == 0) {
+            if (!pending) timed_out();
+            give_up = 1;
+        }
+        sync_exchange();        // B: results are known
+        // The heads that this block's following rows belong to (calls that cleared the words read them
+        // when they convert).
+        if (f_lo < f_hi && !a.cleared && !give_up) {
+            const uint32_t h = f_lo / a.follow_vecs + lane;
+            bool there = true;
+            if (h <= (f_hi - 1) / a.follow_vecs) {
+                const int64_t t0 = clock64();
+                uint32_t raw = peek(a.heads + h);
+                while (there && !tagged(raw, 1)) {
+                    there = clock64() - t0 < limit;
+                    raw = peek(a.heads + h);
+                }
+                follow_acc[lane] = value(raw);
+            }
+            if (!__all_sync(0xffffffffu, there) && lane == 0) {
+                timed_out();
+                give_up = 1;
+            }
+        }
+        // The last warp to get here leaves everything at zero for the next call: its fence and those of the
+        // others put all stores and polls of the words before that.
+        __syncwarp();
+        uint32_t done = 0;
+        if (lane == 0) {
+            __threadfence();
+            done = atomicAdd(a.counter, 1u);
+            __threadfence();
+        }
+        if (__shfl_sync(0xffffffffu, done, 0) == gridDim.x - 1) {
+            for (uint32_t i = lane; i < a.sets * a.slots_per_set; i += 32) a.slots[i] = 0u;
+            if (a.follow_vecs > 0 && !a.cleared)
+                for (int i = lane; i < a.units / a.tensors; i += 32) a.heads[i] = 0u;
+            if (lane == 0) *a.counter = 0u;
+        }
+    } else {
+        // ============================== workers ==============================
+        auto convert_half = [&](int stage, uint32_t part) {
+            const Share& s = stage + 1 < stages ? share_full : share_last;
+            const uint4* buf = reinterpret_cast<const uint4*>(smem) + (stage & 1) * kBufVecs;
+            const uint32_t p0 = part == 0 ? 0 : s.half(), p1 = part == 0 ? s.half() : s.n;
+            for (uint32_t g = 0; g < s.segs; ++g) {
+                const Segment& seg = segment[stage & 1][g];
+                const uint32_t i0 = max(p0, seg.begin), i1 = min(p1, seg.end);
+                if (i0 < i1) convert<kHalf, false>(seg, buf, i0, i1, tid);
+            }
+        };
+        // the share's values, once it has landed
+        auto reduce_share = [&](int stage) {
+            const Share& s = stage + 1 < stages ? share_full : share_last;
+            const uint4* buf = reinterpret_cast<const uint4*>(smem) + (stage & 1) * kBufVecs;
+            const uint32_t bar = smem_u32(&full[stage]), parity = 0;
+            bool landed = mbar_test_wait(bar, parity);
+            if (!landed) {
+                const int64_t t0 = clock64();
+                while (!landed && !lost && clock64() - t0 < limit) landed = mbar_try_wait(bar, parity);
+            }
+            if (!__all_sync(0xffffffffu, landed)) {     // what is published then bears no tag
+                lost = 1;
+                for (uint32_t g = lane; g < s.segs; g += 32) atomicMax(&seg_acc[stage][g], kLost);
+            }
+            for (uint32_t g = 0; g < s.segs; ++g) {
+                const uint32_t b = s.begin(g, vecs), e = s.end(g, vecs);
+                if (b + (tid & ~31) >= e) continue;      // (whole warps)
+                uint32_t v = 0u;
+                if (b + tid < e) v = reduce<kHalf>(buf + b, e - b, tid);
+                v = __reduce_max_sync(0xffffffffu, v);
+                if (lane == 0) atomicMax(&seg_acc[stage][g], v);
+            }
+        };
+#pragma unroll 1
+        for (int stage = 0; stage < stages; ++stage) reduce_share(stage);
+        sync_exchange();    // A
+        sync_exchange();    // B
+#pragma unroll 1
+        for (uint32_t half = 0; half < 2 * kParts && !give_up; ++half) convert_half(half / kParts, half % kParts);
+    }
+    __syncthreads();
+    // ---- a block that gives up leaves when its copies have landed ----
+    if (give_up && tid == kWorkers) {
+        const int64_t t0 = clock64();
+        for (int stage = 0; stage < stages; ++stage)
+            while (!mbar_try_wait(smem_u32(&full[stage]), 0) && clock64() - t0 < kWaitClocks) {}
+    }
+    // ---- rows that follow tensor 0 ----
+    if (!give_up) {
+        bool there = true;
+        const int64_t t0 = clock64();
+        Segment seg;
+        seg.at = 0;
+        seg.out = static_cast<uint8_t*>(a.follow_out);
+        for (uint32_t x = f_lo; x < f_hi && there;) {
+            seg.head = x / a.follow_vecs;
+            const uint32_t end = f_hi - seg.head * a.follow_vecs < a.follow_vecs ? f_hi : (seg.head + 1) * a.follow_vecs;
+            uint32_t v = follow_acc[a.cleared ? 0 : seg.head - f_lo / a.follow_vecs];
+            if (a.cleared) {
+                uint32_t raw = peek(a.heads + seg.head);
+                while (there && !tagged(raw, 1)) {
+                    there = clock64() - t0 < limit;
+                    raw = peek(a.heads + seg.head);
+                }
+                v = value(raw);
+            }
+            seg.divisor = divisor(head_scale(In16<kHalf>::lo(v)));
+            if (there && tid < kWorkers) convert<kHalf, true>(seg, a.follow_x, x, end, tid);
+            x = end;
+        }
+        if (!there) timed_out();
+    }
+}
+
 // Fills what plan() does not get (stage_units and everything behind it) and returns the grid, or 0 where
 // this path does not take the call: a unit that does not fit one buffer of every SM or is no longer than a
 // share, or more words than the workspace has for them.
@@ -541,8 +806,9 @@ constexpr int kRefused = -1;
 
 template <bool kHalf, bool kSelfTest>
 int launch(const Args& a, unsigned grid, cudaStream_t stream) {
+    // Two stages whose test rows do not count: the pair kernel, 5 .. 11 % faster (see there).
     // (the opt-in to large dynamic shared memory is per device and context: set on every call)
-    auto kernel = staged_kernel<kHalf, kSelfTest>;
+    auto kernel = a.stages == 2 && !a.follow_counts ? staged_pair_kernel<kHalf, kSelfTest> : staged_kernel<kHalf, kSelfTest>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) !=
         cudaSuccess)
         return FP8ATTN_ERR_CUDA;
