@@ -281,7 +281,7 @@ int fp8attn_gate_use_fp8(int64_t n_train);
  * blocks fills the SMs at least eight times over or, with FP8ATTN_SPLIT_TAIL, when that of
  * 256-row blocks does or when a launch of less than one round is over sooner that way,
  * or 128 (one) up to 16,384 train rows when even the grid of 128-row blocks leaves SMs
- * free and the keys are not split instead.
+ * free and no split of the keys (FP8ATTN_SPLIT_TAIL) is over sooner.
  * Without a device the SM count of a B200 (148) is assumed.  0 for unsupported sizes.
  * Results do not depend on it beyond the order of the online softmax (steps of 128 or 96
  * keys). */

@@ -20,6 +20,8 @@
 //
 // Scale placement (FP8 path): x = (alpha * s_q * s_k * log2 e) * S feeds exp2;
 // the V scale and 1/rowsum are applied to O in the epilogue.
+#include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include <cuda_bf16.h>
@@ -871,6 +873,20 @@ combine_split_kernel(const KernelArgs args, int units, int out_half, int fp8) {
         *reinterpret_cast<uint2*>(out) = make_uint2(v[0], v[1]);
 }
 
+// Key ranges that FP8ATTN_SPLIT_TAIL divides each block of the last, partly filled round of `grid` blocks of `tiles`
+// tiles into; 1 = no split.
+// Measured: it pays from about one round up to about eight (1.4x at 1.1 rounds, 1.27x
+// at 2.2, 1.1x at 4.3, nothing beyond 8: after many rounds the SMs have drifted apart
+// and the last round is no longer a round), provided a key range keeps at least four
+// steps; below that the extra launches cost more than the split saves.
+int64_t tail_splits(int tiles, int d, int64_t grid, int64_t n_train, int sms, size_t partial_bytes) {
+    const int64_t left = grid % sms, keys = tiles == 3 ? 96 : 128, steps = (n_train + keys - 1) / keys;
+    if (left == 0 || grid >= 8 * (int64_t)sms || steps < 16) return 1;
+    const int64_t room = (int64_t)(partial_bytes / ((size_t)left * tiles * kTileM * (d + 4) * sizeof(float)));
+    const int64_t splits = std::min({sms / left, steps / 4, (int64_t)kMaxSplits, room});
+    return splits >= 2 ? splits : 1;
+}
+
 template <bool kFp8, int kD, bool kHalf, int kT>
 int launch(const AttnParams& p, cudaStream_t stream) {
     using C = Cfg<kFp8, kD, kHalf, kT>;
@@ -914,23 +930,12 @@ int launch(const AttnParams& p, cudaStream_t stream) {
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
             return FP8ATTN_ERR_CUDA;
         const int64_t full = (grid / sms) * sms, left = grid - full;
-        const int64_t steps = (p.n_train + C::kKeys - 1) / C::kKeys;
-        // Measured: it pays from about one round up to about eight (1.4x at 1.1 rounds, 1.27x
-        // at 2.2, 1.1x at 4.3, nothing beyond 8: after many rounds the SMs have drifted apart
-        // and the last round is no longer a round), provided a key range keeps at least four
-        // steps; below that the extra launches cost more than the split saves.
-        if (left > 0 && grid < 8 * (int64_t)sms && steps >= 16) {
-            int64_t splits = sms / left;
-            if (splits > steps / 4) splits = steps / 4;
-            if (splits > kMaxSplits) splits = kMaxSplits;
-            const size_t per_split = (size_t)left * kRowsPerBlock<kT> * kPartialStride<kD> * sizeof(float);
-            while (splits >= 2 && per_split * (size_t)splits > p.partial_bytes) --splits;
-            if (splits >= 2) {
-                a.full_blocks = (int)full;
-                a.splits = (int)splits;
-                a.partial = p.partial;
-                units = (int)left;
-            }
+        const int64_t splits = tail_splits(kT, kD, grid, p.n_train, sms, p.partial_bytes);
+        if (splits >= 2) {
+            a.full_blocks = (int)full;
+            a.splits = (int)splits;
+            a.partial = p.partial;
+            units = (int)left;
         }
     }
     auto kern = icl_attention_kernel<kFp8, kD, kHalf, kT, false>;
@@ -1013,12 +1018,16 @@ int launch_tiles(const AttnParams& p, cudaStream_t stream) {
     return launch<kFp8, 64, kHalf, 2>(p, stream);
 }
 
-// One tile per CTA where all of a launch's tiles fit on the SMs at once and its keys are not split instead: the
-// CTA's steps are what the launch takes.  The same results bit for bit as with two tiles (a tile's rows see the
+// One tile per CTA where all of a launch's tiles fit on the SMs at once and no split of the keys is over sooner: the
+// CTA's steps are what the launch takes.  The same results bit for bit as with two tiles unsplit (a tile's rows see the
 // same keys in the same steps), so the choice may depend on the number of test rows.  Two tiles / one: 2 heads of
 // 512 + 128 x 64 10.1 / 8.1 us; 8 heads of 1,024 + 256 x 64 16.2 / 13.0, x 128 18.6 / 14.4 (bf16 20.3 / 15.3);
 // 2 heads of 8,192 + 1,000 x 128 101 / 77 (bf16 112 / 81); 1 head of 16,000 + 2,000 x 64 174 / 137.  Up to
 // kOneTileKeys keys, as measured: every K and V tile is fetched for half as many rows.
+// With FP8ATTN_SPLIT_TAIL by the times below, one tile / the split that it replaces or leaves: 49 heads of 300 test
+// rows against 16,000 x 64 132 / 98 us (three tiles in three ranges), 29 heads of 600 against 8,000 70 / 76; 8 heads of
+// 1,930 + 250 x 64 22.5 / 23.5, x 128 26.1 / 29.7; 2,300 test rows of 8 heads against 3,000 x 64 31.2 / 29.2, x 128
+// 34.8 / 36.4; against 5,000 47 / 40 and 52 / 48.
 constexpr int64_t kOneTileKeys = 16384;
 
 // d = 64: two or three tiles per CTA.
@@ -1038,26 +1047,37 @@ int attention_rows_per_cta(int B, int H, int64_t n_train, int64_t n_test, int d,
                            size_t partial_bytes) {
     const int64_t heads = (int64_t)B * H, train = (flags & FP8ATTN_TEST_ROWS_ONLY) ? 0 : n_train;
     auto blocks = [&](int64_t rows) { return heads * ((train + rows - 1) / rows + (n_test + rows - 1) / rows); };
-    const int64_t blocks2 = blocks(kRowsPerBlock<2>), blocks3 = blocks(kRowsPerBlock<3>);
-    const bool keys_split = (flags & FP8ATTN_SPLIT_TAIL) && n_train > 15 * 128 && 2 * blocks2 <= sms;
-    if (blocks(kRowsPerBlock<1>) <= sms && n_train <= kOneTileKeys && !keys_split) return kRowsPerBlock<1>;
+    const int64_t blocks1 = blocks(kRowsPerBlock<1>), blocks2 = blocks(kRowsPerBlock<2>), blocks3 = blocks(kRowsPerBlock<3>);
+    const bool split = (flags & FP8ATTN_SPLIT_TAIL) != 0;
+
+    // The time of a launch of less than one round, in steps of 128 keys of two tiles.
+    constexpr float kCost[3] = {0.72f, 1.0f, 1.43f};     // time per key of one, two, three tiles
+    constexpr float kSplitSteps = 6.0f;                  // launch and combine
+    constexpr float kRangeSteps = 0.8f / 16384.0f;       // per row of 64 columns and range
+    const float steps = (float)n_train / 128.0f;
+    const int64_t rows = heads * (train + n_test), tiles = ((train > n_test ? train : n_test) + kTileM - 1) / kTileM;
+    auto unsplit_time = [&](int t) { return kCost[(tiles < t ? tiles : t) - 1] * steps; };
+    auto split_time = [&](int t, int64_t n) {            // infinity where the launch is not split
+        const int64_t ranges = tail_splits(t, d, n, n_train, sms, partial_bytes);
+        const int64_t splits = steps > 15.0f ? std::min(ranges, (int64_t)(steps / 4)) : 1;
+        return splits < 2 ? INFINITY
+                          : unsplit_time(t) / (float)splits + kSplitSteps + kRangeSteps * (float)(rows * splits * (d / 64));
+    };
+    if (blocks1 > 0 && blocks1 <= sms && n_train <= kOneTileKeys) {
+        if (!split) return kRowsPerBlock<1>;
+        // (what one launch costs beside its steps, to be held against kSplitSteps; fitted to the calls above)
+        const float one = unsplit_time(1) + (d == 64 ? 3.5f : 3.0f);
+        const float two = split_time(2, blocks2), three = d == 64 ? split_time(3, blocks3) : INFINITY;
+        if (one <= two && one <= three) return kRowsPerBlock<1>;
+        return three < 0.975f * two ? kRowsPerBlock<3> : kRowsPerBlock<2>;      // (unsplit, neither is as fast as one)
+    }
     if (d != 64) return kRowsPerBlock<2>;
     if (blocks3 >= 8 * (int64_t)sms) return kRowsPerBlock<3>;
-    if ((flags & FP8ATTN_SPLIT_TAIL) && blocks2 >= 8 * (int64_t)sms) return kRowsPerBlock<3>;
-    if ((flags & FP8ATTN_SPLIT_TAIL) && blocks2 > 0 && blocks2 < sms) {
-        constexpr float kCost[3] = {0.72f, 1.0f, 1.43f};     // time per key of one, two, three tiles
-        constexpr float kSplitSteps = 6.0f;                  // launch and combine, in steps of 128 keys
-        constexpr float kRangeSteps = 0.8f / 16384.0f;       // per row and range
-        const int64_t rows = heads * (train + n_test);
-        const float steps = (float)n_train / 128.0f;
-        const int64_t tiles = ((train > n_test ? train : n_test) + kTileM - 1) / kTileM;
+    if (split && blocks2 >= 8 * (int64_t)sms) return kRowsPerBlock<3>;
+    if (split && blocks2 > 0 && blocks2 < sms) {
         auto time = [&](int t, int64_t n) {
-            const int64_t room = (int64_t)(partial_bytes / ((size_t)n * t * kTileM * kPartialStride<64> * sizeof(float)));
-            int64_t splits = sms / n < kMaxSplits ? sms / n : kMaxSplits;
-            if (splits > room) splits = room;
-            if (splits > steps / 4) splits = (int64_t)(steps / 4);
-            const float one = kCost[(tiles < t ? tiles : t) - 1] * steps;
-            return splits >= 2 ? one / (float)splits + kSplitSteps + kRangeSteps * (float)(rows * splits) : one;
+            const float ranges = split_time(t, n);
+            return ranges < INFINITY ? ranges : unsplit_time(t);
         };
         if (time(3, blocks3) < 0.975f * time(2, blocks2)) return kRowsPerBlock<3>;
     }

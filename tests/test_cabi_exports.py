@@ -84,6 +84,22 @@ def test_tiles_per_cta_of_split_launches():
     assert api.attention_rows_per_cta(1, 8, 30011, 2048, 64, api.TEST_ROWS_ONLY) == 256
 
 
+def test_one_tile_gives_way_to_a_split_that_is_over_sooner():
+    """Both sides of the choice between CTAs of one tile and the split of the keys."""
+    api.load()
+    test_rows = api.SPLIT_TAIL | api.TEST_ROWS_ONLY
+    for H, n, m, d, flags, rows in (
+            (49, 16000, 300, 64, test_rows, 384), (49, 4000, 300, 64, test_rows, 384), (40, 8000, 333, 64, test_rows, 384),
+            (29, 8000, 600, 64, test_rows, 128), (49, 16000, 300, 128, test_rows, 128), (49, 1440, 300, 64, test_rows, 128),
+            (8, 1930, 250, 64, api.SPLIT_TAIL, 128), (8, 1930, 250, 128, api.SPLIT_TAIL, 128), (1, 16200, 2600, 64, api.SPLIT_TAIL, 128),
+            (16, 3000, 1000, 64, test_rows, 256), (8, 3000, 2300, 128, test_rows, 128), (16, 5000, 1000, 128, test_rows, 256),
+            (4, 3500, 700, 64, api.SPLIT_TAIL, 256), (4, 4000, 200, 128, api.SPLIT_TAIL, 256),
+            (40, 2000, 257, 64, test_rows, 128), (8, 2000, 1100, 128, test_rows, 256), (2, 16300, 129, 64, test_rows, 256),
+            (8, 4096, 1000, 64, test_rows, 256), (8, 1920, 250, 64, api.SPLIT_TAIL, 128)):
+        assert api.attention_rows_per_cta(1, H, n, m, d, flags) == rows, (H, n, m, d)
+        assert api.attention_rows_per_cta(1, H, n, m, d, flags & ~api.SPLIT_TAIL) == 128, (H, n, m, d)
+
+
 def test_dispatch_gate_matches_the_paper_constant():
     import os
     from helpers import read_golden_table
