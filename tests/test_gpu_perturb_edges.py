@@ -1,8 +1,11 @@
-"""The noise at the ends of what its formula meets: uniforms next to 1, whose logarithm is next to 0."""
+"""The noise at the ends of what its formula meets: uniforms next to 1, whose logarithm is next to 0, and strengths
+whose product with the RMS is next to the largest fp32 number."""
 import numpy as np
 import pytest
 import torch
 
+import oracle
+from helpers import bf16_bits_to_f64
 from paper_2609_13031_b200 import api
 
 pytestmark = pytest.mark.gpu
@@ -56,3 +59,17 @@ def test_uniforms_next_to_one():
         hi = rho * np.sqrt(z ** 2 + off) * (1 + 2.0 ** -8)
         assert np.all(got[:, col] >= lo) and np.all(got[:, col] <= hi), (got[:, col], z)
     assert api.last_device_status(ws) == (0, 0)
+
+
+def test_strengths_next_to_the_largest_number():
+    """epsilon * rho = 1e38: z up to 3 fits bf16, and the same elements are finite as in the oracle."""
+    x = torch.full((1, 1, 256, 64), 1e10, dtype=torch.bfloat16, device="cuda")
+    bits = x.view(torch.int16).cpu().numpy().view(np.uint16)
+    ws = api.new_workspace(1, 1)
+    out, rho = api.perturb(x, 1e28, 11, 2, ws)
+    ref, _ = oracle.perturb(bits, 1e28, 11, 2)
+    want, got = bf16_bits_to_f64(ref), out.double().cpu().numpy()
+    fits = np.abs(want) < 3e38
+    assert fits.mean() > 0.99 and np.abs(want[fits]).max() > 2.5e38
+    assert np.isfinite(got[fits]).all()
+    assert np.all(np.abs(got - want)[fits] <= 2.0 ** -7 * np.abs(want)[fits] + 1e-5 * 1e38)
