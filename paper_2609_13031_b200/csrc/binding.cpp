@@ -3,9 +3,9 @@
 // What bounds a small table's call is the host: marshalled in Python (nine addresses, three allocations through
 // the interpreter, two ctypes calls of twenty arguments each) a call of 2 heads of 512 + 128 x 64 kept it busy for
 // 22.9 us, where the kernels take 11.7.  Here it is one call with the tensors as they are, 10.7 us on the host, and
-// calls follow each other every 16.3 us.  Nothing is computed and nothing is kept: the arguments are checked, the
-// outputs and the buffer of the codes allocated, and the library's two C entry points, whose addresses Python
-// hands in when it loads it, called on the current stream.
+// calls follow each other every 16.3 us.  Nothing is computed and nothing is kept: type, sizes, layout and device of
+// the arguments are checked, the outputs and the buffer of the codes allocated, and the library's two C entry points,
+// whose addresses Python hands in when it loads it, called on the current stream.
 #include <Python.h>
 
 #include <ATen/ATen.h>
@@ -68,6 +68,14 @@ PyObject* icl_attention(PyObject*, PyObject* const* args, Py_ssize_t n) {
     if (q_train.scalar_type() != type || v.scalar_type() != type || (n_test > 0 && q_test.scalar_type() != type) ||
         (type != at::kBFloat16 && type != at::kHalf))
         return refuse("expected bf16 or fp16 tensors of one type");
+    // The kernels read B * H * rows * d values from each address, as k's sizes have it.
+    auto goes_with_k = [&](const at::Tensor& t, int64_t rows) {
+        return t.device() == k.device() && t.is_contiguous() && t.dim() >= 2 && t.size(-2) == rows && t.size(-1) == d &&
+               t.numel() == B * H * rows * d;
+    };
+    if (!goes_with_k(q_train, n_train) || !goes_with_k(v, n_train) || (n_test > 0 && !goes_with_k(q_test, n_test)))
+        return refuse("expected contiguous tensors of k's batch, heads, d and device");
+    if (ws.device() != k.device() || !ws.is_contiguous()) return refuse("expected a contiguous workspace on k's device");
     const bool half = type == at::kHalf, test_only = (flags & FP8ATTN_TEST_ROWS_ONLY) != 0;
     // The codes and scales stay inside this call: one allocation holds them all.
     auto up = [](int64_t x) { return (x + 255) / 256 * 256; };
