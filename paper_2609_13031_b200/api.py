@@ -9,6 +9,8 @@ not been built, loading raises.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 
 import torch
@@ -59,7 +61,7 @@ class Fp8AttnError(RuntimeError):
 def load() -> ctypes.CDLL:
     """Load the CUDA library; raises if it is missing (build it with
     ``python -m paper_2609_13031_b200.build`` or ``__graft_entry__.build()``)."""
-    global _lib, _native
+    global _lib
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -127,14 +129,29 @@ def load() -> ctypes.CDLL:
     lib.fp8attn_icl_step_host.argtypes = [vp, vp, vp, vp, i32, i32, i64, i64, i32, f32, u32, vp, vp, vp, sz, vp]
     lib.fp8attn_host_step_status.restype = i32
     lib.fp8attn_host_step_status.argtypes = [vp, i32, i32, i64, i64, i32, u32, vp, ctypes.POINTER(ctypes.c_uint32)]
-    try:
-        from . import _binding
-    except ImportError as e:
-        raise RuntimeError("the native half of the binding has not been built.  Run "
-                           "`python -m paper_2609_13031_b200.build`.") from e
-    _binding.bind(ctypes.cast(lib.fp8attn_quantize_qkv_ex, vp).value, ctypes.cast(lib.fp8attn_icl_forward_ex, vp).value)
-    _native, _lib = _binding, lib
+    _lib = lib
     return lib
+
+
+def _load_native():
+    """The native half of the binding, which ``icl_attention`` alone goes through."""
+    global _native
+    if _native is None:
+        from .build import binding_path
+        lib, path = load(), binding_path()
+        try:
+            if not os.path.exists(path):
+                raise ImportError(f"{path} not found")
+            loader = importlib.machinery.ExtensionFileLoader(__package__ + "._binding", path)
+            module = importlib.util.module_from_spec(importlib.util.spec_from_file_location(loader.name, path, loader=loader))
+            loader.exec_module(module)
+        except ImportError as e:
+            raise RuntimeError(f"the native half of the binding does not load: {e}.  Run "
+                               "`python -m paper_2609_13031_b200.build --force`.") from e
+        address = lambda f: ctypes.cast(f, ctypes.c_void_p).value
+        module.bind(address(lib.fp8attn_quantize_qkv_ex), address(lib.fp8attn_icl_forward_ex))
+        _native = module
+    return _native
 
 
 def status_string(status: int) -> str:
@@ -467,9 +484,8 @@ def icl_attention(q_train, q_test, k, v, workspace=None, softmax_scale: float = 
     if workspace is None:
         B, H, n_train, d = _dims(k)
         workspace = new_workspace(B, H, k.device, n_train=n_train if flags & SPLIT_TAIL else 0, d=d)
-    if _native is None:
-        load()
-    quantized, forward, out_train, out_test = _native.icl_attention(q_train, q_test, k, v, workspace, softmax_scale, flags)
+    native = _native or _load_native()
+    quantized, forward, out_train, out_test = native.icl_attention(q_train, q_test, k, v, workspace, softmax_scale, flags)
     _check("fp8attn_quantize_qkv", quantized)
     _check("fp8attn_icl_forward", forward)
     return out_train, out_test

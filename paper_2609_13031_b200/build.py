@@ -10,7 +10,6 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(_HERE), "include")
 LIB = os.path.join(_HERE, "libfp8attn.so")
-BINDING = os.path.join(_HERE, "_binding.so")
 SOURCES = ["api.cu", "quantize.cu", "attention.cu", "perturb.cu", "host_step.cu", "key_order.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
@@ -50,21 +49,28 @@ def build_cuda(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def binding_path() -> str:
+    """Where the native half of the binding stands for this interpreter and this torch, whose C++ interface it is
+    compiled against: another one finds no file there instead of one that does not fit."""
+    import torch
+    return os.path.join(_HERE, f"_binding.{sys.implementation.cache_tag}.torch-{torch.__version__}.so")
+
+
 def build_binding(force: bool = False) -> str:
     """csrc/binding.cpp against this torch: a CPython module beside the library."""
     import torch
     from torch.utils import cpp_extension
-    src = os.path.join(CSRC, "binding.cpp")
-    if force or _stale(BINDING, [src, os.path.join(INCLUDE, "fp8attn.h")]):
+    src, target = os.path.join(CSRC, "binding.cpp"), binding_path()
+    if force or _stale(target, [src, os.path.join(INCLUDE, "fp8attn.h")]):
         system = cpp_extension.include_paths("cuda") + [sysconfig.get_paths()["include"]]
-        tmp = BINDING + f".tmp{os.getpid()}"
+        tmp = target + f".tmp{os.getpid()}"
         subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
                         f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}", "-I", INCLUDE,
                         *(a for d in system for a in ("-isystem", d)), src, "-o", tmp,
                         "-L" + os.path.join(os.path.dirname(torch.__file__), "lib"),
                         "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"], check=True)
-        os.replace(tmp, BINDING)
-    return BINDING
+        os.replace(tmp, target)
+    return target
 
 
 if __name__ == "__main__":

@@ -166,3 +166,23 @@ def test_native_binding_refuses_what_the_call_does_not_take():
             api.icl_attention(*args, workspace=torch.zeros(4096, dtype=torch.uint8))
     with pytest.raises(TypeError):
         api.icl_attention(ok, 3, ok, ok, workspace=torch.zeros(4096, dtype=torch.uint8))
+
+
+def test_only_icl_attention_needs_the_native_half(monkeypatch, tmp_path):
+    """Another torch or interpreter, or a module that does not load: every other function works, and the one that
+    needs it says why."""
+    import sys
+    import pytest
+    import torch
+    assert torch.__version__ in build.binding_path() and sys.implementation.cache_tag in build.binding_path()
+    x = torch.zeros((1, 1, 4, 64), dtype=torch.bfloat16)
+    for name, content, why in (("none.so", None, "not found"), ("broken.so", b"no library", "broken.so")):
+        path = tmp_path / name
+        if content is not None:
+            path.write_bytes(content)
+        monkeypatch.setattr(build, "binding_path", lambda: str(path))
+        monkeypatch.setattr(api, "_native", None)
+        monkeypatch.setattr(api, "_lib", None)
+        assert api.status_string(0) == "ok" and api.workspace_bytes(1, 8) > 0
+        with pytest.raises(RuntimeError, match=why):
+            api.icl_attention(x, x, x, x, workspace=torch.zeros(4096, dtype=torch.uint8))
