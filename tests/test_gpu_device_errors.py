@@ -53,7 +53,7 @@ def test_small_fused_quantization_writes_nothing_while_an_error_is_pending(n, m,
     assert api.last_device_status(ws) == (0, 0)
 
 
-@pytest.mark.parametrize("H,n,d,stages", [(4, 3000, 64, 1), (8, 20011, 128, 3), (3, 40000, 128, 3)])
+@pytest.mark.parametrize("H,n,d,stages", [(4, 3000, 64, 1), (8, 20011, 128, 3), (3, 40000, 128, 3), (16, 12289, 64, 2)])
 @pytest.mark.parametrize("limit", [1, 2000, 6000, 20000])
 def test_one_pass_quantizer_gives_up_cleanly(H, n, d, stages, limit):
     """Waits that run out (at once, or in the middle of a stage whose copies are under way): the call

@@ -18,6 +18,10 @@ pytestmark = pytest.mark.gpu
     (3, 1, 8, 8192, 2048, 64),     # 24 units
     (3, 1, 5, 10007, 40000, 64),   # 15 units, test rows outnumber the train rows
     (3, 1, 2, 16000, 1, 128),
+    # above 48 MB: a launch before clears the words, and all threads wait for the heads that their rows follow
+    (3, 1, 16, 2600, 32768, 128),
+    (3, 2, 4, 5000, 32768, 128),
+    (3, 1, 8, 10007, 60000, 64),
 ])
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16])
 def test_matches_two_passes(tensors, B, H, n, m, d, dtype):
