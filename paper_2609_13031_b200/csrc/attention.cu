@@ -1023,9 +1023,10 @@ int launch_tiles(const AttnParams& p, cudaStream_t stream) {
 // same keys in the same steps), so the choice may depend on the number of test rows.  Two tiles / one: 2 heads of
 // 512 + 128 x 64 10.1 / 8.1 us; 8 heads of 1,024 + 256 x 64 16.2 / 13.0, x 128 18.6 / 14.4 (bf16 20.3 / 15.3);
 // 2 heads of 8,192 + 1,000 x 128 101 / 77 (bf16 112 / 81); 1 head of 16,000 + 2,000 x 64 174 / 137; 16 heads of
-// 1,000 test rows against 16,384 x 64 174 / 134, x 128 185 / 143.  Up to kOneTileKeys keys: calls beyond it are made as two
-// tiles by choice, not because one would be slower (the same rows against 32,768 334 / 259 and 351 / 275, against 131,072
-// 1,282 / 1,006 and 1,318 / 1,040; 129 rows of 2 heads against 1,000,000 9,331 / 7,346).
+// 1,000 test rows against 16,384 x 64 174 / 134, x 128 185 / 143.  Up to kOneTileKeys keys, the
+// longest that was measured when the line was drawn; it is no line of the kernel's, beyond it one tile takes a fifth
+// less time as well (the same rows against 32,768 334 / 259 and 351 / 275, against 131,072 1,282 / 1,006 and 1,318 / 1,040; 129
+// rows of 2 heads against 1,000,000 9,331 / 7,346).
 // With FP8ATTN_SPLIT_TAIL by the times below, one tile / the split that it replaces or leaves: 49 heads of 300 test
 // rows against 16,000 x 64 132 / 98 us (three tiles in three ranges), 29 heads of 600 against 8,000 70 / 76; 8 heads of
 // 1,930 + 250 x 64 22.5 / 23.5, x 128 26.1 / 29.7; 2,300 test rows of 8 heads against 3,000 x 64 31.2 / 29.2, x 128

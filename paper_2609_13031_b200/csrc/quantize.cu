@@ -304,7 +304,9 @@ __global__ void __launch_bounds__(1024) quantize_heads_kernel(const __grid_const
 // 42 / 39 us, 4 heads of 33,000 + 5,000 56 / 49 us, 2 heads of 33,200 + 8,300 33 / 28 us, 8 heads of 35,000 +
 // 5,000 100 / 101 us, of 44,000 + 1,000 102 / 120 us, of 65,536 + 16,384 129 / 183 us.  Test rows that enter the
 // maximum of the train queries are read by the blocks that hold those: 8 heads of 20,011 + 3,001 x 128 76 /
-// 58 us, of 65,536 + 16,384 157 / 185 us.
+// 58 us, of 65,536 + 16,384 157 / 185 us.  Calls of two stages have had a kernel of their own since, 1-2 us faster
+// than the estimate knows: 8 heads of 5,000 + 12,000 x 128 26.2 / 28.8 us (two passes here), of 5,000 + 32,768 43.1 / 41.5
+// and 16 heads of 2,600 + 32,768 65.8 / 61.0 (one pass here).
 bool one_pass_pays(const staged::Shape& a) {
     const double heads = a.units / a.tensors, mb = 16e-6;
     const double train = mb * (double)a.vecs * a.units, test = mb * (double)a.follow_vecs * heads;

@@ -505,8 +505,9 @@ __global__ void __launch_bounds__(kThreads, 1) staged_kernel(const __grid_consta
 
 // Two stages fill both buffers and wait for no room: they are loaded at once and exchanged together, so that the
 // workers stand still once, under the second load, instead of twice (2 us each, 3 us where the words wait behind loads
-// from HBM).  Graph-replayed, inputs not in L2 / in L2: 16 heads of 12,289 x 64 19.1 -> 17.8 / 13.1 -> 12.5 us, 8 heads of
-// 16,384 x 128 22.2 -> 20.1 / 13.7 -> 13.6, 8 heads of 8,192 + 2,048 x 64, three tensors, 21.4 -> 19.5 / 16.1 -> 14.5.  Rows
+// from HBM).  Graph-replayed, inputs not in L2 / in L2: 16 heads of 12,289 x 64 19.0 -> 18.0 / 12.9 -> 12.9 us, 8 heads of
+// 16,384 x 128 22.7 -> 19.8 / 13.6 -> 13.7, 2 heads of 40,000 x 128 17.3 -> 16.2 / 12.5 -> 11.4, three tensors of 8 heads of
+// 8,192 + 2,048 x 64 20.8 -> 19.4 / 15.2 -> 14.7, of 5,000 + 32,768 x 128 46.2 -> 44.7 / 42.6 -> 41.4.  Rows
 // that count in the maximum stay with the general form.  (A kernel of its own: as a template parameter of the general
 // one it moved that by up to 3 % through its schedule.)
 template <bool kHalf, bool kSelfTest>
@@ -806,7 +807,8 @@ constexpr int kRefused = -1;
 
 template <bool kHalf, bool kSelfTest>
 int launch(const Args& a, unsigned grid, cudaStream_t stream) {
-    // Two stages whose test rows do not count: the pair kernel, 5 .. 11 % faster (see there).
+    // Two stages whose test rows do not count: the pair kernel, 2 .. 13 % faster where the inputs are not in L2, between
+    // the same and 10 % where they are (see there).
     // (the opt-in to large dynamic shared memory is per device and context: set on every call)
     auto kernel = a.stages == 2 && !a.follow_counts ? staged_pair_kernel<kHalf, kSelfTest> : staged_kernel<kHalf, kSelfTest>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) !=
