@@ -157,6 +157,8 @@ def test_argument_checks_run_on_the_host_before_anything_touches_a_gpu():
 
 
 def test_native_binding_refuses_what_the_call_does_not_take():
+    """Without a GPU: the look at k, which comes first, and at what is no tensor at all.  What follows it needs tensors
+    on a GPU: test_gpu_icl_attention_refusals.py."""
     import pytest
     import torch
     api.load()
